@@ -410,10 +410,9 @@ bbp_status bbp_k_qr(double* A, int m, int n, double* Q, double* R, double* tau, 
  * least bbp_k_panel_cluster(c64, m, n) (the fewest whose shared memory holds
  * the panel with Q; 0 when even 16 do not) and at most 16.  A call with
  * Q = NULL needs a little less shared memory (no reflector scalars), so it
- * may fit where bbp_k_panel_cluster reports 0.  Each CTA caches 32, 64, ...
- * rows per warp lane (complex64 up to 256 rows a CTA, complex128 up to 128),
- * and a CTA beyond the rows a given cluster needs holds none.  BBP_ERR_ARG
- * when m < n or the panel does not fit. */
+ * may fit where bbp_k_panel_cluster reports 0.  A CTA beyond
+ * the rows a given cluster needs holds none.  BBP_ERR_ARG when m < n or the
+ * panel does not fit. */
 int bbp_k_panel_cluster(int c64, int m, int n);
 bbp_status bbp_k_panel_qr(int c64, const void* A, int m, int n, void* Q, void* R, int batch, int cluster,
                           void* stream);

@@ -247,17 +247,26 @@ inline double qr_flops(int m, int n) {
 // A.  batch panels at a stride of `stride` elements (R at n * n).
 // panel_cluster: the fewest CTAs whose shared memory holds an m x n panel of
 // elem-byte entries (with the reflector scalars Q needs when want_q; 0 when
-// even 16 do not); panel_cluster_auto: the cluster size of an automatic
-// launch.  cluster = 0 picks it; a given size must be at least
+// even 16 do not).  cluster = 0 picks it; a given size must be at least
 // panel_cluster(m, n, elem) and at most kPanelMaxCluster.
 constexpr int kPanelMaxCluster = 16;
 int panel_cluster(int m, int n, size_t elem, bool want_q = true);
-int panel_cluster_auto(int m, int n, size_t elem, bool want_q = true);
 cudaError_t init_panel_attributes();
 cudaError_t launch_panel_qr(const float2* A, int m, int n, float2* Q, float2* R, int batch, long long stride,
                             cudaStream_t s, int cluster = 0);
 cudaError_t launch_panel_qr(const double2* A, int m, int n, double2* Q, double2* R, int batch, long long stride,
                             cudaStream_t s, int cluster = 0);
+// The blocked factorisation behind it (k_qr.cu), for any shape: row blocks of
+// rb rows of A (m_all x n, the last one shorter), each k x n with k = min(rows,
+// n): Q (k columns a block, may alias A, may be null) at `stride` elements a
+// block, R k x n, or, of more than one block, n x n each with zero rows below
+// k.  bqr_fits: whether one block fits (cluster CTAs, 0: any number).
+bool bqr_fits(int m, int n, size_t elem, bool want_q, int cluster = 0);
+cudaError_t init_bqr_attributes();
+cudaError_t launch_bqr(const float2* A, int m_all, int n, int rb, long long stride, float2* Q, float2* R, int cluster,
+                       cudaStream_t s);
+cudaError_t launch_bqr(const double2* A, int m_all, int n, int rb, long long stride, double2* Q, double2* R,
+                       int cluster, cudaStream_t s);
 // Panels taller than one cluster holds (panel_cluster = 0): two-level TSQR
 // over row chunks that each fit one cluster; Q is required, R may be null.
 // panel_chunk_scratch_bytes: the device scratch it needs (0 when the panel
