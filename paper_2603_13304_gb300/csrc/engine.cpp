@@ -62,8 +62,8 @@ cudaError_t merge_call(int M, int N, int K, const float2* A, const float2* B, fl
 long long svd_launches(int m, int n, int chi, bool c64, int q) {
   const int M = std::min(m, n);
   const int b = c64 ? rand_block(m, n, chi) : rand_block64(m, n, chi);
-  if (b >= M) return 5;
-  return 12 + 4 * q + (c64 ? 1 : 0);
+  if (b >= M) return 1;
+  return 8 + 4 * q + (c64 ? 1 : 0);
 }
 cudaError_t svd_call(const float2* Z, int m, int n, int chi, float2* U, float2* Rem, void* work, int* status,
                      cudaStream_t s, int power_iters, bool tensor_cores, int* tc_err) {

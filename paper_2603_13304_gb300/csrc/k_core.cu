@@ -517,53 +517,6 @@ __device__ int rotate_pair(C* ra, C* rb, int N, C* wa, C* wb, int M, int lane, d
   return 1;
 }
 
-// The same rotation by a half warp (16 lanes: lane l of the half handles
-// entries l, l + 16, ...): two pairs a warp.  Both halves always run the
-// sums (an invalid pair on zeros), so the shuffles see the whole warp.
-template <typename C>
-__device__ int rotate_pair_half(C* ra, C* rb, int N, C* wa, C* wb, int M, int hl, bool valid, double tol,
-                                typename RealOf<C>::T floor) {
-  using R = typename RealOf<C>::T;
-  R al = 0, be = 0, gx = 0, gy = 0;
-  if (valid)
-    for (int c = hl; c < N; c += 16) {
-      const C x = ra[c], y = rb[c];
-      al += cabs2(x);
-      be += cabs2(y);
-      gx += x.x * y.x + x.y * y.y;
-      gy += x.y * y.x - x.x * y.y;
-    }
-  for (int o = 8; o > 0; o >>= 1) {
-    al += __shfl_xor_sync(0xffffffffu, al, o);
-    be += __shfl_xor_sync(0xffffffffu, be, o);
-    gx += __shfl_xor_sync(0xffffffffu, gx, o);
-    gy += __shfl_xor_sync(0xffffffffu, gy, o);
-  }
-  if (!valid) return 0;
-  R g = sqrt(gx * gx + gy * gy);
-  if (g == 0 || g <= (R)tol * sqrt(al) * sqrt(be)) return 0;
-  if (fmin(al, be) <= floor) return 0;
-  const R far = sizeof(R) == 8 ? (R)1e-60 : (R)1e-30;
-  if (fmin(al, be) <= far * fmax(al, be)) return 0;
-  C e = cx<C>(gx / g, gy / g);
-  R zeta = (be - al) / (2 * g);
-  R t = (zeta >= 0 ? (R)1 : (R)-1) / (fabs(zeta) + sqrt((R)1 + zeta * zeta));
-  R cs = (R)1 / sqrt((R)1 + t * t), sn = cs * t;
-  for (int c = hl; c < N; c += 16) {
-    const C x = ra[c], y = rb[c];
-    const C ey = cmul(e, y);
-    ra[c] = csub(cscale(x, cs), cscale(ey, sn));
-    rb[c] = cadd(cscale(x, sn), cscale(ey, cs));
-  }
-  for (int c = hl; c < M; c += 16) {
-    const C x = wa[c], y = wb[c];
-    const C ey = cmul(e, y);
-    wa[c] = csub(cscale(x, cs), cscale(ey, sn));
-    wb[c] = cadd(cscale(x, sn), cscale(ey, cs));
-  }
-  return 1;
-}
-
 // Algorithmic flops of a one-sided Jacobi run: every sweep tests M(M-1)/2
 // pairs (two squared norms and one complex inner product over N: 16 N), every
 // applied rotation updates two rows of G and two of WH (18 per element pair).
@@ -612,76 +565,6 @@ __global__ void __launch_bounds__(256) k_jacobi(SvdWork<C> w, int M, int N, doub
   if (crank == 0 && threadIdx.x == 0) {
     *status = 1;   // sweep limit reached
     if (flops) atomicAdd(flops, jacobi_flops(max_sweeps, w.counters[3], M, N));
-  }
-}
-
-// One-CTA Jacobi with G and WH resident in shared memory
-// ((M*N + M*M) * sizeof(C) <= kSmemMax); same rounds, tests and counters as
-// k_jacobi, __syncthreads between rounds.
-template <typename C>
-__global__ void __launch_bounds__(1024) k_jacobi_smem(SvdWork<C> w, int M, int N, double tol, double floor_rel,
-                                                     int max_sweeps, int* status, double* flops) {
-  using R = typename RealOf<C>::T;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* G = (C*)smem_raw;
-  C* WH = G + (long long)M * N;
-  __shared__ int s_rot;
-  const R floor = (R)(floor_rel * *w.zn2);
-  for (long long e = threadIdx.x; e < (long long)M * N; e += blockDim.x) G[e] = w.G[e];
-  for (long long e = threadIdx.x; e < (long long)M * M; e += blockDim.x) WH[e] = w.WH[e];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int Mp = M + (M & 1);
-  const int npairs = Mp / 2;
-  int sweeps = 0, rot_total = 0;
-  bool converged = false;
-  __syncthreads();
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
-    int rot = 0;
-    const bool halves = npairs > nw;     // more pairs than warps: a pair per half warp
-    for (int r = 0; r < Mp - 1; ++r) {
-      if (halves) {
-        const int hl = lane & 15, hw = 2 * warp + (lane >> 4);
-        for (int q0 = 2 * warp; q0 < npairs; q0 += 2 * nw) {
-          const int q = hw + (q0 - 2 * warp);   // this half's pair
-          int a = 0, b = 0;
-          if (q < npairs) {
-            if (q == 0) { a = Mp - 1; b = r; }
-            else { a = (r + q) % (Mp - 1); b = (r - q + Mp - 1) % (Mp - 1); }
-          }
-          const bool valid = q < npairs && a < M && b < M;
-          const int aa = valid ? a : 0, bb = valid ? b : 0;
-          rot += rotate_pair_half(G + (long long)aa * N, G + (long long)bb * N, N, WH + (long long)aa * M,
-                                  WH + (long long)bb * M, M, hl, valid, tol, floor);
-        }
-      } else {
-        for (int q = warp; q < npairs; q += nw) {
-          int a, b;
-          if (q == 0) { a = Mp - 1; b = r; }
-          else { a = (r + q) % (Mp - 1); b = (r - q + Mp - 1) % (Mp - 1); }
-          if (a >= M || b >= M) continue;
-          rot += rotate_pair<false>(G + (long long)a * N, G + (long long)b * N, N, WH + (long long)a * M,
-                               WH + (long long)b * M, M, lane, tol, floor);
-        }
-      }
-      __syncthreads();
-    }
-    if ((halves ? (lane & 15) : lane) == 0 && rot) atomicAdd(&s_rot, rot);
-    __syncthreads();
-    const int total = s_rot;
-    ++sweeps;
-    rot_total += total;
-    __syncthreads();
-    if (total == 0) { converged = true; break; }
-  }
-  for (long long e = threadIdx.x; e < (long long)M * N; e += blockDim.x) w.G[e] = G[e];
-  for (long long e = threadIdx.x; e < (long long)M * M; e += blockDim.x) w.WH[e] = WH[e];
-  if (threadIdx.x == 0) {
-    w.counters[2] = sweeps;
-    w.counters[3] = rot_total;
-    if (!converged) *status = 1;
-    if (flops) atomicAdd(flops, jacobi_flops(sweeps, rot_total, M, N));
   }
 }
 
@@ -756,20 +639,12 @@ cudaError_t smem_optin() {
   return e;
 }
 
-// Jacobi on the M x N rows of w: in shared memory when G and WH fit (one CTA,
-// one warp per pair), else on a cluster of up to 8 CTAs.
+// Jacobi on the M x N rows of w in global memory, for problems that no
+// cluster's shared memory holds: a cluster of up to 8 CTAs.
 template <typename C>
 cudaError_t launch_jacobi(SvdWork<C> w, int M, int N, double tol, int max_sweeps, int* status, cudaStream_t s) {
   KTimerScope timer(KC_JACOBI, s, 0.0);
   double* flops = ktimer_device_flops(KC_JACOBI);
-  const size_t jsm = sizeof(C) * ((size_t)M * N + (size_t)M * M);
-  if (jsm <= (size_t)kSmemMax) {
-    cudaError_t e = smem_optin<k_jacobi_smem<C>>();
-    if (e != cudaSuccess) return e;
-    const int threads = std::min(1024, 32 * std::max(1, (M + 1) / 2));
-    k_jacobi_smem<C><<<1, threads, jsm, s>>>(w, M, N, tol, floor_rel_of<C>(), max_sweeps, status, flops);
-    return cudaGetLastError();
-  }
   int cs = (M / 2 + 15) / 16;   // about two pairs per warp per round
   if (cs < 1) cs = 1;
   if (cs > 8) cs = 8;
@@ -809,39 +684,37 @@ cudaError_t jacobi_svd(const C* Z, int m, int n, int chi, C* U, C* Rem, void* wo
   const int M = m < n ? m : n, N = m < n ? n : m;
   const int k = chi < M ? chi : M;
   SvdWork<C> w = carve<C>(work, M, N);
-  cudaError_t e0 = cudaMemsetAsync(w.counters, 0, 64, s);
-  if (e0 != cudaSuccess) return e0;
-  k_svd_init<C><<<grid_for((long long)M * N + (long long)M * M, 256), 256, 0, s>>>(Z, m, n, w);
   cudaError_t e;
   if (jacobi_reduce_fits<C>(M, N)) {
     char* p = (char*)work + jacobi_bytes<C>(M, N);
     C* GH = (C*)p; p += align256(sizeof(C) * (size_t)N * M);
     C* QT = (C*)p; p += align256(sizeof(C) * (size_t)N * M);
-    C* Lm = (C*)p; p += align256(sizeof(C) * (size_t)M * M);
+    C* RT = (C*)p; p += align256(sizeof(C) * (size_t)M * M);
     C* LR = (C*)p;
-    if ((e = launch_conj_transpose(w.G, M, N, GH, s)) != cudaSuccess) return e;
-    if ((e = launch_panel_qr(GH, N, M, QT, LR, 1, 0, s)) != cudaSuccess) return e;      // R_T into LR
-    if ((e = launch_conj_transpose(LR, M, M, Lm, s)) != cudaSuccess) return e;          // L = R_T^H
-    // the M x M problem in its own SvdWork view (WH = I there), same counters
-    SvdWork<C> ws = carve<C>(LR, M, M);
-    ws.counters = w.counters;
-    ws.zn2 = w.zn2;
-    ws.sigma = w.sigma;
-    ws.idx = w.idx;
-    ws.WH = w.WH;
-    ws.G = LR;
-    if ((e = cudaMemcpyAsync(LR, Lm, sizeof(C) * (size_t)M * M, cudaMemcpyDeviceToDevice, s)) != cudaSuccess) return e;
-    if ((e = launch_jacobi(ws, M, M, tol, max_sweeps, status, s)) != cudaSuccess) return e;
+    const C* tall = Z;                   // G^H (N x M): Z itself, or Z^H
+    if (m <= n) {
+      if ((e = launch_conj_transpose(Z, m, n, GH, s)) != cudaSuccess) return e;
+      tall = GH;
+    }
+    if ((e = launch_panel_qr(tall, N, M, QT, RT, 1, 0, s)) != cudaSuccess) return e;
+    // L = R_T^H rotated into LR = WH L, its row norms, their order and ||Z||^2
+    if ((e = launch_jac(RT, M, true, M, M, k, LR, w.WH, w.sigma, w.idx, w.zn2, w.counters, 0, 0, (C*)nullptr,
+                        (C*)nullptr, tol, floor_rel_of<C>(), max_sweeps, status, s)) != cudaSuccess)
+      return e;
     // rotated rows of G: (WH L) Q_T^H (M x N)
     if ((e = launch_zgemm('N', 'C', M, N, M, cx<C>(1, 0), LR, M, 0, QT, M, 0, cx<C>(0, 0), w.G, N, 0, 1, s)) !=
         cudaSuccess)
       return e;
+  } else if (jac_fits(M, N, sizeof(C))) {
+    return launch_jac(Z, n, m > n, M, N, k, (C*)nullptr, (C*)nullptr, nullptr, nullptr, nullptr, w.counters, m, n, U,
+                      Rem, tol, floor_rel_of<C>(), max_sweeps, status, s);
   } else {
-    e = launch_jacobi(w, M, N, tol, max_sweeps, status, s);
-    if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(w.counters, 0, 64, s)) != cudaSuccess) return e;
+    k_svd_init<C><<<grid_for((long long)M * N + (long long)M * M, 256), 256, 0, s>>>(Z, m, n, w);
+    if ((e = launch_jacobi(w, M, N, tol, max_sweeps, status, s)) != cudaSuccess) return e;
+    k_row_norms<C><<<(M * 32 + 255) / 256, 256, 0, s>>>(w, M, N);
+    k_select<C><<<1, 256, 0, s>>>(w, M, k);
   }
-  k_row_norms<C><<<(M * 32 + 255) / 256, 256, 0, s>>>(w, M, N);
-  k_select<C><<<1, 256, 0, s>>>(w, M, k);
   k_svd_out<C><<<grid_for((long long)m * k + (long long)k * n, 256), 256, 0, s>>>(w, m, n, k, floor_rel_of<C>(), U,
                                                                                  Rem);
   return cudaGetLastError();
@@ -1311,13 +1184,19 @@ static cudaError_t rand_svd(const C* Z, int m, int n, int chi, int b, C* U, C* R
   }
   if ((e = zh_times(Q, W)) != cudaSuccess) return e;
   if ((e = orth_panel<C>(W, n, b, Rw, chunk, s)) != cudaSuccess) return e;
-  if ((e = launch_conj_transpose(Rw, b, b, L, s)) != cudaSuccess) return e;
   SvdWork<C> w = carve<C>(jw, b, b);
-  if ((e = cudaMemsetAsync(w.counters, 0, 64, s)) != cudaSuccess) return e;
-  k_svd_init<C><<<grid_for(2LL * b * b, 256), 256, 0, s>>>(L, b, b, w);
-  if ((e = launch_jacobi(w, b, b, jtol, 60, status, s)) != cudaSuccess) return e;
-  k_row_norms<C><<<(b * 32 + 255) / 256, 256, 0, s>>>(w, b, b);
-  k_select<C><<<1, 256, 0, s>>>(w, b, k);
+  if (jac_fits(b, b, z)) {
+    if ((e = launch_jac(Rw, b, true, b, b, k, w.G, w.WH, w.sigma, w.idx, w.zn2, w.counters, 0, 0, (C*)nullptr,
+                        (C*)nullptr, jtol, floor_rel_of<C>(), 60, status, s)) != cudaSuccess)
+      return e;
+  } else {
+    if ((e = launch_conj_transpose(Rw, b, b, L, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(w.counters, 0, 64, s)) != cudaSuccess) return e;
+    k_svd_init<C><<<grid_for(2LL * b * b, 256), 256, 0, s>>>(L, b, b, w);
+    if ((e = launch_jacobi(w, b, b, jtol, 60, status, s)) != cudaSuccess) return e;
+    k_row_norms<C><<<(b * 32 + 255) / 256, 256, 0, s>>>(w, b, b);
+    k_select<C><<<1, 256, 0, s>>>(w, b, k);
+  }
   const double2* WHo;
   const double2* Go;
   const int* idxo;
@@ -1801,14 +1680,13 @@ cudaError_t launch_mps_dot(const ChainDesc& a, const ChainDesc& b, bool c64, dou
 // (done once up front so that no attribute call falls inside a stream capture).
 cudaError_t init_kernel_attributes() {
   cudaError_t e;
-  if ((e = smem_optin<k_jacobi_smem<double2>>()) != cudaSuccess) return e;
-  if ((e = smem_optin<k_jacobi_smem<float2>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_jacobi_cut64>()) != cudaSuccess) return e;
   for (const void* f : {(const void*)k_msg_normalise<double2>, (const void*)k_msg_normalise<float2>,
                         (const void*)k_mps_dot<double2>, (const void*)k_mps_dot<float2>,
                         (const void*)k_jacobi_cut64})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
   if ((e = init_panel_attributes()) != cudaSuccess) return e;
+  if ((e = init_jac_attributes()) != cudaSuccess) return e;
   return init_tc_attributes();
 }
 

@@ -277,6 +277,22 @@ cudaError_t launch_panel_qr_chunked(const float2* A, int m, int n, float2* Q, fl
 cudaError_t launch_panel_qr_chunked(const double2* A, int m, int n, double2* Q, double2* R, void* scratch,
                                     cudaStream_t s);
 
+// One-sided Jacobi of the M rows (length N) of G_0 = Z (Z[a ldz + c]) or, with
+// conj_t, Z^H (conj Z[c ldz + a]), on a cluster of CTAs with the rows in shared
+// memory (k_jac.cu).  Any of the outputs may be null: G (rotated rows), WH (WH
+// G_0 = G), sigma (row norms), idx (the k largest, in order), *zn2 =
+// ||G_0||_F^2, counters[2], [3] (sweeps, rotations); U (m x k) and Rem (k x n)
+// of the truncated SVD of the m x n matrix whose rows (m <= n) or conjugate
+// columns G_0 holds.  jac_fits: whether the problem fits.
+bool jac_fits(int M, int N, size_t elem);
+cudaError_t init_jac_attributes();
+cudaError_t launch_jac(const float2* Z, int ldz, bool conj_t, int M, int N, int k, float2* G, float2* WH,
+                       double* sigma, int* idx, double* zn2, int* counters, int m, int n, float2* U, float2* Rem,
+                       double tol, double floor_rel, int max_sweeps, int* status, cudaStream_t s);
+cudaError_t launch_jac(const double2* Z, int ldz, bool conj_t, int M, int N, int k, double2* G, double2* WH,
+                       double* sigma, int* idx, double* zn2, int* counters, int m, int n, double2* U, double2* Rem,
+                       double tol, double floor_rel, int max_sweeps, int* status, cudaStream_t s);
+
 // Allocation-free truncated SVD (k_noalloc.cu): scratch in a fixed device
 // array of noalloc_scratch_bytes(); *too_large is set when svd_work_bytes(m, n)
 // exceeds it (nothing is launched then).
