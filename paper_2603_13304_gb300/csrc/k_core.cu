@@ -148,9 +148,20 @@ __global__ void __launch_bounds__(256) k_fuse(const double2* __restrict__ t, int
 }
 
 // -------------------------------------------------------------------- gemm
-
-constexpr int GT = 32;   // output tile
-constexpr int GK = 16;   // k tile
+// Complex GEMM on the FP32 / FP64 units: a CTA a TM x TN tile, a thread RM x RN
+// entries of it (rows ty + i TM / RM, columns tx + j TN / RN, so that a warp
+// reads two rows and sixteen consecutive columns of a k slice from shared
+// memory), K in slices of kGemmK double-buffered in shared memory with the
+// next slice on its way in registers.  KG thread groups share a slice's k
+// (summed at the end).
+//
+// complex64: 96 multiply-adds per ten shared-memory loads at 4 x 6 entries, so
+// that the FMA pipe and not the loads bounds it; every product is a chain of
+// fused multiply-adds (a complex product added to the sum takes half as many
+// instructions again).  complex128 is bound by the FP64 rate (two
+// multiply-adds a clock and SM) at any tile, so its tiles are small: padding
+// to a tile costs FP64 time, and a product must spread over many SMs.
+constexpr int kGemmK = 16;
 
 template <typename C>
 __device__ __forceinline__ C load_op(const C* P, int ld, char op, int r, int c, int R, int Cc) {
@@ -159,17 +170,24 @@ __device__ __forceinline__ C load_op(const C* P, int ld, char op, int r, int c, 
   C v = P[(long long)c * ld + r];
   return op == 'C' ? cconj(v) : v;
 }
+template <typename C> __device__ __forceinline__ void cfma(C& s, C a, C b) {   // s += a b
+  s.x = fma(-a.y, b.y, fma(a.x, b.x, s.x));
+  s.y = fma(a.y, b.x, fma(a.x, b.y, s.y));
+}
 
 // With part != null the grid's z index is a slice of K (kchunk entries,
 // batch 1): each CTA writes its raw partial tile to part[z][M][N] and
 // k_gemm_reduce adds the slices in order (split K for skinny products).
-template <typename C>
-__global__ void __launch_bounds__(256) k_gemm(char opA, char opB, int M, int N, int K, C alpha, const C* __restrict__ A,
-                                              int lda, long long sA, const C* __restrict__ B, int ldb, long long sB,
-                                              C beta, C* __restrict__ Cm, int ldc, long long sC, int kchunk,
-                                              C* __restrict__ part) {
-  __shared__ C As[GT][GK + 1];
-  __shared__ C Bs[GK][GT + 1];
+template <typename C, int TM, int TN, int RM, int RN, int KG>
+__global__ void __launch_bounds__((TM / RM) * (TN / RN) * KG, 2)
+    k_gemm(char opA, char opB, int M, int N, int K, C alpha, const C* __restrict__ A, int lda, long long sA,
+           const C* __restrict__ B, int ldb, long long sB, C beta, C* __restrict__ Cm, int ldc, long long sC,
+           int kchunk, C* __restrict__ part) {
+  constexpr int TX = TN / RN, TY = TM / RM, NT = TX * TY * KG;
+  constexpr int PA = (TM * kGemmK + NT - 1) / NT, PB = (TN * kGemmK + NT - 1) / NT;
+  __shared__ C As[2][kGemmK][TM + 1];
+  __shared__ C Bs[2][kGemmK][TN + 1];
+  const int tid = threadIdx.x, g = tid / (TX * TY), tx = tid % TX, ty = (tid / TX) % TY;
   const int bz = blockIdx.z;
   int kb = 0, ke = K;
   if (part) {
@@ -180,47 +198,84 @@ __global__ void __launch_bounds__(256) k_gemm(char opA, char opB, int M, int N, 
     B += bz * sB;
     Cm += bz * sC;
   }
-  const int row0 = blockIdx.y * GT, col0 = blockIdx.x * GT;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  C acc[2][2];
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) acc[i][j] = cx<C>(0, 0);
-  // the next k tile is loaded into registers while the current one is
-  // multiplied (GT * GK / 256 = 2 entries of A and 2 of B a thread)
-  constexpr int kPer = GT * GK / 256;
-  C pa[kPer], pb[kPer];
+  const int tn = (N + TN - 1) / TN;
+  const int row0 = (int)(blockIdx.x / tn) * TM, col0 = (int)(blockIdx.x % tn) * TN;
+  C acc[RM][RN];
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j) acc[i][j] = cx<C>(0, 0);
+  C pa[PA], pb[PB];
+  // neighbouring threads along the operand's contiguous index
   auto fetch = [&](int k0) {
 #pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      pa[u] = load_op(A, lda, opA, row0 + e / GK, k0 + e % GK, M, ke);
-      pb[u] = load_op(B, ldb, opB, k0 + e / GT, col0 + e % GT, ke, N);
+    for (int u = 0; u < PA; ++u) {
+      const int e = tid + NT * u;
+      const int r = opA == 'N' ? e / kGemmK : e % TM, k = opA == 'N' ? e % kGemmK : e / TM;
+      pa[u] = e < TM * kGemmK ? load_op(A, lda, opA, row0 + r, k0 + k, M, ke) : cx<C>(0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int e = tid + NT * u;
+      const int c = opB == 'N' ? e % TN : e / kGemmK, k = opB == 'N' ? e / TN : e % kGemmK;
+      pb[u] = e < TN * kGemmK ? load_op(B, ldb, opB, k0 + k, col0 + c, ke, N) : cx<C>(0, 0);
     }
   };
-  if (kb < ke) fetch(kb);
-  for (int k0 = kb; k0 < ke; k0 += GK) {
+  auto stage = [&](int b) {
 #pragma unroll
-    for (int u = 0; u < kPer; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      As[e / GK][e % GK] = pa[u];
-      Bs[e / GT][e % GT] = pb[u];
+    for (int u = 0; u < PA; ++u) {
+      const int e = tid + NT * u;
+      const int r = opA == 'N' ? e / kGemmK : e % TM, k = opA == 'N' ? e % kGemmK : e / TM;
+      if (e < TM * kGemmK) As[b][k][r] = pa[u];
     }
-    __syncthreads();
-    if (k0 + GK < ke) fetch(k0 + GK);
-#pragma unroll 4
-    for (int kk = 0; kk < GK; ++kk) {
-      C a0 = As[ty][kk], a1 = As[ty + 16][kk];
-      C b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      acc[0][0] = cadd(acc[0][0], cmul(a0, b0));
-      acc[0][1] = cadd(acc[0][1], cmul(a0, b1));
-      acc[1][0] = cadd(acc[1][0], cmul(a1, b0));
-      acc[1][1] = cadd(acc[1][1], cmul(a1, b1));
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int e = tid + NT * u;
+      const int c = opB == 'N' ? e % TN : e / kGemmK, k = opB == 'N' ? e / TN : e % kGemmK;
+      if (e < TN * kGemmK) Bs[b][k][c] = pb[u];
     }
-    __syncthreads();
+  };
+  if (kb < ke) {
+    fetch(kb);
+    stage(0);
   }
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) {
-      int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = kb; k0 < ke; k0 += kGemmK) {
+    const bool more = k0 + kGemmK < ke;
+    if (more) fetch(k0 + kGemmK);
+    constexpr int KK = kGemmK / KG;
+#pragma unroll 4
+    for (int q = 0; q < KK; ++q) {
+      const int kk = KG > 1 ? g * KK + q : q;
+      C a[RM], b[RN];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) a[i] = As[buf][kk][ty + TY * i];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) b[j] = Bs[buf][kk][tx + TX * j];
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) cfma(acc[i][j], a[i], b[j]);
+    }
+    if (more) stage(buf ^ 1);
+    __syncthreads();
+    buf ^= 1;
+  }
+  if constexpr (KG > 1) {                // the groups' sums, in order
+    C* sum = &As[0][0][0];
+    static_assert(RM * RN == 1 && TX * TY * KG <= 2 * kGemmK * (TM + 1), "the sums fit the staging buffer");
+    sum[tid] = acc[0][0];
+    __syncthreads();
+    if (g > 0) return;
+#pragma unroll
+    for (int q = 1; q < KG; ++q) acc[0][0] = cadd(acc[0][0], sum[q * TX * TY + tid]);
+  }
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      const int r = row0 + ty + TY * i, c = col0 + tx + TX * j;
       if (r < M && c < N) {
         if (part) {
           part[((long long)bz * M + r) * N + c] = acc[i][j];
@@ -834,32 +889,19 @@ __global__ void __launch_bounds__(1024) k_jacobi_cut64(SvdWork<float2> w, int b,
   }
 }
 
-// U = Q WH[top]^H (m x k) and Rem = G'[top] W^H (k x n): WH and G' of the
-// reduced SVD in complex128, Q and W in the path's element type.
-// (products in the element type: Q and W carry its accuracy; for complex64
-// the complex128 factors are rounded once, since FP64 arithmetic here would
-// cost 64x the FP32 rate and add nothing)
-template <typename C>
-__device__ __forceinline__ C as_elem(double2 v) { return cx<C>(v.x, v.y); }
-
-template <typename C>
-__global__ void k_rand_out64(const C* __restrict__ Q, int m, int b, const double2* __restrict__ WH64,
-                             const double2* __restrict__ G64, const int* __restrict__ idx64, const C* __restrict__ W,
-                             int n, int k, C* U, C* Rem) {
-  long long totU = (long long)m * k, totR = (long long)k * n;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < totU + totR;
-       e += (long long)gridDim.x * blockDim.x) {
-    C acc = cx<C>(0.0, 0.0);
-    if (e < totU) {
-      const int i = (int)(e / k), a = min(max(idx64[(int)(e % k)], 0), b - 1);
-      for (int j = 0; j < b; ++j) acc = cadd(acc, cmul(Q[(long long)i * b + j], cconj(as_elem<C>(WH64[(long long)a * b + j]))));
-      U[e] = acc;
-    } else {
-      const long long f = e - totU;
-      const int a = min(max(idx64[(int)(f / n)], 0), b - 1), c = (int)(f % n);
-      for (int j = 0; j < b; ++j) acc = cadd(acc, cmul(as_elem<C>(G64[(long long)a * b + j]), cconj(W[(long long)c * b + j])));
-      Rem[f] = acc;
-    }
+// The kept rows of WH and G' of the reduced SVD, in order, in the path's
+// element type, for U = Q WH[top]^H (m x k) and Rem = G'[top] W^H (k x n): Q
+// and W carry that type's accuracy; for complex64 the complex128 factors are
+// rounded once, since FP64 arithmetic here would cost 64x the FP32 rate and
+// add nothing.
+template <typename C, typename S>
+__global__ void k_gather_top(const S* __restrict__ WH, const S* __restrict__ G, const int* __restrict__ idx, int k,
+                             int b, C* __restrict__ Wt, C* __restrict__ Gt) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < k * b; e += gridDim.x * blockDim.x) {
+    const int a = min(max(idx[e / b], 0), b - 1), c = e % b;
+    const S w = WH[a * b + c], g = G[a * b + c];
+    Wt[e] = cx<C>(w.x, w.y);
+    Gt[e] = cx<C>(g.x, g.y);
   }
 }
 
@@ -890,31 +932,66 @@ cudaError_t launch_fuse(const double2* t, int d, int D, const int n[4], const do
 // K slices of a skinny product (few output tiles, long K) when a scratch of
 // kSplitMax x M x N entries is given
 constexpr int kSplitMax = 8;
+
+template <typename C, int TM, int TN, int RM, int RN, int KG>
+static cudaError_t gemm_tile(char opA, char opB, int M, int N, int K, C alpha, const C* A, int lda, long long sA,
+                             const C* B, int ldb, long long sB, C beta, C* Cm, int ldc, long long sC, int batch,
+                             int S, C* part, cudaStream_t s) {
+  constexpr int NT = (TM / RM) * (TN / RN) * KG;
+  const long long tiles = ((long long)(N + TN - 1) / TN) * ((M + TM - 1) / TM);
+  if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  if (S > 1) {
+    const int kchunk = ((K + S - 1) / S + kGemmK - 1) / kGemmK * kGemmK;
+    S = (K + kchunk - 1) / kchunk;
+    k_gemm<C, TM, TN, RM, RN, KG><<<dim3((unsigned)tiles, 1, S), NT, 0, s>>>(opA, opB, M, N, K, alpha, A, lda, sA, B,
+                                                                            ldb, sB, beta, Cm, ldc, sC, kchunk, part);
+    k_gemm_reduce<C><<<grid_for((long long)M * N, 256), 256, 0, s>>>(part, S, M, N, alpha, beta, Cm, ldc);
+    return cudaGetLastError();
+  }
+  k_gemm<C, TM, TN, RM, RN, KG><<<dim3((unsigned)tiles, 1, batch), NT, 0, s>>>(
+      opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, 0, nullptr);
+  return cudaGetLastError();
+}
+
 template <typename C>
 static cudaError_t gemm_t(char opA, char opB, int M, int N, int K, C alpha, const C* A, int lda, long long sA,
                           const C* B, int ldb, long long sB, C beta, C* Cm, int ldc, long long sC, int batch,
                           cudaStream_t s, void* work = nullptr, size_t work_bytes = 0) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   KTimerScope timer(KC_GEMM, s, 8.0 * M * N * (double)K * batch);
-  const int tiles = ((N + GT - 1) / GT) * ((M + GT - 1) / GT);
-  int S = 1;
-  if (batch == 1 && work && tiles < 2 * 152 && K >= 8 * GK) {
-    S = std::min(kSplitMax, std::max(2, (6 * 152) / tiles));   // about six CTAs an SM
-    S = std::min(S, K / (4 * GK));
+  // slices that bring `tiles` tiles to `want` CTAs, at least four k steps each
+  auto slices = [&](long long tiles, long long want) {
+    if (batch != 1 || !work || tiles >= want || K < 8 * kGemmK) return 1;
+    int S = (int)std::min<long long>(kSplitMax, (want + tiles - 1) / tiles);
+    S = std::max(1, std::min(S, K / (4 * kGemmK)));
     while (S > 1 && (size_t)S * M * N * sizeof(C) > work_bytes) --S;
+    return S;
+  };
+  auto tiles_of = [&](int tm, int tn) { return ((long long)(M + tm - 1) / tm) * ((N + tn - 1) / tn) * batch; };
+#define BBP_GEMM(TM, TN, RM, RN, KG, S)                                                                      \
+  return gemm_tile<C, TM, TN, RM, RN, KG>(opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, \
+                                          batch, S, (C*)work, s)
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    // 64-row tiles of the width that pads N least, once they and the slices
+    // of K fill the SMs; else 32 x 32
+    int tn = 96;
+    for (int w : {64, 48})
+      if ((N + w - 1) / w * w < (N + tn - 1) / tn * tn) tn = w;
+    const long long tiles = tiles_of(64, tn);
+    const int S = slices(tiles, 2 * 152);
+    if (M > 32 && tiles * S >= 152) {
+      if (tn == 96) { BBP_GEMM(64, 96, 4, 6, 1, S); }
+      if (tn == 64) { BBP_GEMM(64, 64, 4, 4, 1, S); }
+      BBP_GEMM(64, 48, 4, 3, 1, S);
+    }
+    BBP_GEMM(32, 32, 2, 2, 1, slices(tiles_of(32, 32), 6 * 152));
+  } else {
+    const long long tiles = tiles_of(16, 16);
+    const int S = slices(tiles, 5 * 152);
+    if (tiles * S >= 2 * 152) { BBP_GEMM(16, 16, 1, 2, 1, S); }
+    BBP_GEMM(8, 8, 1, 1, 2, slices(tiles_of(8, 8), 5 * 152));
   }
-  if (S > 1) {
-    const int kchunk = ((K + S - 1) / S + GK - 1) / GK * GK;
-    S = (K + kchunk - 1) / kchunk;
-    dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, S);
-    k_gemm<C><<<grid, 256, 0, s>>>(opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, kchunk,
-                                   (C*)work);
-    k_gemm_reduce<C><<<grid_for((long long)M * N, 256), 256, 0, s>>>((const C*)work, S, M, N, alpha, beta, Cm, ldc);
-    return cudaGetLastError();
-  }
-  dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, batch);
-  k_gemm<C><<<grid, 256, 0, s>>>(opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, 0, nullptr);
-  return cudaGetLastError();
+#undef BBP_GEMM
 }
 cudaError_t launch_zgemm(char opA, char opB, int M, int N, int K, double2 alpha, const double2* A, int lda,
                          long long sA, const double2* B, int ldb, long long sB, double2 beta, double2* C, int ldc,
@@ -1223,8 +1300,9 @@ static cudaError_t rand_svd(const C* Z, int m, int n, int chi, int b, C* U, C* R
     Go = w.G;
     idxo = w.idx;
   }
-  k_rand_out64<C><<<grid_for((long long)m * k + (long long)k * n, 256), 256, 0, s>>>(Q, m, b, WHo, Go, idxo, W, n, k,
-                                                                                  U, Rem);
+  k_gather_top<C><<<grid_for((long long)k * b, 256), 256, 0, s>>>(WHo, Go, idxo, k, b, Rw, L);
+  if ((e = gemm_t('N', 'C', m, k, b, one, Q, b, 0, Rw, b, 0, zero, U, k, 0, 1, s)) != cudaSuccess) return e;
+  if ((e = gemm_t('N', 'C', k, n, b, one, L, b, 0, W, b, 0, zero, Rem, n, 0, 1, s)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
