@@ -487,6 +487,7 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
   if (tid == 0 && !converged) *status = 1;   // the sweep limit, or an exchange that ran out
   if (cr == 0 && tid == 0) {
     if (counters) {
+      counters[0] = counters[1] = 0;
       counters[2] = sweeps;
       counters[3] = rot_total;
     }

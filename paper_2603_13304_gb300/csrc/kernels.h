@@ -281,7 +281,7 @@ cudaError_t launch_panel_qr_chunked(const double2* A, int m, int n, double2* Q, 
 // conj_t, Z^H (conj Z[c ldz + a]), on a cluster of CTAs with the rows in shared
 // memory (k_jac.cu).  Any of the outputs may be null: G (rotated rows), WH (WH
 // G_0 = G), sigma (row norms), idx (the k largest, in order), *zn2 =
-// ||G_0||_F^2, counters[2], [3] (sweeps, rotations); U (m x k) and Rem (k x n)
+// ||G_0||_F^2, counters ([0], [1] zero, [2] sweeps, [3] rotations); U (m x k) and Rem (k x n)
 // of the truncated SVD of the m x n matrix whose rows (m <= n) or conjugate
 // columns G_0 holds.  jac_fits: whether the problem fits.
 bool jac_fits(int M, int N, size_t elem);

@@ -91,3 +91,17 @@ def test_degenerate_and_vanishing(c64):
 def test_scales(c64, scale):
     rng = np.random.default_rng(6)
     check(gauss(rng, 24, 36) * 0.8 ** np.arange(36)[None, :] * scale, 12, c64)
+
+
+@pytest.mark.parametrize("m,n,chi,plateau", [(400, 380, 32, 8), (400, 380, 32, 0), (260, 300, 21, 3)])
+def test_randomised_cut(m, n, chi, plateau):
+    """The complex128 finish across the cut: a plateau of equal singular values
+    (pairs that are rotated one by one) or none (all at once)."""
+    rng = np.random.default_rng(m + chi)
+    r = 4 * chi
+    a = np.linalg.qr(gauss(rng, m, r))[0]
+    b = np.linalg.qr(gauss(rng, n, r))[0]
+    s = np.exp(-np.arange(r) * 6.0 / chi)
+    if plateau:
+        s[chi - plateau // 2:chi + plateau] = s[chi]
+    check((a * s) @ b.conj().T, chi, True)
