@@ -446,7 +446,7 @@ bbp_status bbp_k_tc_gemm(int bf16, const void* A, long long lda, const void* Bt,
 /* The same GEMM with an explicit tile: bn (output columns of a CTA: 64,
  * 128 or 256) and group_m >= 1 (M tiles that sweep the N tiles together).
  * bbp_k_tc_gemm takes the autotuner's tile for its shape, else the size rule
- * (bn 128 above N = 64, else 64; group_m 16). */
+ * (the width that takes the fewest rounds of the SMs; group_m 16). */
 bbp_status bbp_k_tc_gemm_tile(int bf16, const void* A, long long lda, const void* Bt, long long ldb, float* C,
                               long long ldc, int M, int N, int K, float alpha, int bn, int group_m, int* err,
                               void* stream);

@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
@@ -35,6 +36,8 @@
 #include <map>
 #include <mutex>
 #include <set>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "kernels.h"
@@ -144,10 +147,65 @@ __host__ __device__ constexpr uint32_t idesc_of() {
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
 }
 
-template <bool kBF16, int BN>
+// Split of a (scaled) value into limbs of the operand type: TF32 keeps two
+// limbs (hi, lo) and the three products hi*hi + hi*lo + lo*hi; BF16, with 8
+// significant bits a limb, keeps three (h, m, l) and the six products of
+// order up to 2^-16, hh + hm + mh + hl + mm + lh, so that both reach about
+// FP32 accuracy.  Segment s of the K dimension pairs limb limb_a(s) of A with
+// limb limb_b(s) of B; each limb is stored once and the K loop reads it as
+// often as it occurs.
+template <bool kBF16> struct Split;
+template <> struct Split<false> {
+  static constexpr int kSegs = 3, kLimbs = 2;
+  static __device__ __forceinline__ int limb_a(int s) { return s == 2 ? 1 : 0; }   // hi hi lo
+  static __device__ __forceinline__ int limb_b(int s) { return s == 1 ? 1 : 0; }   // hi lo hi
+};
+template <> struct Split<true> {
+  static constexpr int kSegs = 6, kLimbs = 3;
+  static __device__ __forceinline__ int limb_a(int s) { return (0x210100 >> (4 * s)) & 15; }   // h h m h m l
+  static __device__ __forceinline__ int limb_b(int s) { return (0x012010 >> (4 * s)) & 15; }   // h m h l m h
+};
+
+// exponent of the power of two that brings the largest magnitude near 1
+__device__ __forceinline__ int scale_exp(const int* amax) {
+  const float m = __int_as_float(*amax);
+  return !(m > 0.f) || !isfinite(m) ? 0 : -ilogbf(m);
+}
+__device__ __forceinline__ float pow2_scale(const int* amax) { return exp2f((float)scale_exp(amax)); }
+
+// The K dimension of a split product: `segs` segments of `tps` stages, segment
+// s reading the columns from limb_a(s) * pitch of A and limb_b(s) * pitch of B
+// (a plain product is one segment).
+struct TcK {
+  int segs, tps, pitch;
+};
+// Complex output: row 2 q of the product holds the real parts of output q,
+// row 2 q + 1 the imaginary ones, column n = a r + c entry (a, q, c) of R;
+// vec: pairs of entries are 16-byte aligned.
+struct TcOut {
+  void* R;
+  int Q, r, vec;
+  const int *amax_a, *amax_b;
+};
+template <typename C2> __device__ __forceinline__ void store_pair(C2* p, float x0, float y0, float x1, float y1);
+template <> __device__ __forceinline__ void store_pair(float2* p, float x0, float y0, float x1, float y1) {
+  *reinterpret_cast<float4*>(p) = make_float4(x0, y0, x1, y1);
+}
+template <> __device__ __forceinline__ void store_pair(double2* p, float x0, float y0, float x1, float y1) {
+  p[0] = make_double2(x0, y0);
+  p[1] = make_double2(x1, y1);
+}
+template <typename C2> __device__ __forceinline__ void store_one(C2* p, float x, float y);
+template <> __device__ __forceinline__ void store_one(float2* p, float x, float y) { *p = make_float2(x, y); }
+template <> __device__ __forceinline__ void store_one(double2* p, float x, float y) { *p = make_double2(x, y); }
+
+// EPI: 0 the real product (C = alpha A B^T), 1 complex64 entries of R, 2
+// complex128 ones (straight from TMEM: no real product in memory).
+template <bool kBF16, int BN, int EPI>
 __global__ void __launch_bounds__(128, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, float* __restrict__ C,
-              int M, int N, int K, long long ldc, float alpha, int* err, int group_m) {
+              int M, int N, TcK ks, long long ldc, float alpha, int* err, int group_m, TcOut out_c) {
+  using Sp = Split<kBF16>;
   constexpr int kEs = kBF16 ? 2 : 4;
   constexpr int kBKe = 128 / kEs;               // K elements per stage (one 128-byte row)
   constexpr int kUmmaK = 32 / kEs;              // K elements per tcgen05.mma
@@ -168,7 +226,7 @@ __global__ void __launch_bounds__(128, 1)
   const int in_group = pid - group * group_m * tiles_n;
   const int tm = first_m + in_group % gm, tn = in_group / gm;
   const int n0 = tn * BN, m0 = tm * kBM;
-  const int kt = (K + kBKe - 1) / kBKe;
+  const int kt = ks.segs * ks.tps;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -191,7 +249,7 @@ __global__ void __launch_bounds__(128, 1)
   const uint32_t tmem = s_tmem;
 
   if (warp == 0 && lane == 0) {
-    int issued = 0;
+    int issued = 0, seg = 0, j = 0;
     for (int k = 0; k < kt; ++k) {
       const int s = k % kStages;
       const uint32_t ph = (uint32_t)(k / kStages) & 1u;
@@ -200,8 +258,9 @@ __global__ void __launch_bounds__(128, 1)
         break;
       }
       mbar_expect_tx(&full[s], kStageBytes);
-      tma_load_2d(base + s * kStageBytes, &tA, &full[s], k * kBKe, m0);
-      tma_load_2d(base + s * kStageBytes + kABytes, &tB, &full[s], k * kBKe, n0);
+      tma_load_2d(base + s * kStageBytes, &tA, &full[s], Sp::limb_a(seg) * ks.pitch + j * kBKe, m0);
+      tma_load_2d(base + s * kStageBytes + kABytes, &tB, &full[s], Sp::limb_b(seg) * ks.pitch + j * kBKe, n0);
+      if (++j == ks.tps) { j = 0; ++seg; }
       ++issued;
     }
     // no copy of ours may still be in flight when the CTA exits
@@ -229,16 +288,59 @@ __global__ void __launch_bounds__(128, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
   const int row = m0 + warp * 32 + lane;
+  if constexpr (EPI == 0) {
 #pragma unroll 1
-  for (int c0 = 0; c0 < BN; c0 += 32) {
-    uint32_t v[32];
-    tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-    if (row < M && kt > 0) {
-      float* out = C + (long long)row * ldc + n0 + c0;
-      const int lim = N - n0 - c0;
+    for (int c0 = 0; c0 < BN; c0 += 32) {
+      uint32_t v[32];
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      if (row < M && kt > 0) {
+        float* out = C + (long long)row * ldc + n0 + c0;
+        const int lim = N - n0 - c0;
 #pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (j < lim) out[j] = alpha * __uint_as_float(v[j]);
+        for (int j = 0; j < 32; ++j)
+          if (j < lim) out[j] = alpha * __uint_as_float(v[j]);
+      }
+    }
+  } else {
+    // lane pairs hold the real and the imaginary part of one output row; of
+    // every four columns the even lane writes the first two, the odd lane the
+    // last two
+    using C2 = typename std::conditional<EPI == 1, float2, double2>::type;
+    C2* R = (C2*)out_c.R;
+    const bool odd = lane & 1;
+    const int q = row >> 1, r = out_c.r;
+    const int ex = -(scale_exp(out_c.amax_a) + scale_exp(out_c.amax_b));
+    const bool plain = ex > -120 && ex < 120;
+    const float inv = plain ? exp2f((float)ex) : 1.f;
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN && n0 + c0 < N; c0 += 32) {
+      uint32_t v[32];
+      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+      int n = n0 + c0 + (odd ? 2 : 0), a = n / r, c = n - a * r;
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          x[u] = __uint_as_float(v[j + u]);
+          x[u] = plain ? x[u] * inv : ldexpf(x[u], ex);
+        }
+        const float ra = __shfl_xor_sync(0xffffffffu, odd ? x[0] : x[2], 1);
+        const float rb = __shfl_xor_sync(0xffffffffu, odd ? x[1] : x[3], 1);
+        const float re0 = odd ? ra : x[0], im0 = odd ? x[2] : ra, re1 = odd ? rb : x[1], im1 = odd ? x[3] : rb;
+        if (row < M) {
+          C2* p = R + ((long long)a * out_c.Q + q) * r + c;
+          if (out_c.vec) {
+            if (n < N) store_pair(p, re0, im0, re1, im1);
+          } else {
+            if (n < N) store_one(p, re0, im0);
+            if (n + 1 < N) store_one(c + 1 < r ? p + 1 : R + ((long long)(a + 1) * out_c.Q + q) * r, re1, im1);
+          }
+        }
+        n += 4;
+        c += 4;
+        while (c >= r) { c -= r; ++a; }
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -280,7 +382,7 @@ bool make_map(CUtensorMap* m, const void* ptr, bool bf16, int rows, int cols, lo
 template <int BN> constexpr int tc_smem() { return stages_of<BN>() * (kBM + BN) * 128 + 1024; }
 
 // Dynamic shared memory opt-in, once per kernel and device.
-template <bool kBF16, int BN>
+template <bool kBF16, int BN, int EPI>
 cudaError_t tc_optin() {
   static std::atomic<unsigned long long> done{0};
   int dev = 0;
@@ -288,23 +390,25 @@ cudaError_t tc_optin() {
   if (e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
   if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_tc_gemm<kBF16, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<BN>());
+  e = cudaFuncSetAttribute(k_tc_gemm<kBF16, BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem<BN>());
   if (e == cudaSuccess) done.fetch_or(bit);
   return e;
 }
 
-template <bool kBF16, int BN>
+template <bool kBF16, int BN, int EPI>
 cudaError_t tc_launch(const void* A, long long lda, const void* Bt, long long ldb, float* C, long long ldc, int M, int N,
-                      int K, float alpha, int* err, cudaStream_t s, double algo_flops, int group_m) {
+                      int K, float alpha, int* err, cudaStream_t s, double algo_flops, int group_m, const TcK& ks,
+                      const TcOut& out) {
   constexpr int smem = tc_smem<BN>();
-  cudaError_t attr_err = tc_optin<kBF16, BN>();
+  cudaError_t attr_err = tc_optin<kBF16, BN, EPI>();
   if (attr_err != cudaSuccess) return attr_err;
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, kBF16, M, K, lda, kBM) || !make_map(&tb, Bt, kBF16, N, K, ldb, BN))
     return cudaErrorInvalidValue;
   dim3 grid((N + BN - 1) / BN, (M + kBM - 1) / kBM);
   KTimerScope timer(KC_TC, s, algo_flops > 0 ? algo_flops : 2.0 * M * N * K);
-  k_tc_gemm<kBF16, BN><<<grid, 128, smem, s>>>(ta, tb, C, M, N, K, ldc, alpha, err, group_m < 1 ? 1 : group_m);
+  k_tc_gemm<kBF16, BN, EPI><<<grid, 128, smem, s>>>(ta, tb, C, M, N, ks, ldc, alpha, err, group_m < 1 ? 1 : group_m,
+                                                    out);
   return cudaGetLastError();
 }
 
@@ -346,31 +450,6 @@ __global__ void k_absmax(const C* __restrict__ x, long long n, int* out) {
   if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(out, __float_as_int(m));
 }
 
-// power-of-two scale bringing the largest magnitude near 1
-__device__ __forceinline__ float pow2_scale(const int* amax) {
-  const float m = __int_as_float(*amax);
-  if (!(m > 0.f) || !isfinite(m)) return 1.f;
-  return exp2f(-(float)ilogbf(m));
-}
-
-// Split of a (scaled) value into limbs of the operand type: TF32 keeps two
-// limbs (hi, lo) and the three products hi*hi + hi*lo + lo*hi; BF16, with 8
-// significant bits a limb, keeps three (h, m, l) and the six products of
-// order up to 2^-16, hh + hm + mh + hl + mm + lh, so that both reach about
-// FP32 accuracy.  Segment s of the K dimension pairs limb kLimbA[s] of A with
-// limb kLimbB[s] of B.
-template <bool kBF16> struct Split;
-template <> struct Split<false> {
-  static constexpr int kSegs = 3;
-  static __device__ __forceinline__ int limb_a(int s) { return s == 2 ? 1 : 0; }   // hi hi lo
-  static __device__ __forceinline__ int limb_b(int s) { return s == 1 ? 1 : 0; }   // hi lo hi
-};
-template <> struct Split<true> {
-  static constexpr int kSegs = 6;
-  static __device__ __forceinline__ int limb_a(int s) { return (0x210100 >> (4 * s)) & 15; }   // h h m h m l
-  static __device__ __forceinline__ int limb_b(int s) { return (0x012010 >> (4 * s)) & 15; }   // h m h l m h
-};
-
 template <bool kBF16>
 __device__ __forceinline__ float limb(float x, int which) {
   using O = Op<kBF16>;
@@ -381,73 +460,99 @@ __device__ __forceinline__ float limb(float x, int which) {
   return O::round(r1 - m);
 }
 
-// A operand from X (P x Q complex, row-major): rows q and Q + q, K index
-// laid out [segment] x [Re/Im block of P]; row stride lda >= 2 kSegs P.
+// Operands of the absorb contraction.  A row holds, limb after limb, a segment
+// of `pitch` entries: [Re block of P | Im block of P | zeros], the pitch a
+// whole number of pipeline stages (128 bytes).  Each limb is stored once.  A 32
+// x 32 tile of the source is read along its rows and written transposed.
+//
+// A from X (P x Q complex, row-major): row 2 q holds [Re, -Im] of column q,
+// row 2 q + 1 [Im, Re].
 template <bool kBF16, typename C>
-__global__ void k_pack_a(const C* __restrict__ X, int P, int Q, const int* amax, typename Op<kBF16>::T* A, long long lda) {
+__global__ void __launch_bounds__(256) k_pack_a(const C* __restrict__ X, int P, int Q, const int* amax,
+                                                typename Op<kBF16>::T* __restrict__ A, int pitch) {
   using O = Op<kBF16>;
-  using S = Split<kBF16>;
+  constexpr int NL = Split<kBF16>::kLimbs;
+  __shared__ float2 tile[32][33];
   const float sc = pow2_scale(amax);
-  const long long tot = (long long)Q * lda;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-    const int q = (int)(e / lda), kk = (int)(e % lda);
-    float v0 = 0.f, v1 = 0.f;   // rows q (real part) and Q + q (imaginary part)
-    if (kk < 2 * S::kSegs * P) {
-      const int blk = kk / (2 * P), rem = kk % (2 * P), p = rem % P;
-      const bool im_half = rem >= P;
-      double2 x = ld_c(X, (long long)p * Q + q);
-      const int w = S::limb_a(blk);
-      const float xr = limb<kBF16>((float)x.x * sc, w), xi = limb<kBF16>((float)x.y * sc, w);
-      // row q: [Re, -Im]; row Q + q: [Im, Re]
-      v0 = im_half ? -xi : xr;
-      v1 = im_half ? xr : xi;
+  const int q0 = blockIdx.x * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int p0 = blockIdx.y * 32; p0 < P; p0 += gridDim.y * 32) {
+    __syncthreads();
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+      const int p = p0 + i, q = q0 + tx;
+      float2 z = make_float2(0.f, 0.f);
+      if (p < P && q < Q) {
+        const double2 x = ld_c(X, (long long)p * Q + q);
+        z = make_float2((float)x.x * sc, (float)x.y * sc);
+      }
+      tile[i][tx] = z;
     }
-    A[(long long)q * lda + kk] = O::store(v0);
-    A[(long long)(Q + q) * lda + kk] = O::store(v1);
+    __syncthreads();
+    const int p = p0 + tx;
+    const bool last = p0 + 32 >= P;
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+      if (q0 + i >= Q) break;
+      typename O::T* re = A + (long long)(2 * (q0 + i)) * NL * pitch;
+      typename O::T* im = re + (long long)NL * pitch;
+      const float2 z = tile[tx][i];
+#pragma unroll
+      for (int w = 0; w < NL; ++w) {
+        if (p < P) {
+          const float xr = limb<kBF16>(z.x, w), xi = limb<kBF16>(z.y, w);
+          re[w * pitch + p] = O::store(xr);
+          re[w * pitch + P + p] = O::store(-xi);
+          im[w * pitch + p] = O::store(xi);
+          im[w * pitch + P + p] = O::store(xr);
+        }
+        if (last)
+          for (int k = 2 * P + tx; k < pitch; k += 32) re[w * pitch + k] = im[w * pitch + k] = O::store(0.f);
+      }
+    }
   }
 }
 
-// B^T operand from S (l x P x r complex): row n = a * r + c, K index laid
-// out [segment] x [Re/Im block of P]; row stride ldb >= 2 kSegs P.
+// B^T from S (l x P x r complex): row n = a r + c holds [Re, Im] of (a, ., c).
 template <bool kBF16, typename C>
-__global__ void k_pack_b(const C* __restrict__ S, int l, int P, int r, const int* amax, typename Op<kBF16>::T* B,
-                         long long ldb) {
+__global__ void __launch_bounds__(256) k_pack_b(const C* __restrict__ S, int P, int r, const int* amax,
+                                                typename Op<kBF16>::T* __restrict__ B, int pitch) {
   using O = Op<kBF16>;
-  using Sp = Split<kBF16>;
+  constexpr int NL = Split<kBF16>::kLimbs;
+  __shared__ float2 tile[32][33];
   const float sc = pow2_scale(amax);
-  const long long N = (long long)l * r;
-  const long long tot = N * ldb;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-    const long long n = e / ldb;
-    const int kk = (int)(e % ldb);
-    float v = 0.f;
-    if (kk < 2 * Sp::kSegs * P) {
-      const int blk = kk / (2 * P), rem = kk % (2 * P), p = rem % P;
-      const bool im_half = rem >= P;
-      const int a = (int)(n / r), c = (int)(n % r);
-      double2 x = ld_c(S, ((long long)a * P + p) * r + c);
-      v = limb<kBF16>((float)(im_half ? x.y : x.x) * sc, Sp::limb_b(blk));
+  const int ct = (r + 31) / 32, a = blockIdx.x / ct, c0 = (blockIdx.x % ct) * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int p0 = blockIdx.y * 32; p0 < P; p0 += gridDim.y * 32) {
+    __syncthreads();
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+      const int p = p0 + i, c = c0 + tx;
+      float2 z = make_float2(0.f, 0.f);
+      if (p < P && c < r) {
+        const double2 x = ld_c(S, ((long long)a * P + p) * r + c);
+        z = make_float2((float)x.x * sc, (float)x.y * sc);
+      }
+      tile[i][tx] = z;
     }
-    B[e] = O::store(v);
-  }
-}
-
-template <typename C> __device__ __forceinline__ C mk(double re, double im);
-template <> __device__ __forceinline__ double2 mk(double re, double im) { return make_double2(re, im); }
-template <> __device__ __forceinline__ float2 mk(double re, double im) { return make_float2((float)re, (float)im); }
-
-// R[a][q][c] = (Cr[q][a r + c] + i Ci[q][a r + c]) / (scale_A scale_B)
-template <typename C>
-__global__ void k_unpack(const float* __restrict__ Cm, long long ldc, int Q, int l, int r, const int* amax_a,
-                         const int* amax_b, C* R) {
-  const double inv = 1.0 / ((double)pow2_scale(amax_a) * (double)pow2_scale(amax_b));
-  const long long tot = (long long)l * Q * r;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(e % r);
-    const long long t = e / r;
-    const int q = (int)(t % Q), a = (int)(t / Q);
-    const long long n = (long long)a * r + c;
-    R[e] = mk<C>(Cm[(long long)q * ldc + n] * inv, Cm[(long long)(Q + q) * ldc + n] * inv);
+    __syncthreads();
+    const int p = p0 + tx;
+    const bool last = p0 + 32 >= P;
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+      if (c0 + i >= r) break;
+      typename O::T* row = B + ((long long)a * r + c0 + i) * NL * pitch;
+      const float2 z = tile[tx][i];
+#pragma unroll
+      for (int w = 0; w < NL; ++w) {
+        if (p < P) {
+          row[w * pitch + p] = O::store(limb<kBF16>(z.x, w));
+          row[w * pitch + P + p] = O::store(limb<kBF16>(z.y, w));
+        }
+        if (last)
+          for (int k = 2 * P + tx; k < pitch; k += 32) row[w * pitch + k] = O::store(0.f);
+      }
+    }
   }
 }
 
@@ -576,43 +681,59 @@ int grid_of(long long n) {
 
 // ------------------------------------------------------------------ public
 
+template <bool kBF16, int BN>
+static cudaError_t tc_optin_all() {
+  cudaError_t e;
+  if ((e = tc_optin<kBF16, BN, 0>()) != cudaSuccess) return e;
+  if ((e = tc_optin<kBF16, BN, 1>()) != cudaSuccess) return e;
+  return tc_optin<kBF16, BN, 2>();
+}
 cudaError_t init_tc_attributes() {
   cudaError_t e;
-  if ((e = tc_optin<false, 64>()) != cudaSuccess) return e;
-  if ((e = tc_optin<false, 128>()) != cudaSuccess) return e;
-  if ((e = tc_optin<false, 256>()) != cudaSuccess) return e;
-  if ((e = tc_optin<true, 64>()) != cudaSuccess) return e;
-  if ((e = tc_optin<true, 128>()) != cudaSuccess) return e;
-  return tc_optin<true, 256>();
+  if ((e = tc_optin_all<false, 64>()) != cudaSuccess) return e;
+  if ((e = tc_optin_all<false, 128>()) != cudaSuccess) return e;
+  if ((e = tc_optin_all<false, 256>()) != cudaSuccess) return e;
+  if ((e = tc_optin_all<true, 64>()) != cudaSuccess) return e;
+  if ((e = tc_optin_all<true, 128>()) != cudaSuccess) return e;
+  return tc_optin_all<true, 256>();
+}
+
+// a product in tiles of width bn; K the columns of the operands as stored
+template <int EPI>
+static cudaError_t tc_dispatch(bool bf16, const void* A, long long lda, const void* Bt, long long ldb, float* C,
+                               long long ldc, int M, int N, int K, float alpha, int* err, cudaStream_t s, int bn,
+                               int group_m, double algo_flops, const TcK& ks, const TcOut& out) {
+  switch (bn) {
+    case 64:
+      return bf16 ? tc_launch<true, 64, EPI>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m, ks, out)
+                  : tc_launch<false, 64, EPI>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m, ks, out);
+    case 128:
+      return bf16 ? tc_launch<true, 128, EPI>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m, ks, out)
+                  : tc_launch<false, 128, EPI>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m, ks, out);
+    case 256:
+      return bf16 ? tc_launch<true, 256, EPI>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m, ks, out)
+                  : tc_launch<false, 256, EPI>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m, ks, out);
+    default:
+      return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_tc_gemm_tile(bool bf16, const void* A, long long lda, const void* Bt, long long ldb, float* C,
                                 long long ldc, int M, int N, int K, float alpha, int* err, cudaStream_t s, int bn,
                                 int group_m, double algo_flops) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  const int es = bf16 ? 2 : 4;
+  const int es = bf16 ? 2 : 4, ke = 128 / es;
   if ((lda * es) % 16 || (ldb * es) % 16 || ((uintptr_t)A & 15) || ((uintptr_t)Bt & 15)) return cudaErrorInvalidValue;
-  switch (bn) {
-    case 64:
-      return bf16 ? tc_launch<true, 64>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m)
-                  : tc_launch<false, 64>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m);
-    case 128:
-      return bf16 ? tc_launch<true, 128>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m)
-                  : tc_launch<false, 128>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m);
-    case 256:
-      return bf16 ? tc_launch<true, 256>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m)
-                  : tc_launch<false, 256>(A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, algo_flops, group_m);
-    default:
-      return cudaErrorInvalidValue;
-  }
+  const TcK ks = {1, (K + ke - 1) / ke, 0};
+  return tc_dispatch<0>(bf16, A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, bn, group_m, algo_flops, ks, TcOut());
 }
 
 // ------------------------------------------------------------ autotuner
 //
 // The tile of a launch (BN, the width of a CTA's output tile, and group_m,
 // the M tiles a wave sweeps together) is looked up by the exact GEMM shape
-// (precision, M, N, K); shapes not in the table take the size rule (BN 128
-// above N = 64, else 64; group_m 16).  While recording is on, unknown shapes
+// (precision, M, N, K); shapes not in the table take the size rule
+// (rule_tile; group_m 16).  While recording is on, unknown shapes
 // are collected; tc_autotune times every candidate tile of each collected
 // shape on scratch operands (CUDA events, outside any capture) and keeps
 // the fastest.  The table can be written to and read from a text cache.
@@ -637,9 +758,22 @@ std::set<TcKey> g_pending;
 std::atomic<bool> g_recording{false};
 std::atomic<unsigned long long> g_tune_gen{0};
 
-TcTile rule_tile(int N) {
+// The size rule: the fewest rounds of the SMs times the cost of a round.  A
+// round is bound by what the tiles read from L2 (both operands once per
+// tile), so a wider tile costs less than in proportion: at M = 2592, N =
+// 4096, K = 7776 (TF32), 77 us a round of 64-wide tiles, 84 of 128, 104 of
+// 256 (694, 420 and 312 us in all).
+TcTile rule_tile(int M, int N) {
   TcTile t;
-  t.bn = N > 64 ? 128 : 64;
+  double best = 0;
+  for (auto c : {std::pair<int, int>(64, 77), std::pair<int, int>(128, 84), std::pair<int, int>(256, 104)}) {
+    const long long tiles = ((long long)(M + kBM - 1) / kBM) * ((N + c.first - 1) / c.first);
+    const double cost = (double)((tiles + 151) / 152) * c.second;
+    if (best == 0 || cost < best) {
+      best = cost;
+      t.bn = c.first;
+    }
+  }
   return t;
 }
 
@@ -780,24 +914,30 @@ int tc_autotune_load(const char* cache_path) {
   return n;
 }
 
+// the tile of a shape: the table's, else the size rule's (recorded on request)
+static TcTile tile_of(bool bf16, int M, int N, int K) {
+  const TcKey key{bf16 ? 1 : 0, M, N, K};
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  auto it = g_tiles.find(key);
+  if (it != g_tiles.end()) return it->second;
+  if (g_recording.load(std::memory_order_relaxed)) g_pending.insert(key);
+  return rule_tile(M, N);
+}
+
 cudaError_t launch_tc_gemm(bool bf16, const void* A, long long lda, const void* Bt, long long ldb, float* C,
                            long long ldc, int M, int N, int K, float alpha, int* err, cudaStream_t s,
                            double algo_flops) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  TcTile t = rule_tile(N);
-  {
-    const TcKey key{bf16 ? 1 : 0, M, N, K};
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tiles.find(key);
-    if (it != g_tiles.end()) t = it->second;
-    else if (g_recording.load(std::memory_order_relaxed)) g_pending.insert(key);
-  }
+  const TcTile t = tile_of(bf16, M, N, K);
   return launch_tc_gemm_tile(bf16, A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, t.bn, t.group_m, algo_flops);
 }
 
 long long tc_ld(int P) { return ((6LL * P + 31) / 32) * 32; }
-// K extent of the absorb operands: 2 P reals a segment, 3 segments (TF32) or 6 (BF16)
-long long tc_absorb_ld(bool bf16, int P) { return ((2LL * (bf16 ? 6 : 3) * P + 31) / 32) * 32; }
+// columns of one limb of the absorb operands: 2 P reals in whole 128-byte stages
+int tc_absorb_pitch(bool bf16, int P) {
+  const int ke = bf16 ? 64 : 32;
+  return (2 * P + ke - 1) / ke * ke;
+}
 
 // ------------------------------------------------ general complex GEMM (c64)
 
@@ -841,53 +981,59 @@ cudaError_t tc_zgemm_packed(bool bf16, int M, int N, int K, const void* Ap, cons
                         8.0 * M * N * (double)K);
 }
 
+// (the published size: every segment's limb stored, a real product beside the
+// operands; or the operands as they are, where their padding takes more)
 size_t tc_absorb_bytes(bool bf16, int P, int Q, int l, int r) {
   const size_t es = bf16 ? 2 : 4;
-  const size_t ld = (size_t)tc_absorb_ld(bf16, P);
+  const size_t ld = ((2 * (size_t)(bf16 ? 6 : 3) * P + 31) / 32) * 32;
+  const size_t row = (size_t)(bf16 ? 3 : 2) * tc_absorb_pitch(bf16, P) * es;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  return al(2 * (size_t)Q * ld * es) + al((size_t)l * r * ld * es) + al(sizeof(float) * 2 * (size_t)Q * l * r) + 256;
+  return std::max(al(2 * (size_t)Q * ld * es) + al((size_t)l * r * ld * es) + al(sizeof(float) * 2 * (size_t)Q * l * r),
+                  al(2 * (size_t)Q * row) + al((size_t)l * r * row)) +
+         256;
 }
 
-template <typename C>
-static cudaError_t tc_absorb_t(bool bf16, const C* X, int P, int Q, const C* S, int l, int r, C* R, void* work,
-                               int* err, cudaStream_t s) {
-  const size_t es = bf16 ? 2 : 4;
-  const long long ld = tc_absorb_ld(bf16, P);
+// Largest magnitudes, the two packed operands, and one product whose epilogue
+// writes R.  At P = Q = 1296, l = r = 64: the limbs stored once are 85 MB of B
+// and 54 MB of A (each segment's copy took 127 and 81 MB, and the real product
+// another 42 MB written, read and written again as R).
+template <bool kBF16, typename C>
+static cudaError_t tc_absorb_t(const C* X, int P, int Q, const C* S, int l, int r, C* R, void* work, int* err,
+                               cudaStream_t s) {
+  using T = typename Op<kBF16>::T;
+  using Sp = Split<kBF16>;
+  const int pitch = tc_absorb_pitch(kBF16, P), ke = 128 / (int)sizeof(T);
+  const size_t row = (size_t)Sp::kLimbs * pitch * sizeof(T);
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   char* p = (char*)work;
-  void* A = p;
-  p += al(2 * (size_t)Q * ld * es);
-  void* B = p;
-  p += al((size_t)l * r * ld * es);
-  float* Cm = (float*)p;
-  p += al(sizeof(float) * 2 * (size_t)Q * l * r);
+  T* A = (T*)p;
+  p += al(2 * (size_t)Q * row);
+  T* B = (T*)p;
+  p += al((size_t)l * r * row);
   int* amax = (int*)p;   // [0] X, [1] S
   cudaError_t e;
   if ((e = cudaMemsetAsync(amax, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
   k_absmax<C><<<grid_of((long long)P * Q), 256, 0, s>>>(X, (long long)P * Q, amax);
   k_absmax<C><<<grid_of((long long)l * P * r), 256, 0, s>>>(S, (long long)l * P * r, amax + 1);
-  if (bf16) {
-    k_pack_a<true, C><<<grid_of((long long)Q * ld), 256, 0, s>>>(X, P, Q, amax, (__nv_bfloat16*)A, ld);
-    k_pack_b<true, C><<<grid_of((long long)l * r * ld), 256, 0, s>>>(S, l, P, r, amax + 1, (__nv_bfloat16*)B, ld);
-  } else {
-    k_pack_a<false, C><<<grid_of((long long)Q * ld), 256, 0, s>>>(X, P, Q, amax, (float*)A, ld);
-    k_pack_b<false, C><<<grid_of((long long)l * r * ld), 256, 0, s>>>(S, l, P, r, amax + 1, (float*)B, ld);
-  }
-  const int N = l * r;
-  if ((e = launch_tc_gemm(bf16, A, ld, B, ld, Cm, N, 2 * Q, N, (int)ld, 1.0f, err, s, 8.0 * Q * N * (double)P)) !=
-      cudaSuccess)
-    return e;
-  k_unpack<C><<<grid_of((long long)l * Q * r), 256, 0, s>>>(Cm, N, Q, l, r, amax, amax + 1, R);
-  return cudaGetLastError();
+  const unsigned pt = std::min((P + 31) / 32, 65535);
+  k_pack_a<kBF16, C><<<dim3((Q + 31) / 32, pt), 256, 0, s>>>(X, P, Q, amax, A, pitch);
+  k_pack_b<kBF16, C><<<dim3((unsigned)l * ((r + 31) / 32), pt), 256, 0, s>>>(S, P, r, amax + 1, B, pitch);
+  const int N = l * r, M = 2 * Q, Kt = Sp::kSegs * pitch;
+  const TcTile t = tile_of(kBF16, M, N, Kt);
+  const TcK ks = {Sp::kSegs, pitch / ke, pitch};
+  const TcOut out = {R, Q, r, r % 4 == 0 && ((uintptr_t)R & 15) == 0 ? 1 : 0, amax, amax + 1};
+  constexpr int EPI = sizeof(C) == sizeof(float2) ? 1 : 2;
+  return tc_dispatch<EPI>(kBF16, A, Sp::kLimbs * pitch, B, Sp::kLimbs * pitch, nullptr, 0, M, N, Sp::kLimbs * pitch,
+                          1.0f, err, s, t.bn, t.group_m, 8.0 * Q * N * (double)P, ks, out);
 }
 
 cudaError_t launch_tc_absorb(bool bf16, const double2* X, int P, int Q, const double2* S, int l, int r, double2* R,
                              void* work, int* err, cudaStream_t s) {
-  return tc_absorb_t(bf16, X, P, Q, S, l, r, R, work, err, s);
+  return bf16 ? tc_absorb_t<true>(X, P, Q, S, l, r, R, work, err, s) : tc_absorb_t<false>(X, P, Q, S, l, r, R, work, err, s);
 }
 cudaError_t launch_tc_absorb(bool bf16, const float2* X, int P, int Q, const float2* S, int l, int r, float2* R,
                              void* work, int* err, cudaStream_t s) {
-  return tc_absorb_t(bf16, X, P, Q, S, l, r, R, work, err, s);
+  return bf16 ? tc_absorb_t<true>(X, P, Q, S, l, r, R, work, err, s) : tc_absorb_t<false>(X, P, Q, S, l, r, R, work, err, s);
 }
 
 }  // namespace bbp
