@@ -863,7 +863,7 @@ int Engine::reserve_workers(const std::vector<SweepJob>& jobs, int nstreams) {
 }
 
 template <typename C>
-int Engine::run_sweep(SweepJob& job, SweepWork& w) {
+int Engine::run_sweep(SweepJob& job, SweepWork& w, bool want_log) {
   const SweepPlan& plan = *job.plan;
   const ShapeTrace& tr = job.tr;
   cudaStream_t s = w.stream;
@@ -911,9 +911,15 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w) {
   auto qr_move = [&](int c) -> int {   // centre c -> c + 1
     TShape a = sh[c], b = sh[c + 1];
     const int m = a.l * a.p, n = a.r, kk = std::min(m, n);
-    CK(cudaMemcpyAsync(qrA, slot(pos[c]), sizeof(C) * (size_t)m * n, cudaMemcpyDeviceToDevice, s));
-    CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
-    CK(cudaMemcpyAsync(slot(pos[c]), qrQ, sizeof(C) * (size_t)m * kk, cudaMemcpyDeviceToDevice, s));
+    if (qr_in_place(m, n, sizeof(C))) {
+      KTimerScope timer(KC_QR, s, qr_flops(m, n));
+      CK(launch_bqr(slot(pos[c]), m, n, m, 0, slot(pos[c]), qrR, 0, s));
+    } else {
+      CK(cudaMemcpyAsync(qrA, slot(pos[c]), sizeof(C) * (size_t)m * n, cudaMemcpyDeviceToDevice, s));
+      CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
+      CK(cudaMemcpyAsync(slot(pos[c]), qrQ, sizeof(C) * (size_t)m * kk, cudaMemcpyDeviceToDevice, s));
+      launches += 2;
+    }
     sh[c].r = kk;
     const int t = take();
     CK(launch_zgemm('N', 'N', kk, b.p * b.r, n, one, qrR, n, 0, slot(pos[c + 1]), b.p * b.r, 0, zero, slot(t),
@@ -921,26 +927,32 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w) {
     give(pos[c + 1]);
     pos[c + 1] = t;
     sh[c + 1].l = kk;
-    launches += 4;
+    launches += 2;
     return 0;
   };
   auto lq_move = [&](int c) -> int {   // centre c -> c - 1
     TShape b = sh[c], a = sh[c - 1];
     const int m = b.p * b.r, n = b.l, kk = std::min(m, n);
-    CK(launch_conj_transpose(slot(pos[c]), b.l, b.p * b.r, qrA, s));
-    CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
-    CK(launch_conj_transpose(qrQ, m, kk, slot(pos[c]), s));
+    if (qr_in_place(m, n, sizeof(C))) {
+      KTimerScope timer(KC_QR, s, qr_flops(m, n));
+      CK(launch_blq(slot(pos[c]), n, m, qrR, s));
+    } else {
+      CK(launch_conj_transpose(slot(pos[c]), b.l, b.p * b.r, qrA, s));
+      CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
+      CK(launch_conj_transpose(qrQ, m, kk, slot(pos[c]), s));
+      launches += 2;
+    }
     sh[c].l = kk;
     const int t = take();
     CK(launch_zgemm('N', 'C', a.l * a.p, kk, n, one, slot(pos[c - 1]), n, 0, qrR, n, 0, zero, slot(t), kk, 0, 1, s));
     give(pos[c - 1]);
     pos[c - 1] = t;
     sh[c - 1].r = kk;
-    launches += 4;
+    launches += 2;
     return 0;
   };
   auto normalise = [&](int c) -> int {
-    CK(launch_normalise(slot(pos[c]), sh[c].size(), w.logscale, s));
+    CK(launch_normalise(slot(pos[c]), sh[c].size(), w.logscale, want_log, s));
     launches += 1;
     return 0;
   };
@@ -1042,7 +1054,7 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w) {
     } else {
       const C* cur = Rb[0];
       int rbuf = 1;
-      int ll = l;
+      int ll = l, last = -1;
       long long rest = Q;
       for (int q = 0; q + 1 < st.nout; ++q) {
         const int q1 = rec.out_dims[q];
@@ -1056,18 +1068,24 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w) {
         // the range-finder products stay on the SIMT GEMM: their K is the
         // full split width (2304 at D = 6, chi = 64), where the tensor cores'
         // FP32 accumulation loses an order of magnitude against it
-        CK(svd_call(cur, rows, (int)cols, chi, slot(t), Rb[rbuf], w.svd, w.status, s, qsteps, false, w.status + 1));
+        // the last split's remainder is the new centre tensor
+        if (q + 2 == st.nout) last = take();
+        C* rem = last >= 0 ? slot(last) : Rb[rbuf];
+        CK(svd_call(cur, rows, (int)cols, chi, slot(t), rem, w.svd, w.status, s, qsteps, false, w.status + 1));
         launches += svd_launches(rows, (int)cols, chi, c64, qsteps);
         newpos.push_back(t);
         newsh.push_back(TShape{ll, q1, k});
-        cur = Rb[rbuf];
+        cur = rem;
         rbuf ^= 1;
         ll = k;
       }
       const int qlast = rec.out_dims[st.nout - 1];
-      const int t = take();
-      CK(cudaMemcpyAsync(slot(t), cur, sizeof(C) * (size_t)ll * qlast * r, cudaMemcpyDeviceToDevice, s));
-      ++launches;
+      if (last < 0) {                    // (one out leg: no split)
+        last = take();
+        CK(cudaMemcpyAsync(slot(last), cur, sizeof(C) * (size_t)ll * qlast * r, cudaMemcpyDeviceToDevice, s));
+        ++launches;
+      }
+      const int t = last;
       newpos.push_back(t);
       newsh.push_back(TShape{ll, qlast, r});
       for (int q = st.i; q <= st.j; ++q) give(pos[q]);
@@ -1250,7 +1268,7 @@ int Engine::iter_launch_t() {
       SweepWork& w = *workers->w[u % nstreams];
       const auto& up = ups[u];
       Message& dst = msgs.at({up.recv_block, up.recv_face});
-      if ((e = run_sweep<C>(jobs[u], w))) break;
+      if ((e = run_sweep<C>(jobs[u], w, false))) break;   // (messages are normalised as a whole: no log-scale)
       if ((e = finalize_message<C>(dst, 1 - dst.cur, w, w.stream, (double*)dist_dev.p + u, true))) break;
       CK(cudaMemcpyAsync(status_dev + 2 * u, w.status, 2 * sizeof(int), cudaMemcpyDeviceToDevice, w.stream));
     }

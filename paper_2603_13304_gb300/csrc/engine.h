@@ -193,7 +193,7 @@ class Engine {
   template <typename C>
   int fill_job(const Region& R, const SweepPlan& plan, SweepJob& job, const OpList& ops, std::vector<DBuf*>& tmp);
   int reserve_workers(const std::vector<SweepJob>& jobs, int nstreams);
-  template <typename C> int run_sweep(SweepJob& job, SweepWork& w);
+  template <typename C> int run_sweep(SweepJob& job, SweepWork& w, bool want_log = true);
   template <typename C>
   int finalize_message(Message& m, int which, SweepWork& w, cudaStream_t s, double* dist_slot, bool with_distance);
   template <typename C> int compress_lrn(Message& m, std::vector<TShape>& sh, SweepWork& w, cudaStream_t s);

@@ -317,9 +317,9 @@ __device__ __forceinline__ int columns_per_warp(int width, int nw) {
 
 // RPT: rows a thread holds in the steps; CL: a cluster of more than one CTA.
 template <typename C, int RPT, bool CL>
-__global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* __restrict__ Ag, int m_all, int n, int rb,
-                                                       long long stride, int rows, int dots_by_column,
-                                                       C* __restrict__ Qg, C* __restrict__ Rg) {
+__global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* Ag, int m_all, int n, int rb,
+                                                       long long stride, int rows, int dots_by_column, int conj_t,
+                                                       C* Qg, C* __restrict__ Rg) {
   using R = typename RealT<C>::T;
   constexpr bool c64 = sizeof(R) == 4;
   cg::cluster_group cl = cg::this_cluster();
@@ -365,10 +365,21 @@ __global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* __restrict__ Ag,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
 
-  for (int t = warp; t < mr; t += nw) {
-    const C* src = Ag + (long long)(r0 + t) * n;
+  if (conj_t) {                          // the panel is the conjugate transpose of an n x m matrix
+    for (int c = warp; c < n; c += nw) {
+      const C* src = Ag + (long long)c * m + r0;
 #pragma unroll 4
-    for (int c = lane; c < n; c += 32) A[c * ld + t] = src[c];
+      for (int t = lane; t < mr; t += 32) {
+        const C x = src[t];
+        A[c * ld + t] = mk<C>(x.x, -x.y);
+      }
+    }
+  } else {
+    for (int t = warp; t < mr; t += nw) {
+      const C* src = Ag + (long long)(r0 + t) * n;
+#pragma unroll 4
+      for (int c = lane; c < n; c += 32) A[c * ld + t] = src[c];
+    }
   }
   const int ks = Qg ? (k + kNB - 1) / kNB * kNB : kNB;
   for (int e = tid; e < ks * kNB; e += nt) sv[e] = zero;   // (a last block of fewer columns reads all of T)
@@ -1032,14 +1043,22 @@ __global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* __restrict__ Ag,
       __syncthreads();
     }
   }
-  for (int t = warp; t < mr; t += nw)
-    for (int c = lane; c < k; c += 32) Qg[(long long)(r0 + t) * k + c] = A[c * ld + t];
+  if (conj_t) {                          // Q^H (k x m)
+    for (int c = warp; c < k; c += nw)
+      for (int t = lane; t < mr; t += 32) {
+        const C x = A[c * ld + t];
+        Qg[(long long)c * m + r0 + t] = mk<C>(x.x, -x.y);
+      }
+  } else {
+    for (int t = warp; t < mr; t += nw)
+      for (int c = lane; c < k; c += 32) Qg[(long long)(r0 + t) * k + c] = A[c * ld + t];
+  }
   __syncthreads();
-  leave(Qg + (size_t)r0 * k);
+  leave(conj_t ? Qg + r0 : Qg + (size_t)r0 * k);
 }
 
 template <typename C, int RPT, bool CL>
-cudaError_t bqr_run(const C* A, int m_all, int n, int rb, long long stride, const QrPlan& p, C* Q, C* R,
+cudaError_t bqr_run(const C* A, int m_all, int n, int rb, long long stride, const QrPlan& p, bool conj_t, C* Q, C* R,
                     cudaStream_t s) {
   auto kern = k_bqr<C, RPT, CL>;
   static std::atomic<unsigned long long> done{0};
@@ -1066,29 +1085,30 @@ cudaError_t bqr_run(const C* A, int m_all, int n, int rb, long long stride, cons
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = CL ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, A, m_all, n, rb, stride, p.rows, p.dots_by_column ? 1 : 0, Q, R);
+  return cudaLaunchKernelEx(&cfg, kern, A, m_all, n, rb, stride, p.rows, p.dots_by_column ? 1 : 0, conj_t ? 1 : 0, Q, R);
 }
 
 template <typename C>
-cudaError_t bqr_pick(const C* A, int m_all, int n, int rb, long long stride, const QrPlan& p, bool cl, C* Q, C* R,
-                     cudaStream_t s) {
+cudaError_t bqr_pick(const C* A, int m_all, int n, int rb, long long stride, const QrPlan& p, bool cl, bool conj_t, C* Q,
+                     C* R, cudaStream_t s) {
   switch (p.rpt) {
-    case 1: return cl ? bqr_run<C, 1, true>(A, m_all, n, rb, stride, p, Q, R, s)
-                      : bqr_run<C, 1, false>(A, m_all, n, rb, stride, p, Q, R, s);
-    case 2: return cl ? bqr_run<C, 2, true>(A, m_all, n, rb, stride, p, Q, R, s)
-                      : bqr_run<C, 2, false>(A, m_all, n, rb, stride, p, Q, R, s);
-    case 4: return cl ? bqr_run<C, 4, true>(A, m_all, n, rb, stride, p, Q, R, s)
-                      : bqr_run<C, 4, false>(A, m_all, n, rb, stride, p, Q, R, s);
+    case 1: return cl ? bqr_run<C, 1, true>(A, m_all, n, rb, stride, p, conj_t, Q, R, s)
+                      : bqr_run<C, 1, false>(A, m_all, n, rb, stride, p, conj_t, Q, R, s);
+    case 2: return cl ? bqr_run<C, 2, true>(A, m_all, n, rb, stride, p, conj_t, Q, R, s)
+                      : bqr_run<C, 2, false>(A, m_all, n, rb, stride, p, conj_t, Q, R, s);
+    case 4: return cl ? bqr_run<C, 4, true>(A, m_all, n, rb, stride, p, conj_t, Q, R, s)
+                      : bqr_run<C, 4, false>(A, m_all, n, rb, stride, p, conj_t, Q, R, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 template <typename C>
-cudaError_t bqr_t(const C* A, int m_all, int n, int rb, long long stride, C* Q, C* R, int cluster, cudaStream_t s) {
+cudaError_t bqr_t(const C* A, int m_all, int n, int rb, long long stride, bool conj_t, C* Q, C* R, int cluster,
+                  cudaStream_t s) {
   QrPlan p;
   rb = std::min(rb, m_all);
   if (!qr_plan<C>(rb, n, Q != nullptr, cluster, p)) return cudaErrorInvalidValue;
-  return bqr_pick(A, m_all, n, rb, stride, p, p.cs > 1, Q, R, s);
+  return bqr_pick(A, m_all, n, rb, stride, p, p.cs > 1, conj_t, Q, R, s);
 }
 
 template <typename C>
@@ -1097,7 +1117,7 @@ cudaError_t bqr_optin() {
   for (int rpt : {1, 2, 4})
     for (bool cl : {false, true}) {
       p.rpt = rpt;
-      cudaError_t e = bqr_pick<C>(nullptr, 1, 1, 1, 0, p, cl, nullptr, nullptr, 0);
+      cudaError_t e = bqr_pick<C>(nullptr, 1, 1, 1, 0, p, cl, false, nullptr, nullptr, 0);
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
@@ -1118,11 +1138,18 @@ bool bqr_fits(int m, int n, size_t elem, bool want_q, int cluster) {
 
 cudaError_t launch_bqr(const float2* A, int m_all, int n, int rb, long long stride, float2* Q, float2* R, int cluster,
                        cudaStream_t s) {
-  return bqr_t(A, m_all, n, rb, stride, Q, R, cluster, s);
+  return bqr_t(A, m_all, n, rb, stride, false, Q, R, cluster, s);
 }
 cudaError_t launch_bqr(const double2* A, int m_all, int n, int rb, long long stride, double2* Q, double2* R,
                        int cluster, cudaStream_t s) {
-  return bqr_t(A, m_all, n, rb, stride, Q, R, cluster, s);
+  return bqr_t(A, m_all, n, rb, stride, false, Q, R, cluster, s);
+}
+
+cudaError_t launch_blq(float2* T, int n, int m, float2* R, cudaStream_t s) {
+  return bqr_t<float2>(T, m, n, m, 0, true, T, R, 0, s);
+}
+cudaError_t launch_blq(double2* T, int n, int m, double2* R, cudaStream_t s) {
+  return bqr_t<double2>(T, m, n, m, 0, true, T, R, 0, s);
 }
 
 }  // namespace bbp

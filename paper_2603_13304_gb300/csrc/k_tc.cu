@@ -437,17 +437,30 @@ template <> __device__ __forceinline__ double2 ld_c(const float2* p, long long i
   return make_double2(v.x, v.y);
 }
 
-// largest |Re|, |Im| of n complex entries -> *out (as the bits of a
-// non-negative float, so atomicMax on int orders them)
+// largest |Re|, |Im| of the nx entries of x -> out[0] and of the ny entries of y
+// -> out[1] (as the bits of a non-negative float, so atomicMax on int orders
+// them); the first gx CTAs take x
 template <typename C>
-__global__ void k_absmax(const C* __restrict__ x, long long n, int* out) {
+__global__ void __launch_bounds__(256) k_absmax(const C* __restrict__ x, long long nx, int gx,
+                                                const C* __restrict__ y, long long ny, int* out) {
+  const bool second = (int)blockIdx.x >= gx;
+  const C* p = second ? y : x;
+  const long long n = second ? ny : nx, b = second ? blockIdx.x - gx : blockIdx.x;
+  const long long step = (long long)(second ? gridDim.x - gx : gx) * blockDim.x;
   float m = 0.f;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    double2 v = ld_c(x, i);
+#pragma unroll 4
+  for (long long i = b * blockDim.x + threadIdx.x; i < n; i += step) {
+    const double2 v = ld_c(p, i);
     m = fmaxf(m, fmaxf(fabsf((float)v.x), fabsf((float)v.y)));
   }
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(out, __float_as_int(m));
+  __shared__ float sm[8];
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) m = fmaxf(m, sm[w]);
+    if (m > 0.f) atomicMax(out + (second ? 1 : 0), __float_as_int(m));
+  }
 }
 
 template <bool kBF16>
@@ -1013,8 +1026,10 @@ static cudaError_t tc_absorb_t(const C* X, int P, int Q, const C* S, int l, int 
   int* amax = (int*)p;   // [0] X, [1] S
   cudaError_t e;
   if ((e = cudaMemsetAsync(amax, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
-  k_absmax<C><<<grid_of((long long)P * Q), 256, 0, s>>>(X, (long long)P * Q, amax);
-  k_absmax<C><<<grid_of((long long)l * P * r), 256, 0, s>>>(S, (long long)l * P * r, amax + 1);
+  // (four entries a thread, at most two CTAs an SM for each)
+  auto ctas = [](long long n) { return (int)std::max(1LL, std::min((n + 1023) / 1024, 304LL)); };
+  const long long nx = (long long)P * Q, ns = (long long)l * P * r;
+  k_absmax<C><<<ctas(nx) + ctas(ns), 256, 0, s>>>(X, nx, ctas(nx), S, ns, amax);
   const unsigned pt = std::min((P + 31) / 32, 65535);
   k_pack_a<kBF16, C><<<dim3((Q + 31) / 32, pt), 256, 0, s>>>(X, P, Q, amax, A, pitch);
   k_pack_b<kBF16, C><<<dim3((unsigned)l * ((r + 31) / 32), pt), 256, 0, s>>>(S, P, r, amax + 1, B, pitch);

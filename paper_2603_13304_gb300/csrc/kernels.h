@@ -78,8 +78,10 @@ cudaError_t launch_svd_trunc_rand64(const double2* Z, int m, int n, int chi, dou
 cudaError_t svd_stats(const void* work, int m, int n, int* sweeps, long long* rotations, cudaStream_t s);
 
 // Frobenius norm of a tensor: A /= ||A||, *logscale += log ||A|| (0 norm: logscale = -inf).
-cudaError_t launch_normalise(double2* A, long long n, double* logscale, cudaStream_t s);
-cudaError_t launch_normalise(float2* A, long long n, double* logscale, cudaStream_t s);
+// logscale: two doubles, the second scratch; without want_log the sum of logs may
+// be left as it is (a sweep whose log-scale nobody reads).
+cudaError_t launch_normalise(double2* A, long long n, double* logscale, bool want_log, cudaStream_t s);
+cudaError_t launch_normalise(float2* A, long long n, double* logscale, bool want_log, cudaStream_t s);
 
 // Out-of-place copy with the (l, p, r) -> (r, p, l) transpose, or a plain copy.
 cudaError_t launch_copy_tensor(const double2* src, double2* dst, int l, int p, int r, bool transpose, cudaStream_t s);
@@ -267,6 +269,13 @@ cudaError_t launch_bqr(const float2* A, int m_all, int n, int rb, long long stri
                        cudaStream_t s);
 cudaError_t launch_bqr(const double2* A, int m_all, int n, int rb, long long stride, double2* Q, double2* R,
                        int cluster, cudaStream_t s);
+// T (n x m, row-major) = R^H Q^H from the QR of its conjugate transpose, T^H =
+// Q R: T is overwritten by Q^H (k x m), R is k x n, k = min(m, n).  qr_in_place:
+// whether launch_bqr and launch_blq take an m x n factorisation with Q over
+// its input (else launch_qr with separate buffers).
+cudaError_t launch_blq(float2* T, int n, int m, float2* R, cudaStream_t s);
+cudaError_t launch_blq(double2* T, int n, int m, double2* R, cudaStream_t s);
+bool qr_in_place(int m, int n, size_t elem);
 // Panels taller than one cluster holds (panel_cluster = 0): two-level TSQR
 // over row chunks that each fit one cluster; Q is required, R may be null.
 // panel_chunk_scratch_bytes: the device scratch it needs (0 when the panel
