@@ -1705,19 +1705,30 @@ int Engine::get_message_t(int block, int face, int* k, int* shapes, double* data
   for (int q = 0; q < m.k(); ++q) need += 2 * (size_t)m.sh[m.cur][q].size();
   if (need > cap) return fail(this, 1, "output buffer too small");
   *k = m.k();
-  size_t off = 0;
+  // small messages in one copy (a copy to pageable memory costs about 8 us
+  // whatever its size), large ones tensor by tensor
+  const bool whole = sizeof(C) * m.cap * m.k() <= (size_t)256 << 10;
   std::vector<C> tmp;
+  if (whole) {
+    tmp.resize(m.cap * (size_t)m.k());
+    CK(cudaMemcpyAsync(tmp.data(), m.tensor<C>(m.cur, 0), sizeof(C) * tmp.size(), cudaMemcpyDeviceToHost, stream));
+    CK(cudaStreamSynchronize(stream));
+  }
+  size_t off = 0;
   for (int q = 0; q < m.k(); ++q) {
     const TShape t = m.sh[m.cur][q];
     shapes[3 * q] = t.l;
     shapes[3 * q + 1] = t.p;
     shapes[3 * q + 2] = t.r;
-    tmp.resize(t.size());
-    CK(cudaMemcpyAsync(tmp.data(), m.tensor<C>(m.cur, q), sizeof(C) * t.size(), cudaMemcpyDeviceToHost, stream));
-    CK(cudaStreamSynchronize(stream));
+    if (!whole) {
+      tmp.resize(t.size());
+      CK(cudaMemcpyAsync(tmp.data(), m.tensor<C>(m.cur, q), sizeof(C) * t.size(), cudaMemcpyDeviceToHost, stream));
+      CK(cudaStreamSynchronize(stream));
+    }
+    const C* src = tmp.data() + (whole ? (size_t)q * m.cap : 0);
     for (long long e = 0; e < t.size(); ++e) {
-      data[off + 2 * e] = tmp[e].x;
-      data[off + 2 * e + 1] = tmp[e].y;
+      data[off + 2 * e] = src[e].x;
+      data[off + 2 * e + 1] = src[e].y;
     }
     off += 2 * (size_t)t.size();
   }
