@@ -5,15 +5,17 @@
 //
 //  K1 fuse           double-layer (ket-bra) tensor, Sec. 1.2 / Sec. 2.1
 //  gemm              complex GEMM used for merges, contractions and gauge moves
-//  qr                Householder QR (canonical-form moves, Sec. 2.3.3)
+//  qr                Householder QR (canonical-form moves, Sec. 2.3.3): which
+//                    kernel takes a shape (k_qr.cu, k_panel.cu), and the one
+//                    on device memory for what fits neither
 //  K3 svd_trunc      truncated SVD (Sec. 1.1.1, 1.1.3): one-sided (row) Jacobi;
 //                    in complex64, large matrices are first reduced by a
 //                    randomised subspace iteration and Jacobi runs on the
 //                    small projected matrix
 //  K4 msg_*          message normalisation, phase and distance
 //
-// Large Jacobi problems run on a thread-block cluster (one matrix per
-// cluster, cluster barriers between rounds); every loop is bounded.
+// Jacobi problems run on a cluster's shared memory (k_jac.cu) and, beyond
+// that, on device memory (k_jacobi); every loop is bounded.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 

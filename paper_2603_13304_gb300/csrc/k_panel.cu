@@ -5,7 +5,7 @@
 // cluster's shared memory, so that its block buffers do not fit beside them,
 // take the column-by-column kernel of this file (a few kilobytes of buffers).
 //
-// Convention (the same in both): H = I - tau v v^H, v_j = 1, R has a real
+// Convention (as in k_qr.cu): H = I - tau v v^H, v_j = 1, R has a real
 // diagonal beta_j, the factorisation applies H_j^H.
 #include <cooperative_groups.h>
 
