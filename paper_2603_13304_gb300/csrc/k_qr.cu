@@ -564,14 +564,23 @@ __global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* Ag, int m_all, i
     }
     return f;
   };
-  // W -> F for columns [c0, c1), F to every CTA
-  auto factors = [&](int b0, int c0, int c1, bool fwd) {
+  // The phases of the W and F exchange of columns [c0, c1), armed by one thread
+  // before the block barrier that precedes the dots.  A CTA that owns none of
+  // the columns receives no W and sends no F, so its phase completes as it is
+  // armed; what keeps a peer's next W from arriving before that is that the
+  // peer needs this CTA's W first, and that is sent after the block barrier.
+  auto arm = [&](int c0, int c1) {
     if constexpr (CL) {
       if (tid == 0) {
         const int own = (c1 - cr + cs - 1) / cs - (c0 - cr + cs - 1) / cs;   // own columns in [c0, c1)
         bar_expect(bars + 16, k16 * (uint32_t)(own * cs));
         bar_expect(bars + 24, k16 * (uint32_t)(c1 - c0));
       }
+    }
+  };
+  // W -> F for columns [c0, c1), F to every CTA
+  auto factors = [&](int b0, int c0, int c1, bool fwd) {
+    if constexpr (CL) {
       bar_wait(bars + 16, ph_w, failed);
       ph_w ^= 1;
       // a half warp per own column, dealt over the warps first
@@ -934,6 +943,7 @@ __global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* Ag, int m_all, i
     const int nbB = min(kNB, k - b0), b1 = b0 + nbB, sb = Qg ? b0 : 0;
     if constexpr (c64) steps_rows(b0, nbB, sb);
     else steps_pairs(b0, nbB, sb);
+    if (b1 < n) arm(b1, n);              // (the last exchange's waits are over: a block barrier ends every update)
     __syncthreads();
     if (b1 < n) {
       dots(b0, nbB, b1, n);
@@ -1002,6 +1012,7 @@ __global__ void __launch_bounds__(kQrThreads, 1) k_bqr(const C* Ag, int m_all, i
       update(b0, nbB, b1, k);
     }
     __syncthreads();
+    if (b0 > 0) arm(b0, k);              // the next block's, ahead of a barrier
     if constexpr (c64) {
       for (int t = tid; t < mr; t += nt) {           // a thread per row
         const int g = r0 + t;
