@@ -613,9 +613,9 @@ bbp_status bbp_k_panel_qr(int c64, const void* A, int m, int n, void* Q, void* R
   const long long stride = (long long)m * n;
   if (c64)
     return cuda_status(bbp::launch_panel_qr((const float2*)A, m, n, (float2*)Q, (float2*)R, batch, stride,
-                                            (cudaStream_t)stream, cluster));
+                                            (cudaStream_t)stream, cluster, true));
   return cuda_status(bbp::launch_panel_qr((const double2*)A, m, n, (double2*)Q, (double2*)R, batch, stride,
-                                          (cudaStream_t)stream, cluster));
+                                          (cudaStream_t)stream, cluster, true));
 }
 
 size_t bbp_k_svd_work_bytes_rand(int c64, int m, int n, int chi, int tensor_cores) {

@@ -912,8 +912,7 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w, bool want_log) {
     TShape a = sh[c], b = sh[c + 1];
     const int m = a.l * a.p, n = a.r, kk = std::min(m, n);
     if (qr_in_place(m, n, sizeof(C))) {
-      KTimerScope timer(KC_QR, s, qr_flops(m, n));
-      CK(launch_bqr(slot(pos[c]), m, n, m, 0, slot(pos[c]), qrR, 0, s));
+      CK(launch_qr(slot(pos[c]), m, n, slot(pos[c]), qrR, tau, s));
     } else {
       CK(cudaMemcpyAsync(qrA, slot(pos[c]), sizeof(C) * (size_t)m * n, cudaMemcpyDeviceToDevice, s));
       CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
@@ -933,22 +932,16 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w, bool want_log) {
   auto lq_move = [&](int c) -> int {   // centre c -> c - 1
     TShape b = sh[c], a = sh[c - 1];
     const int m = b.p * b.r, n = b.l, kk = std::min(m, n);
-    if (qr_in_place(m, n, sizeof(C))) {
-      KTimerScope timer(KC_QR, s, qr_flops(m, n));
-      CK(launch_blq(slot(pos[c]), n, m, qrR, s));
-    } else {
-      CK(launch_conj_transpose(slot(pos[c]), b.l, b.p * b.r, qrA, s));
-      CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
-      CK(launch_conj_transpose(qrQ, m, kk, slot(pos[c]), s));
-      launches += 2;
-    }
+    CK(launch_conj_transpose(slot(pos[c]), b.l, b.p * b.r, qrA, s));
+    CK(launch_qr(qrA, m, n, qrQ, qrR, tau, s));
+    CK(launch_conj_transpose(qrQ, m, kk, slot(pos[c]), s));
     sh[c].l = kk;
     const int t = take();
     CK(launch_zgemm('N', 'C', a.l * a.p, kk, n, one, slot(pos[c - 1]), n, 0, qrR, n, 0, zero, slot(t), kk, 0, 1, s));
     give(pos[c - 1]);
     pos[c - 1] = t;
     sh[c - 1].r = kk;
-    launches += 2;
+    launches += 4;
     return 0;
   };
   auto normalise = [&](int c) -> int {

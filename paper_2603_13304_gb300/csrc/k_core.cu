@@ -5,9 +5,7 @@
 //
 //  K1 fuse           double-layer (ket-bra) tensor, Sec. 1.2 / Sec. 2.1
 //  gemm              complex GEMM used for merges, contractions and gauge moves
-//  qr                Householder QR (canonical-form moves, Sec. 2.3.3): which
-//                    kernel takes a shape (k_qr.cu, k_panel.cu), and the one
-//                    on device memory for what fits neither
+//  qr                Householder QR (canonical-form moves, Sec. 2.3.3)
 //  K3 svd_trunc      truncated SVD (Sec. 1.1.1, 1.1.3): one-sided (row) Jacobi;
 //                    in complex64, large matrices are first reduced by a
 //                    randomised subspace iteration and Jacobi runs on the
@@ -429,19 +427,417 @@ __global__ void __launch_bounds__(256) k_qr(C* A, int m, int n, C* Q, C* Rm, C* 
 // a margin for their static shared arrays
 constexpr int kSmemMax = 211 * 1024;
 
-// One-CTA panels of the staged factorisation: what fits beside its scalars.
+// Large dynamic shared memory is opt-in, once per kernel and device.
+template <auto kKernel>
+cudaError_t smem_optin() {
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  if (e == cudaSuccess) done.fetch_or(bit);
+  return e;
+}
+
+// QR with the matrix staged in shared memory, column-major with a padded
+// column stride (m + 1), one warp per column (column c belongs to warp
+// c % 32, lanes run over rows).  Householder step j: every warp applies
+// H_j to its columns right of j, reading the unscaled column j; the owner
+// of column j + 1 then forms the next reflector's parameters, and the owner
+// of column j writes v_j and beta_j once nobody reads column j any more;
+// one barrier per step.  Q is formed in place backwards, the next reflector
+// prefetched into a double buffer, again one barrier per step.  Same
+// convention as cta_householder: R has a real diagonal beta_j,
+// Q = H_0 ... H_{k-1}, H = I - tau v v^H.
 template <typename C>
 struct TsqrSmem {
-  static size_t bytes(int m, int n) {
+  static size_t bytes(int m, int n) {   // column-major (m + 1) x n or row-major m x (n + 1) panel
     const int k = m < n ? m : n;
     return sizeof(C) * ((size_t)m * n + (size_t)(m > n ? m : n) + 2 * (size_t)m + 3 * (size_t)k + 8);
   }
 };
 
-// One staged QR launch (grid = row blocks of rb rows).
+template <typename C>
+__device__ void tsqr_params(const C* col, int j, int m, C* s_tau, C* s_sc, C* s_beta) {
+  // reflector of column j (rows j..m-1); computed by one warp in the
+  // element's real type, with the column scaled by its largest magnitude
+  // first so that tiny columns neither underflow nor divide by zero
+  using R = typename RealOf<C>::T;
+  const int lane = threadIdx.x & 31;
+  const C alpha = col[j];
+  R amax = fmax(fabs(alpha.x), fabs(alpha.y));
+  for (int r = j + 1 + lane; r < m; r += 32) amax = fmax(amax, fmax(fabs(col[r].x), fabs(col[r].y)));
+  for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  const R sa = (amax > (R)0 && isfinite(amax)) ? (R)1 / amax : (R)0;
+  R xn2 = 0;
+  for (int r = j + 1 + lane; r < m; r += 32) xn2 += cabs2(cscale(col[r], sa));
+  xn2 = warp_sum(xn2);
+  if (lane == 0) {
+    C tau = cx<C>(0, 0), sc = cx<C>(0, 0), beta = alpha;
+    if (sa > (R)0 && !(xn2 == (R)0 && alpha.y == (R)0)) {
+      const R ax = alpha.x * sa, ay = alpha.y * sa;          // scaled, |.| <= 1
+      const R bs = -copysign(sqrt(ax * ax + ay * ay + xn2), ax);
+      const R dx = ax - bs, dy = ay, dd = dx * dx + dy * dy;
+      const R ib = (R)1 / bs, idd = sa / dd;                 // 1 / (alpha - beta) = sa conj(d') / |d'|^2
+      tau = cx<C>((bs - ax) * ib, -ay * ib);
+      sc = cx<C>(dx * idd, -dy * idd);
+      beta = cx<C>(bs * amax, 0.0);
+      if (!(isfinite(tau.x) && isfinite(tau.y) && isfinite(sc.x) && isfinite(sc.y) && isfinite(beta.x))) {
+        tau = cx<C>(0, 0);                                     // leave the column as it is
+        sc = cx<C>(0, 0);
+        beta = alpha;
+      }
+    }
+    s_tau[j] = tau;
+    s_sc[j] = sc;
+    s_beta[j] = beta;
+  }
+}
+
+template <typename C>
+__global__ void __launch_bounds__(1024) k_tsqr_smem(const C* __restrict__ Ag, int m_all, int n, C* __restrict__ Q,
+                                                    C* __restrict__ Rm, int rb) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int row0 = blockIdx.x * rb;
+  const int m = min(rb, m_all - row0);
+  Ag += (size_t)row0 * n;
+  if (gridDim.x > 1) Rm += (size_t)blockIdx.x * n * n;
+  const int k = m < n ? m : n;
+  const int ld = m + 1;
+  C* A = (C*)smem_raw;                       // column c at A + c * ld
+  C* vbuf = A + (size_t)ld * n;              // 2 x m
+  C* s_tau = vbuf + 2 * (size_t)m;
+  C* s_sc = s_tau + k;
+  C* s_beta = s_sc + k;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (long long e = threadIdx.x; e < (long long)m * n; e += blockDim.x) {
+    const int r = (int)(e / n), c = (int)(e % n);
+    A[(size_t)c * ld + r] = Ag[e];
+  }
+  __syncthreads();
+  if (warp == 0 && k > 0) tsqr_params(A, 0, m, s_tau, s_sc, s_beta);
+  __syncthreads();
+  // ---- factorisation
+  for (int j = 0; j < k; ++j) {
+    const C* cj = A + (size_t)j * ld;
+    const C tj = s_tau[j], sc = s_sc[j];
+    const C ctau = cconj(tj);
+    if (j > 0 && warp == (j - 1) % nw) {     // finalise column j - 1 (no longer read)
+      C* cp = A + (size_t)(j - 1) * ld;
+      const C scp = s_sc[j - 1];
+      for (int r = j + lane; r < m; r += 32) cp[r] = cmul(cp[r], scp);
+      if (lane == 0) cp[j - 1] = s_beta[j - 1];
+    }
+    if (!(tj.x == 0 && tj.y == 0)) {
+      for (int c = j + 1 + ((warp - (j + 1)) % nw + nw) % nw; c < n; c += nw) {
+        C* cc = A + (size_t)c * ld;
+        C acc = cx<C>(0, 0);
+        for (int r = j + 1 + lane; r < m; r += 32) acc = cadd(acc, cmulc(cj[r], cc[r]));
+        acc.x = warp_sum(acc.x);
+        acc.y = warp_sum(acc.y);
+        // v^H a = a_j + conj(sc) sum conj(x_r) a_r
+        const C dot = cadd(cc[j], cmulc(sc, acc));
+        const C f = cmul(ctau, dot);       // a -= conj(tau) v (v^H a)
+        const C fs = cmul(f, sc);
+        for (int r = j + 1 + lane; r < m; r += 32) cc[r] = csub(cc[r], cmul(cj[r], fs));
+        if (lane == 0) cc[j] = csub(cc[j], f);
+      }
+    }
+    __syncwarp();
+    if (j + 1 < k && warp == (j + 1) % nw) tsqr_params(A + (size_t)(j + 1) * ld, j + 1, m, s_tau, s_sc, s_beta);
+    __syncthreads();
+  }
+  if (k > 0 && warp == (k - 1) % nw) {
+    C* cp = A + (size_t)(k - 1) * ld;
+    const C scp = s_sc[k - 1];
+    for (int r = k + lane; r < m; r += 32) cp[r] = cmul(cp[r], scp);
+    if (lane == 0) cp[k - 1] = s_beta[k - 1];
+  }
+  __syncthreads();
+  if (Rm) {
+    const int krows = gridDim.x > 1 ? n : k;
+    for (long long e = threadIdx.x; e < (long long)krows * n; e += blockDim.x) {
+      const int i = (int)(e / n), c = (int)(e % n);
+      Rm[e] = (i < k && c >= i) ? A[(size_t)c * ld + i] : cx<C>(0, 0);
+    }
+  }
+  if (!Q) return;
+  // ---- Q = H_0 ... H_{k-1} [I; 0], backwards, in place over columns 0..k-1
+  if (warp == (k - 1) % nw && k > 0) {
+    const C* cp = A + (size_t)(k - 1) * ld;
+    for (int r = k - 1 + lane; r < m; r += 32) vbuf[((k - 1) & 1) * m + r] = (r == k - 1) ? cx<C>(1, 0) : cp[r];
+  }
+  __syncthreads();
+  for (int i = k - 1; i >= 0; --i) {
+    const C* v = vbuf + (i & 1) * m;
+    const C ti = s_tau[i];
+    for (int c = i + 1 + ((warp - (i + 1)) % nw + nw) % nw; c < k; c += nw) {
+      C* cc = A + (size_t)c * ld;
+      C acc = cx<C>(0, 0);
+      for (int r = i + lane; r < m; r += 32) acc = cadd(acc, cmulc(v[r], cc[r]));
+      acc.x = warp_sum(acc.x);
+      acc.y = warp_sum(acc.y);
+      const C f = cmul(ti, acc);
+      for (int r = i + lane; r < m; r += 32) cc[r] = csub(cc[r], cmul(v[r], f));
+    }
+    if (warp == i % nw) {                   // column i := e_i - tau_i v_i
+      C* ci = A + (size_t)i * ld;
+      const C mt = cx<C>(-ti.x, -ti.y);
+      for (int r = lane; r < m; r += 32) {
+        C q = cx<C>(0, 0);
+        if (r == i) q = cx<C>(1.0 - ti.x, -ti.y);
+        else if (r > i) q = cmul(mt, v[r]);
+        ci[r] = q;
+      }
+    }
+    if (i > 0 && warp == (i - 1) % nw) {    // prefetch v_{i-1}
+      const C* cp = A + (size_t)(i - 1) * ld;
+      for (int r = i - 1 + lane; r < m; r += 32) vbuf[((i - 1) & 1) * m + r] = (r == i - 1) ? cx<C>(1, 0) : cp[r];
+    }
+    __syncthreads();
+  }
+  for (long long e = threadIdx.x; e < (long long)m * k; e += blockDim.x) {
+    const int r = (int)(e / k), c = (int)(e % k);
+    Q[e] = A[(size_t)c * ld + r];
+  }
+}
+
+
+// complex64 variant of k_tsqr_smem: the panel is kept row-major with an odd
+// row stride (n + 1, so that a warp reading one column down 32 rows touches
+// distinct banks), global loads and stores run along rows, and the columns a
+// warp works on are cached in registers: lane l holds rows l + 32 i,
+// i < MAXR (m <= 32 MAXR), so every column pass issues its loads back to
+// back; 16 warps.  Same steps, barriers and results as k_tsqr_smem.
+template <int MAXR>
+__device__ __forceinline__ void tsqr_params_reg(const float2* A, int ldr, int c, int j, int m, float2* s_tau,
+                                                float2* s_sc, float2* s_beta) {
+  const int lane = threadIdx.x & 31;
+  float2 x[MAXR];
+#pragma unroll
+  for (int i = 0; i < MAXR; ++i) {
+    const int r = lane + 32 * i;
+    x[i] = (r > j && r < m) ? A[(size_t)r * ldr + c] : make_float2(0.f, 0.f);
+  }
+  const float2 alpha = A[(size_t)j * ldr + c];
+  float amax = fmaxf(fabsf(alpha.x), fabsf(alpha.y));
+#pragma unroll
+  for (int i = 0; i < MAXR; ++i) amax = fmaxf(amax, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  const float sa = (amax > 0.f && isfinite(amax)) ? 1.f / amax : 0.f;
+  float xn2 = 0.f;
+#pragma unroll
+  for (int i = 0; i < MAXR; ++i) xn2 += (x[i].x * sa) * (x[i].x * sa) + (x[i].y * sa) * (x[i].y * sa);
+  xn2 = warp_sum(xn2);
+  if (lane == 0) {
+    float2 tau = make_float2(0.f, 0.f), sc = make_float2(0.f, 0.f), beta = alpha;
+    if (sa > 0.f && !(xn2 == 0.f && alpha.y == 0.f)) {
+      const float ax = alpha.x * sa, ay = alpha.y * sa;
+      const float bs = -copysignf(sqrtf(ax * ax + ay * ay + xn2), ax);
+      const float dx = ax - bs, dy = ay, dd = dx * dx + dy * dy;
+      const float ib = 1.f / bs, idd = sa / dd;
+      tau = make_float2((bs - ax) * ib, -ay * ib);
+      sc = make_float2(dx * idd, -dy * idd);
+      beta = make_float2(bs * amax, 0.f);
+      if (!(isfinite(tau.x) && isfinite(tau.y) && isfinite(sc.x) && isfinite(sc.y) && isfinite(beta.x))) {
+        tau = make_float2(0.f, 0.f);
+        sc = make_float2(0.f, 0.f);
+        beta = alpha;
+      }
+    }
+    s_tau[j] = tau;
+    s_sc[j] = sc;
+    s_beta[j] = beta;
+  }
+}
+
+inline size_t tsqr_reg_bytes(int m, int n) {
+  const int k = m < n ? m : n;
+  return sizeof(float2) * ((size_t)m * (n + 1) + 2 * (size_t)m + 3 * (size_t)k + 8);
+}
+
+template <int MAXR>
+__global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ Ag, int m_all, int n, float2* Q,
+                                                     float2* Rm, int rb) {
+  using C = float2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int row0 = blockIdx.x * rb;
+  const int m = min(rb, m_all - row0);
+  Ag += (size_t)row0 * n;
+  if (gridDim.x > 1) Rm += (size_t)blockIdx.x * n * n;
+  const int k = m < n ? m : n;
+  const int ldr = n + 1;
+  C* A = (C*)smem_raw;                       // (r, c) at A[r * ldr + c]
+  C* vbuf = A + (size_t)m * ldr;
+  C* s_tau = vbuf + 2 * (size_t)m;
+  C* s_sc = s_tau + k;
+  C* s_beta = s_sc + k;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int c0 = 0; c0 < n; c0 += 64)
+    for (int r0 = warp * 4; r0 < m; r0 += nw * 4) {
+      C v[4][2];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = r0 + q, c = c0 + lane + 32 * h;
+          v[q][h] = (r < m && c < n) ? Ag[(size_t)r * n + c] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = r0 + q, c = c0 + lane + 32 * h;
+          if (r < m && c < n) A[(size_t)r * ldr + c] = v[q][h];
+        }
+    }
+  __syncthreads();
+  if (warp == 0 && k > 0) tsqr_params_reg<MAXR>(A, ldr, 0, 0, m, s_tau, s_sc, s_beta);
+  __syncthreads();
+  for (int j = 0; j < k; ++j) {
+    const C tj = s_tau[j], sc = s_sc[j];
+    const C ctau = cconj(tj);
+    if (j > 0 && warp == (j - 1) % nw) {     // finalise column j - 1
+      const C scp = s_sc[j - 1];
+      for (int r = j + lane; r < m; r += 32) A[(size_t)r * ldr + j - 1] = cmul(A[(size_t)r * ldr + j - 1], scp);
+      if (lane == 0) A[(size_t)(j - 1) * ldr + j - 1] = s_beta[j - 1];
+    }
+    const int c0 = j + 1 + ((warp - (j + 1)) % nw + nw) % nw;
+    if (!(tj.x == 0.f && tj.y == 0.f) && c0 < n) {
+      C xj[MAXR];
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) {
+        const int r = lane + 32 * i;
+        xj[i] = (r > j && r < m) ? A[(size_t)r * ldr + j] : make_float2(0.f, 0.f);
+      }
+      for (int c = c0; c < n; c += nw) {
+        C y[MAXR];
+#pragma unroll
+        for (int i = 0; i < MAXR; ++i) {
+          const int r = lane + 32 * i;
+          y[i] = (r > j && r < m) ? A[(size_t)r * ldr + c] : make_float2(0.f, 0.f);
+        }
+        C a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < MAXR; i += 2) {
+          a0 = cadd(a0, cmulc(xj[i], y[i]));
+          if (i + 1 < MAXR) a1 = cadd(a1, cmulc(xj[i + 1], y[i + 1]));
+        }
+        C acc = cadd(a0, a1);
+        acc.x = warp_sum(acc.x);
+        acc.y = warp_sum(acc.y);
+        const C ajc = A[(size_t)j * ldr + c];
+        const C dot = cadd(ajc, cmulc(sc, acc));
+        const C f = cmul(ctau, dot);
+        const C fs = cmul(f, sc);
+#pragma unroll
+        for (int i = 0; i < MAXR; ++i) {
+          const int r = lane + 32 * i;
+          if (r > j && r < m) A[(size_t)r * ldr + c] = csub(y[i], cmul(xj[i], fs));
+        }
+        __syncwarp();
+        if (lane == 0) A[(size_t)j * ldr + c] = csub(ajc, f);
+      }
+    }
+    __syncwarp();
+    if (j + 1 < k && warp == (j + 1) % nw) tsqr_params_reg<MAXR>(A, ldr, j + 1, j + 1, m, s_tau, s_sc, s_beta);
+    __syncthreads();
+  }
+  if (k > 0 && warp == (k - 1) % nw) {
+    const C scp = s_sc[k - 1];
+    for (int r = k + lane; r < m; r += 32) A[(size_t)r * ldr + k - 1] = cmul(A[(size_t)r * ldr + k - 1], scp);
+    if (lane == 0) A[(size_t)(k - 1) * ldr + k - 1] = s_beta[k - 1];
+  }
+  __syncthreads();
+  if (Rm) {
+    const int krows = gridDim.x > 1 ? n : k;
+    for (int i = warp; i < krows; i += nw)
+      for (int c = lane; c < n; c += 32)
+        Rm[(size_t)i * n + c] = (i < k && c >= i) ? A[(size_t)i * ldr + c] : make_float2(0.f, 0.f);
+  }
+  if (!Q) return;
+  if (k > 0 && warp == (k - 1) % nw)
+    for (int r = k - 1 + lane; r < m; r += 32)
+      vbuf[((k - 1) & 1) * m + r] = (r == k - 1) ? make_float2(1.f, 0.f) : A[(size_t)r * ldr + k - 1];
+  __syncthreads();
+  for (int i = k - 1; i >= 0; --i) {
+    const C* v = vbuf + (i & 1) * m;
+    const C ti = s_tau[i];
+    const int c0 = i + 1 + ((warp - (i + 1)) % nw + nw) % nw;
+    const bool own_i = warp == i % nw;
+    if (c0 < k || own_i) {
+      C vv[MAXR];
+#pragma unroll
+      for (int q = 0; q < MAXR; ++q) {
+        const int r = lane + 32 * q;
+        vv[q] = (r >= i && r < m) ? v[r] : make_float2(0.f, 0.f);
+      }
+      for (int c = c0; c < k; c += nw) {
+        C y[MAXR];
+#pragma unroll
+        for (int q = 0; q < MAXR; ++q) {
+          const int r = lane + 32 * q;
+          y[q] = (r >= i && r < m) ? A[(size_t)r * ldr + c] : make_float2(0.f, 0.f);
+        }
+        C a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < MAXR; q += 2) {
+          a0 = cadd(a0, cmulc(vv[q], y[q]));
+          if (q + 1 < MAXR) a1 = cadd(a1, cmulc(vv[q + 1], y[q + 1]));
+        }
+        C acc = cadd(a0, a1);
+        acc.x = warp_sum(acc.x);
+        acc.y = warp_sum(acc.y);
+        const C f = cmul(ti, acc);
+#pragma unroll
+        for (int q = 0; q < MAXR; ++q) {
+          const int r = lane + 32 * q;
+          if (r >= i && r < m) A[(size_t)r * ldr + c] = csub(y[q], cmul(vv[q], f));
+        }
+      }
+      if (own_i) {                          // column i := e_i - tau_i v_i
+        const C mt = make_float2(-ti.x, -ti.y);
+#pragma unroll
+        for (int q = 0; q < MAXR; ++q) {
+          const int r = lane + 32 * q;
+          if (r < m)
+            A[(size_t)r * ldr + i] =
+                (r == i) ? make_float2(1.f - ti.x, -ti.y) : (r > i ? cmul(mt, vv[q]) : make_float2(0.f, 0.f));
+        }
+      }
+    }
+    if (i > 0 && warp == (i - 1) % nw)
+      for (int r = i - 1 + lane; r < m; r += 32)
+        vbuf[((i - 1) & 1) * m + r] = (r == i - 1) ? make_float2(1.f, 0.f) : A[(size_t)r * ldr + i - 1];
+    __syncthreads();
+  }
+  for (int r = warp; r < m; r += nw)
+    for (int c = lane; c < k; c += 32) Q[(size_t)r * k + c] = A[(size_t)r * ldr + c];
+}
+
+// One staged QR launch (grid = row blocks): the register-cached kernel for
+// complex64 panels of at most 512 rows per block, the generic one otherwise.
+template <auto kKernel, typename C>
+cudaError_t tsqr_run(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, int threads, size_t bytes, cudaStream_t s) {
+  cudaError_t e = smem_optin<kKernel>();
+  if (e != cudaSuccess) return e;
+  kKernel<<<(m_all + rb - 1) / rb, threads, bytes, s>>>(Ag, m_all, n, Q, Rm, rb);
+  return cudaGetLastError();
+}
+
 template <typename C>
 cudaError_t tsqr_launch(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, cudaStream_t s) {
-  return launch_bqr(Ag, m_all, n, rb, (long long)rb * n, Q, Rm, 0, s);
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    const size_t sr = tsqr_reg_bytes(rb, n);
+    if (sr <= (size_t)kSmemMax) {
+      if (rb <= 128) return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, 512, sr, s);
+      if (rb <= 256) return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, 512, sr, s);
+      if (rb <= 512) return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, 512, sr, s);
+    }
+  }
+  return tsqr_run<k_tsqr_smem<C>>(Ag, m_all, n, Q, Rm, rb, 1024, TsqrSmem<C>::bytes(rb, n), s);
 }
 
 // ---------------------------------------------------------------- K3 Jacobi
@@ -681,20 +1077,6 @@ __global__ void k_svd_out(SvdWork<C> w, int m, int n, int k, double floor_rel, C
 
 // Rows below sqrt(floor_rel) ||Z|| are left unrotated (eps^2 of the type).
 template <typename C> constexpr double floor_rel_of() { return sizeof(typename RealOf<C>::T) == 8 ? 1e-32 : 1e-14; }
-
-// Large dynamic shared memory is opt-in, once per kernel and device.
-template <auto kKernel>
-cudaError_t smem_optin() {
-  static std::atomic<unsigned long long> done{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-  if (e == cudaSuccess) done.fetch_or(bit);
-  return e;
-}
 
 // Jacobi on the M x N rows of w in global memory, for problems that no
 // cluster's shared memory holds: a cluster of up to 8 CTAs.
@@ -1129,12 +1511,13 @@ static cudaError_t qr_t(C* A, int m, int n, C* Q, C* R, C* tau, cudaStream_t s) 
   }
   return cudaGetLastError();
 }
+// One CTA or one cluster holds the matrix before the first entry of Q is
+// written, so Q may overwrite A (the canonical moves do that: two copies less).
 bool qr_in_place(int m, int n, size_t elem) {
-  const size_t sm = elem == sizeof(double2) ? TsqrSmem<double2>::bytes(m, n) : TsqrSmem<float2>::bytes(m, n);
-  if (sm > (size_t)kSmemMax && (m < n || panel_cluster(m, n, elem) == 0)) return false;
-  return bqr_fits(m, n, elem, true);
+  const bool c128 = elem == sizeof(double2);
+  const size_t sm = c128 ? TsqrSmem<double2>::bytes(m, n) : TsqrSmem<float2>::bytes(m, n);
+  return sm <= (size_t)kSmemMax || (m >= n && panel_cluster(m, n, elem) > 0);
 }
-
 // R factor only (Q discarded): row blocks that fit shared memory are
 // factorised independently and their R's stacked and factorised again.
 // R factor of a panel too wide for the staged kernels: Householder in
@@ -1907,6 +2290,11 @@ cudaError_t launch_mps_dot(const ChainDesc& a, const ChainDesc& b, bool c64, dou
 // (done once up front so that no attribute call falls inside a stream capture).
 cudaError_t init_kernel_attributes() {
   cudaError_t e;
+  if ((e = smem_optin<k_tsqr_smem<double2>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_smem<float2>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<4>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<8>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<16>>()) != cudaSuccess) return e;
   for (const void* f : {(const void*)k_msg_normalise<double2>, (const void*)k_msg_normalise<float2>,
                         (const void*)k_mps_dot<double2>, (const void*)k_mps_dot<float2>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;

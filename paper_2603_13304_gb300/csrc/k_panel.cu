@@ -1,12 +1,28 @@
-// Which tall panels a thread-block cluster holds (Sec. 2.3.3: the canonical
-// moves and the orthonormalisations of the truncation), how they are
-// launched, and the two-level TSQR over row chunks for taller ones.  The
-// factorisation itself is the blocked one of k_qr.cu; panels that fill the
-// cluster's shared memory, so that its block buffers do not fit beside them,
-// take the column-by-column kernel of this file (a few kilobytes of buffers).
+// Householder QR of tall panels on a thread-block cluster (Sec. 2.3.3: the
+// canonical moves and the orthonormalisations of the truncation).
 //
-// Convention (as in k_qr.cu): H = I - tau v v^H, v_j = 1, R has a real
-// diagonal beta_j, the factorisation applies H_j^H.
+// A panel A (m x n, m >= n, row-major) is cut into row slices of 32 MAXR
+// rows, one per CTA of a cluster of cs <= 16 CTAs; each slice stays in that
+// CTA's shared memory (column-major, zero-padded to 32 MAXR rows) for the
+// whole factorisation, and lane l of a warp caches rows l + 32 i of the
+// columns it works on.  Householder step j needs three sums over all rows
+// below the diagonal: the squared norm of column j, and x^H a_c for every
+// trailing column c (x = column j below row j).  Because the reflector is
+// v = [1; x / (alpha - beta)], v^H a_c = a_jc + conj(sc) x^H a_c follows from
+// those raw sums and row j, so one cluster-wide exchange per column
+// suffices.  The exchange is pushed: every CTA stores its partial sums (and
+// the owner of row j stores row j) straight into every CTA's receive buffer
+// in distributed shared memory before the cluster barrier, so that after it
+// every CTA reads only its own shared memory and forms the same reflector
+// from the same values in the same order (bitwise identical in every CTA).
+// Q = H_0 ... H_{k-1} [I; 0] is then formed in place backwards with one
+// exchange per reflector.
+//
+// Convention (the same as the one-CTA kernels): H = I - tau v v^H, v_j = 1,
+// R has a real diagonal beta_j, the factorisation applies H_j^H.  Column
+// norms are exchanged as (power-of-two scale, scaled sum of squares) pairs in
+// the element's real type, so complex64 columns neither overflow nor
+// underflow when squared and the complex64 kernel does no FP64 arithmetic.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -57,12 +73,50 @@ template <typename R> __device__ __forceinline__ R wmax(R v) {
   return v;
 }
 
+// y[q] for a warp-uniform q, by bit masks (a select chain here is turned
+// into an indexed access, which puts the array in local memory)
+template <int MAXR>
+__device__ __forceinline__ float2 pick(const float2 (&y)[MAXR], int q) {
+  unsigned a = 0, b = 0;
+#pragma unroll
+  for (int i = 0; i < MAXR; ++i) {
+    const unsigned msk = q == i ? ~0u : 0u;
+    a |= msk & __float_as_uint(y[i].x);
+    b |= msk & __float_as_uint(y[i].y);
+  }
+  return make_float2(__uint_as_float(a), __uint_as_float(b));
+}
+template <int MAXR>
+__device__ __forceinline__ double2 pick(const double2 (&y)[MAXR], int q) {
+  unsigned long long a = 0, b = 0;
+#pragma unroll
+  for (int i = 0; i < MAXR; ++i) {
+    const unsigned long long msk = q == i ? ~0ull : 0ull;
+    a |= msk & (unsigned long long)__double_as_longlong(y[i].x);
+    b |= msk & (unsigned long long)__double_as_longlong(y[i].y);
+  }
+  return make_double2(__longlong_as_double((long long)a), __longlong_as_double((long long)b));
+}
+
 constexpr int kPanelThreads = 512;
 constexpr int kPanelSmemMax = 227 * 1024;
 constexpr int kQBlock = 8;               // reflectors a block of the Q formation
 
-// The published minimum (bbp_k_panel_cluster) is that of row slices of 32,
-// 64, ... rows with these exchange buffers beside them, in elements: the slice (n columns of ld >= 32
+// distributed shared memory through 32-bit shared-window addresses
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t dsmem_addr(uint32_t a, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_dsmem(uint32_t a, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_dsmem(uint32_t a, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+
+// Shared memory of one CTA, in elements: the slice (n columns of ld >= 32
 // MAXR entries), the receive buffers of the partial sums ([2][cs][n], by
 // step parity and source CTA), row j ([2][n]), the gathered sums (n, when
 // staged), the partial norms ([2][cs]), tau of every step (n, when Q is
@@ -90,6 +144,524 @@ __host__ __device__ inline PanelLayout panel_layout(int maxr, int n, int cs, boo
   L.ring = o; o += 6;
   L.bytes = sizeof(C) * o;
   return L;
+}
+
+// Householder step j, with the partial sums of step j already received:
+//  gather   threads c > j sum the received partial dots of column c (in
+//           source order); one thread forms the reflector from the partial
+//           norms and row j
+//  pass     every warp forms the updated column j + 1 in registers from the
+//           step's reflector and factor (x' = x - v f_{j+1}), updates its
+//           columns c > j + 1 and, from the same registers, takes the
+//           partial dots x'^H a_c of step j + 1 and pushes them (and row
+//           j + 1, from its owner CTA) to every CTA; the warp of column j + 1
+//           pushes its partial norm and stores the column after the cluster
+//           barrier, when no warp reads the old one any more
+// (one block barrier and one cluster barrier per step).  Column c is always
+// worked on by warp c mod nw, so a warp's own deferred stores and later loads
+// of a column are ordered by program order.  Column j stays unscaled while it
+// is read as the reflector of step j; its warp scales it in the next step.
+template <typename C, int MAXR>
+__global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restrict__ Ag, int m, int n,
+                                                            C* __restrict__ Qg, C* __restrict__ Rg, long long stride,
+                                                            int ld, int use_gs, int scaled) {
+  using R = typename Real<C>::T;
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), cr = (int)cl.block_rank();
+  const long long panel = blockIdx.x / cs;
+  Ag += panel * stride;
+  if (Qg) Qg += panel * stride;
+  if (Rg) Rg += panel * (long long)n * n;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const PanelLayout L = panel_layout<C>(MAXR, n, cs, Qg != nullptr, (ld & 1) != 0, use_gs != 0);
+  C* A = (C*)smem_raw;                   // local row t of column c at A[c * ld + t]
+  C* recv = A + L.recv;
+  C* rowb = A + L.rowb;
+  C* gs = A + L.gs;
+  C* pp = A + L.pp;                      // (scale, scaled sum of squares)
+  C* s_tau = A + L.tau;
+  C* ring = A + L.ring;                  // [2][3]: tau, sc, diagonal
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  constexpr int rows = 32 * MAXR;
+  const int r0 = cr * rows;
+  const int mr = max(0, min(rows, m - r0));
+  const int k = min(m, n);
+  const C zero = mkc<C>(0, 0), one = mkc<C>(1, 0);
+  // lane q < cs pushes to CTA q
+  const uint32_t recv_q = lane < cs ? dsmem_addr(smem_addr(recv), lane) : 0u;
+  const uint32_t rowb_q = lane < cs ? dsmem_addr(smem_addr(rowb), lane) : 0u;
+  const uint32_t pp_q = lane < cs ? dsmem_addr(smem_addr(pp), lane) : 0u;
+
+  for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+    const int t = e / n, c = e % n;
+    A[(size_t)c * ld + t] = t < mr ? Ag[(long long)(r0 + t) * n + c] : zero;
+  }
+  cl.sync();                             // every CTA of the cluster runs before the first push
+  // complex64 columns of any magnitude: each is scaled by the power of two near
+  // its largest entry (exact, so every factor and every bit of Q stays what it
+  // is), or the product of two large columns would overflow; R is scaled back
+  float* s_scale = (float*)(smem_raw + L.bytes);
+  if constexpr (sizeof(R) == 4) {
+    if (scaled) {
+      for (int c = warp; c < n; c += nw) {
+        R a = 0;
+        for (int t = lane; t < mr; t += 32) {
+          const C x = A[(size_t)c * ld + t];
+          a = fmaxf(a, fmaxf(fabsf(x.x), fabsf(x.y)));
+        }
+        a = wmax(a);
+        if (lane == 0) s_scale[c] = a;
+      }
+      cl.sync();
+      unsigned mx[2] = {0, 0};           // (n < 2 x 512: 32 rows of n columns fit a CTA)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int c = threadIdx.x + u * kPanelThreads;
+        if (c < n)
+          for (int q = 0; q < cs; ++q) mx[u] = max(mx[u], __float_as_uint(cl.map_shared_rank(s_scale, q)[c]));
+      }
+      cl.sync();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {      // (columns that are zero or not finite stay as they are)
+        const int c = threadIdx.x + u * kPanelThreads;
+        if (c < n)
+          s_scale[c] = mx[u] == 0 || mx[u] >= 0x7f800000u ? 1.f : __uint_as_float(min(max(mx[u] >> 23, 1u), 253u) << 23);
+      }
+      __syncthreads();
+      for (int c = warp; c < n; c += nw) {
+        const float is = __uint_as_float((254u << 23) - __float_as_uint(s_scale[c]));
+        for (int t = lane; t < mr; t += 32) {
+          C x = A[(size_t)c * ld + t];
+          x.x *= is;
+          x.y *= is;
+          A[(size_t)c * ld + t] = x;
+        }
+      }
+      __syncthreads();
+    }
+  }
+
+  auto load_col = [&](int c, C (&v)[MAXR]) {
+    const C* p = A + (size_t)c * ld + lane;
+#pragma unroll
+    for (int i = 0; i < MAXR; ++i) v[i] = p[32 * i];
+  };
+  auto store_col = [&](int c, const C (&v)[MAXR]) {
+    C* p = A + (size_t)c * ld + lane;
+#pragma unroll
+    for (int i = 0; i < MAXR; ++i) p[32 * i] = v[i];
+  };
+  auto mask_below = [&](C (&x)[MAXR], int g0) {   // keep global rows > g0
+#pragma unroll
+    for (int i = 0; i < MAXR; ++i)
+      if (r0 + lane + 32 * i <= g0) x[i] = zero;
+  };
+  auto dot = [&](const C (&x)[MAXR], const C (&y)[MAXR]) {   // sum over the slice of conj(x) y
+    C acc = pmulc(x[0], y[0]);
+#pragma unroll
+    for (int i = 1; i < MAXR; ++i) acc = padd(acc, pmulc(x[i], y[i]));
+    acc.x = wsum(acc.x);
+    acc.y = wsum(acc.y);
+    return acc;
+  };
+  // (scale, sum of squares / scale^2) of the slice; complex128: (1, sum)
+  auto norm_part = [&](const C (&x)[MAXR]) {
+    if constexpr (sizeof(R) == 8) {
+      R s2 = 0;
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) s2 += x[i].x * x[i].x + x[i].y * x[i].y;
+      return mkc<C>(1, wsum(s2));
+    } else {
+      R amax = 0;
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) amax = fmaxf(amax, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
+      amax = wmax(amax);
+      if (amax == 0) return zero;
+      int ex;
+      frexpf(amax, &ex);                 // amax < 2^ex; 2^-ex in two in-range factors
+      const R s1 = ldexpf(1.f, -(ex / 2)), s2 = ldexpf(1.f, -(ex - ex / 2));
+      R ss = 0;
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) {
+        const R a = x[i].x * s1 * s2, b = x[i].y * s1 * s2;
+        ss += a * a + b * b;
+      }
+      return mkc<C>(ldexpf(1.f, ex), wsum(ss));
+    }
+  };
+  auto push_recv = [&](int par, int c, C d) {
+    if (lane < cs) st_dsmem(recv_q + (uint32_t)(sizeof(C) * ((size_t)(par * cs + cr) * n + c)), d);
+  };
+  auto push_norm = [&](int par, C np) {
+    if (lane < cs) st_dsmem(pp_q + (uint32_t)(sizeof(C) * (size_t)(par * cs + cr)), np);
+  };
+  // row g of column values y, from the CTA that holds it, into every CTA
+  auto push_row = [&](const C (&y)[MAXR], int g, int par, int c) {
+    const int t = g - r0;
+    if (t < 0 || t >= mr) return;        // uniform over the CTA
+    C val = pick(y, t >> 5);
+    val.x = __shfl_sync(0xffffffffu, val.x, t & 31);
+    val.y = __shfl_sync(0xffffffffu, val.y, t & 31);
+    if (lane < cs) st_dsmem(rowb_q + (uint32_t)(sizeof(C) * ((size_t)par * n + c)), val);
+  };
+  auto sum_recv = [&](int par, int c) {   // the cluster sum of column c, in source order
+    C s = zero;
+    for (int q = 0; q < cs; ++q) s = padd(s, recv[(size_t)(par * cs + q) * n + c]);
+    return s;
+  };
+
+  // ---- factorisation
+  if (k > 0) {                           // sums of step 0
+    C x[MAXR];
+    load_col(0, x);
+    if (warp == 0) push_row(x, 0, 0, 0);
+    mask_below(x, 0);
+    if (warp == 0) push_norm(0, norm_part(x));
+    for (int c = warp == 0 ? nw : warp; c < n; c += nw) {
+      C y[MAXR];
+      load_col(c, y);
+      push_recv(0, c, dot(x, y));
+      push_row(y, 0, 0, c);
+    }
+  }
+  cl.sync();
+  for (int j = 0; j < k; ++j) {
+    const int par = j & 1;
+    if (use_gs)
+      for (int c = j + 1 + threadIdx.x; c < n; c += blockDim.x) gs[c] = sum_recv(par, c);
+    if (threadIdx.x == blockDim.x - 1) {
+      // the reflector of step j from the norm of x and alpha = A[j][j]
+      R M = 0, S = 0;
+      for (int q = 0; q < cs; ++q) M = fmax(M, pp[par * cs + q].x);
+      if (M > 0) {
+        const R iM = (R)1 / M;           // (the scales are powers of two: exact)
+        for (int q = 0; q < cs; ++q) {
+          const C np = pp[par * cs + q];
+          const R rq = np.x * iM;
+          S += np.y * rq * rq;
+        }
+      }
+      const R xnorm = M * sqrt(S);
+      const C alpha = rowb[(size_t)par * n + j];
+      const R ar = alpha.x, ai = alpha.y;
+      R taur = 0, taui = 0, scr = 0, sci = 0, beta = ar;
+      if (!(xnorm == 0 && ai == 0)) {
+        // beta = -sign(ar) |(alpha, x)| from scaled terms; alpha - beta
+        // scaled by 1 / |beta| (|alpha - beta| >= |beta|), so that nothing
+        // overflows or underflows
+        const R mx = fmax(fmax(fabs(ar), fabs(ai)), xnorm), imx = (R)1 / mx;
+        const R u = ar * imx, w = ai * imx, z = xnorm * imx;
+        beta = -copysign(mx * sqrt(u * u + w * w + z * z), ar);
+        const R ib = (R)1 / beta, sb = fabs(ib);
+        const R dx = (ar - beta) * sb, dy = ai * sb, idd = sb / (dx * dx + dy * dy);
+        taur = (beta - ar) * ib;
+        taui = -ai * ib;
+        scr = dx * idd;
+        sci = -dy * idd;
+        // (the element type must hold sc too: columns near the bottom of its
+        // range leave the column as it is)
+        const R smax = sizeof(R) == 4 ? (R)1e37 : (R)1e300;
+        if (!(isfinite(taur) && isfinite(taui) && isfinite(scr) && isfinite(sci) && isfinite(beta)) ||
+            fabs(scr) > smax || fabs(sci) > smax || beta == (R)0) {
+          taur = taui = scr = sci = 0;
+          beta = ar;
+        }
+      }
+      const bool act = !(taur == 0 && taui == 0);
+      ring[par * 3 + 0] = mkc<C>(taur, taui);
+      ring[par * 3 + 1] = mkc<C>(scr, sci);
+      ring[par * 3 + 2] = mkc<C>(beta, act ? (R)0 : ai);
+      if (Qg) s_tau[j] = mkc<C>(taur, taui);
+    }
+    __syncthreads();
+    const C tj = ring[par * 3 + 0], sc = ring[par * 3 + 1], ctau = mkc<C>(tj.x, -tj.y);
+    const bool active = !(tj.x == 0 && tj.y == 0);
+    // scale the reflector of step j - 1 (no longer read)
+    if (j > 0 && warp == (j - 1) % nw) {
+      C x[MAXR];
+      load_col(j - 1, x);
+      const C scp = ring[(par ^ 1) * 3 + 1], dg = ring[(par ^ 1) * 3 + 2];
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) {
+        const int g = r0 + lane + 32 * i;
+        if (g > j - 1) x[i] = pmul(x[i], scp);
+        else if (g == j - 1) x[i] = dg;
+      }
+      store_col(j - 1, x);
+    }
+    C v[MAXR];                           // v of step j: x sc below row j, 1 at row j
+    load_col(j, v);
+#pragma unroll
+    for (int i = 0; i < MAXR; ++i) {
+      const int g = r0 + lane + 32 * i;
+      v[i] = g > j ? pmul(v[i], sc) : (g == j ? one : zero);
+    }
+    auto fac = [&](int c) {
+      const C s = use_gs ? gs[c] : sum_recv(par, c);
+      return active ? pmul(ctau, padd(rowb[(size_t)par * n + c], pmulc(sc, s))) : zero;
+    };
+    const bool own = j + 1 < n && warp == (j + 1) % nw;
+    C xm[MAXR];                          // column j + 1 after step j, then its rows > j + 1
+    C keep_j = zero, keep_j1 = zero;     // (owner) its rows j and j + 1, in the lanes that hold them
+    if (j + 1 < n) {
+      load_col(j + 1, xm);
+      const C f1 = fac(j + 1);
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) xm[i] = psub(xm[i], pmul(v[i], f1));
+      if (own) {
+#pragma unroll
+        for (int i = 0; i < MAXR; ++i) {
+          const int g = r0 + lane + 32 * i;
+          if (g == j) keep_j = xm[i];
+          if (g == j + 1) keep_j1 = xm[i];
+        }
+        if (j + 1 < k) push_row(xm, j + 1, par ^ 1, j + 1);
+      }
+      mask_below(xm, j + 1);
+      if (own && j + 1 < k) push_norm(par ^ 1, norm_part(xm));
+      int c = j + 2 + ((warp - (j + 2)) % nw + nw) % nw;
+      if constexpr ((sizeof(R) == 4 && MAXR <= 6) || (sizeof(R) == 8 && MAXR <= 2)) {
+        // two columns at a time (two independent chains, one reduction
+        // tree for both dots: lanes 0-7 end with the first real part, 8-15
+        // its imaginary part, 16-31 the second column's)
+        for (; c + nw < n; c += 2 * nw) {
+          const int c2 = c + nw;
+          C y[MAXR], y2[MAXR];
+          load_col(c, y);
+          load_col(c2, y2);
+          const C f = fac(c), f2 = fac(c2);
+#pragma unroll
+          for (int i = 0; i < MAXR; ++i) {
+            y[i] = psub(y[i], pmul(v[i], f));
+            y2[i] = psub(y2[i], pmul(v[i], f2));
+          }
+          store_col(c, y);
+          store_col(c2, y2);
+          if (j + 1 < k) {
+            C d = pmulc(xm[0], y[0]), d2 = pmulc(xm[0], y2[0]);
+#pragma unroll
+            for (int i = 1; i < MAXR; ++i) {
+              d = padd(d, pmulc(xm[i], y[i]));
+              d2 = padd(d2, pmulc(xm[i], y2[i]));
+            }
+            const bool h4 = lane & 16, h3 = lane & 8;
+            R a0 = h4 ? d2.x : d.x, a1 = h4 ? d2.y : d.y;     // kept halves
+            a0 += __shfl_xor_sync(0xffffffffu, h4 ? d.x : d2.x, 16);
+            a1 += __shfl_xor_sync(0xffffffffu, h4 ? d.y : d2.y, 16);
+            R b = (h3 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h3 ? a0 : a1, 8);
+            b += __shfl_xor_sync(0xffffffffu, b, 4);
+            b += __shfl_xor_sync(0xffffffffu, b, 2);
+            b += __shfl_xor_sync(0xffffffffu, b, 1);
+            const C s1 = mkc<C>(__shfl_sync(0xffffffffu, b, 0), __shfl_sync(0xffffffffu, b, 8));
+            const C s2 = mkc<C>(__shfl_sync(0xffffffffu, b, 16), __shfl_sync(0xffffffffu, b, 24));
+            push_recv(par ^ 1, c, s1);
+            push_recv(par ^ 1, c2, s2);
+            push_row(y, j + 1, par ^ 1, c);
+            push_row(y2, j + 1, par ^ 1, c2);
+          }
+        }
+      }
+      for (; c < n; c += nw) {
+        C y[MAXR];
+        load_col(c, y);
+        const C f = fac(c);
+#pragma unroll
+        for (int i = 0; i < MAXR; ++i) y[i] = psub(y[i], pmul(v[i], f));
+        store_col(c, y);
+        if (j + 1 < k) {
+          push_recv(par ^ 1, c, dot(xm, y));
+          push_row(y, j + 1, par ^ 1, c);
+        }
+      }
+    }
+    cl.sync();
+    if (own) {                           // column j + 1, rows >= j (rows above are unchanged)
+      C* p = A + (size_t)(j + 1) * ld + lane;
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) {
+        const int g = r0 + lane + 32 * i;
+        if (g > j + 1) p[32 * i] = xm[i];
+        else if (g == j + 1) p[32 * i] = keep_j1;
+        else if (g == j) p[32 * i] = keep_j;
+      }
+    }
+  }
+  if (k > 0 && warp == (k - 1) % nw) {   // scale the last reflector
+    C x[MAXR];
+    load_col(k - 1, x);
+    const C scp = ring[((k - 1) & 1) * 3 + 1], dg = ring[((k - 1) & 1) * 3 + 2];
+#pragma unroll
+    for (int i = 0; i < MAXR; ++i) {
+      const int g = r0 + lane + 32 * i;
+      if (g > k - 1) x[i] = pmul(x[i], scp);
+      else if (g == k - 1) x[i] = dg;
+    }
+    store_col(k - 1, x);
+  }
+  __syncthreads();
+
+  // R (k x n, upper triangular) from the rows this CTA holds
+  if (Rg)
+    for (int e = threadIdx.x; e < mr * n; e += blockDim.x) {
+      const int t = e / n, c = e % n, g = r0 + t;
+      C x = (c >= g) ? A[(size_t)c * ld + t] : zero;
+      if constexpr (sizeof(R) == 4)
+        if (scaled) x = mkc<C>(x.x * s_scale[c], x.y * s_scale[c]);
+      if (g < k) Rg[(long long)g * n + c] = x;
+    }
+  if (!Qg) return;     // nothing is pushed after the last cluster barrier above
+
+  // ---- Q = H_0 ... H_{k-1} [I; 0] by blocks of NB reflectors, the last
+  // block first, in place: H_{b0} ... H_{b1-1} = I - V T V^H (compact WY;
+  // T upper triangular, T_jj = tau_j, T_{0:j,j} = -tau_j T_{0:j,0:j}
+  // (V^H V)_{0:j,j}), so with Q' the columns >= b1 built so far and e_c the
+  // block's own columns,  Q_{:,c} = Q'_{:,c} - V (T (V^H Q'_{:,c})).
+  // One cluster exchange per block: every CTA writes its partial V^H Q'
+  // and V^H V over its rows into its own shared memory, and after the
+  // barrier every CTA sums all CTAs' partials remotely in rank order (the
+  // same T and the same products in every CTA).
+  constexpr int NB = kQBlock;
+  const int W = k + NB;                  // a row of the block buffers: V^H Q' at c < k, V^H V at k + b
+  C* Pb = A + L.recv;                    // [2][NB][W]: own partials, by block parity
+  C* Sb = Pb + 2 * (size_t)NB * W;       // [NB][W]: cluster sums, then T V^H Q'
+  C* Tb = Sb + (size_t)NB * W;           // [NB][NB]
+  constexpr int rows_pad = 32 * MAXR;
+  const int ngroups = max(1, (int)blockDim.x / rows_pad);
+  // V_B[t][a] of the block starting at column b0: reflector b0 + a at local row t
+  auto vb = [&](int b0, int a, int t) {
+    const int col = b0 + a, g = r0 + t;
+    return g > col ? A[(size_t)col * ld + t] : (g == col ? one : zero);
+  };
+  const int nblk = (k + NB - 1) / NB;
+  for (int B = nblk - 1; B >= 0; --B) {
+    const int b0 = B * NB, b1 = min(k, b0 + NB), nbB = b1 - b0;
+    C* Pw = Pb + (size_t)(B & 1) * NB * W;
+    // partials V^H Q' (columns c >= b1): a warp per column, the block's
+    // reflectors four at a time in registers
+    for (int a0 = 0; a0 < nbB; a0 += 4) {
+      C vch[4][MAXR];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int i = 0; i < MAXR; ++i) vch[u][i] = a0 + u < nbB ? vb(b0, a0 + u, lane + 32 * i) : zero;
+      for (int c = b1 + ((warp - b1) % nw + nw) % nw; c < k; c += nw) {
+        C y[MAXR];
+        load_col(c, y);
+        R acc[8];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          C d = pmulc(vch[u][0], y[0]);
+#pragma unroll
+          for (int i = 1; i < MAXR; ++i) d = padd(d, pmulc(vch[u][i], y[i]));
+          acc[2 * u] = d.x;
+          acc[2 * u + 1] = d.y;
+        }
+        // eight sums over the warp, halving the set at every level: lane l
+        // ends with sum r = 4 b4 + 2 b3 + b2 of its lane bits
+        const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const R send = h4 ? acc[q] : acc[4 + q];
+          acc[q] = (h4 ? acc[4 + q] : acc[q]) + __shfl_xor_sync(0xffffffffu, send, 16);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const R send = h3 ? acc[q] : acc[2 + q];
+          acc[q] = (h3 ? acc[2 + q] : acc[q]) + __shfl_xor_sync(0xffffffffu, send, 8);
+        }
+        {
+          const R send = h2 ? acc[0] : acc[1];
+          acc[0] = (h2 ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, send, 4);
+        }
+        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+        if ((lane & 3) == 0) {
+          const int r = (h4 ? 4 : 0) + (h3 ? 2 : 0) + (h2 ? 1 : 0), u = r >> 1;
+          if (a0 + u < nbB) ((R*)&Pw[(size_t)(a0 + u) * W + c])[r & 1] = acc[0];
+        }
+      }
+    }
+    // the block's own columns e_c (c in [b0, b1)): conj(V_B[c][a]) from the
+    // CTA that holds row c, zero elsewhere
+    for (int e = threadIdx.x; e < nbB * nbB; e += blockDim.x) {
+      const int a = e / nbB, c = b0 + e % nbB, t = c - r0;
+      const C v = (t >= 0 && t < mr) ? vb(b0, a, t) : zero;
+      Pw[(size_t)a * W + c] = mkc<C>(v.x, -v.y);
+    }
+    // V^H V (a < b) over the slice: a warp per pair
+    for (int pr = warp; pr < nbB * nbB; pr += nw) {
+      const int a = pr / nbB, b = pr % nbB;
+      if (a >= b) continue;
+      C x[MAXR], y[MAXR];
+#pragma unroll
+      for (int i = 0; i < MAXR; ++i) {
+        x[i] = vb(b0, a, lane + 32 * i);
+        y[i] = vb(b0, b, lane + 32 * i);
+      }
+      const C d = dot(x, y);
+      if (lane == 0) Pw[(size_t)a * W + k + b] = d;
+    }
+    cl.sync();
+    // cluster sums of the block's partials, read from every CTA in rank order
+    for (int e = threadIdx.x; e < nbB * W; e += blockDim.x) {
+      const int a = e / W, col = e % W;
+      if (col < b0 || (col >= k && (col - k <= a || col - k >= nbB))) continue;
+      C sum = zero;
+      for (int q0 = 0; q0 < cs; q0 += 8) {
+        C vq[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) vq[u] = q0 + u < cs ? cl.map_shared_rank(Pw, q0 + u)[e] : zero;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) sum = padd(sum, vq[u]);
+      }
+      Sb[e] = sum;
+    }
+    __syncthreads();
+    if (warp == 0) {                     // T of the block, lane a holds row a
+      const int a = lane;
+      if (a < NB)
+        for (int b = 0; b < NB; ++b) Tb[a * NB + b] = (a == b && a < nbB) ? s_tau[b0 + a] : zero;
+      __syncwarp();
+      for (int j = 1; j < nbB; ++j) {
+        if (a < j) {
+          C acc = zero;
+          for (int b = a; b < j; ++b) acc = padd(acc, pmul(Tb[a * NB + b], Sb[(size_t)b * W + k + j]));
+          const C tj = s_tau[b0 + j];
+          Tb[a * NB + j] = mkc<C>(-(tj.x * acc.x - tj.y * acc.y), -(tj.x * acc.y + tj.y * acc.x));
+        }
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    for (int c = b0 + threadIdx.x; c < k; c += blockDim.x)   // T V^H Q' in place, rows in ascending order
+      for (int a = 0; a < nbB; ++a) {
+        C acc = zero;
+        for (int b = a; b < nbB; ++b) acc = padd(acc, pmul(Tb[a * NB + b], Sb[(size_t)b * W + c]));
+        Sb[(size_t)a * W + c] = acc;
+      }
+    // every thread takes its row's V_B before the block's columns change
+    const int t = threadIdx.x % rows_pad, grp = threadIdx.x / rows_pad;
+    C v[NB];
+#pragma unroll
+    for (int a = 0; a < NB; ++a) v[a] = a < nbB ? vb(b0, a, t) : zero;
+    __syncthreads();
+    if (grp < ngroups) {
+      const int g = r0 + t;
+      for (int c = b0 + grp; c < k; c += ngroups) {
+        C q = c >= b1 ? A[(size_t)c * ld + t] : (g == c ? one : zero);
+#pragma unroll
+        for (int a = 0; a < NB; ++a)
+          if (a < nbB) q = psub(q, pmul(v[a], Sb[(size_t)a * W + c]));
+        A[(size_t)c * ld + t] = q;
+      }
+    }
+    __syncthreads();
+  }
+  cl.sync();                             // no CTA still reads this CTA's partials
+  for (int e = threadIdx.x; e < mr * k; e += blockDim.x) {
+    const int t = e / k, c = e % k;
+    Qg[(long long)(r0 + t) * k + c] = A[(size_t)c * ld + t];
+  }
 }
 
 // sum of slot[off] over the cluster's CTAs in rank order (the same grouping
@@ -438,6 +1010,21 @@ constexpr int kMaxrF[] = {1, 2, 3, 4, 5, 6, 8};   // complex64
 constexpr int kMaxrD[] = {1, 2, 3, 4};            // complex128 (twice the registers per entry)
 
 template <typename C, int MAXR>
+cudaError_t panel_optin_one() {
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(k_panel_qr<C, MAXR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPanelSmemMax);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_panel_qr<C, MAXR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) done.fetch_or(bit);
+  return e;
+}
+
+template <typename C, int MAXR>
 cudaError_t panel_optin_pull() {
   static std::atomic<unsigned long long> done{0};
   int dev = 0;
@@ -457,26 +1044,49 @@ cudaError_t panel_optin() {
   cudaError_t e;
   if ((e = panel_optin_pull<C, 2>()) != cudaSuccess) return e;
   if ((e = panel_optin_pull<C, 4>()) != cudaSuccess) return e;
-  if constexpr (sizeof(C) == sizeof(float2)) return panel_optin_pull<C, 8>();
+  if constexpr (sizeof(C) == sizeof(float2))
+    if ((e = panel_optin_pull<C, 8>()) != cudaSuccess) return e;
+  if ((e = panel_optin_one<C, 1>()) != cudaSuccess) return e;
+  if ((e = panel_optin_one<C, 2>()) != cudaSuccess) return e;
+  if ((e = panel_optin_one<C, 3>()) != cudaSuccess) return e;
+  if ((e = panel_optin_one<C, 4>()) != cudaSuccess) return e;
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    if ((e = panel_optin_one<C, 5>()) != cudaSuccess) return e;
+    if ((e = panel_optin_one<C, 6>()) != cudaSuccess) return e;
+    return panel_optin_one<C, 8>();
+  }
   return cudaSuccess;
 }
 
 struct PanelPlan {
+  bool pull = false;
   int maxr = 0, cs = 0, ld = 0, rows = 0;
+  bool gs = true;
   size_t bytes = 0;
 };
 
-// whether the slice of 32 maxr rows fits: odd column stride with staged
-// sums, even stride, then sums taken in place
+// the first layout that fits: odd column stride (no bank conflicts in the
+// row-major copies) with staged sums, even stride, then sums taken in place
 template <typename C>
-bool panel_fit(int n, int maxr, int cs, bool want_q) {
-  for (int v = 0; v < 3; ++v)
-    if (panel_layout<C>(maxr, n, cs, want_q, v == 0, v < 2).bytes <= (size_t)kPanelSmemMax) return true;
+bool panel_fit(int n, int maxr, int cs, bool want_q, PanelPlan& p) {
+  for (int v = 0; v < 3; ++v) {
+    const PanelLayout L = panel_layout<C>(maxr, n, cs, want_q, v == 0, v < 2);
+    if (L.bytes <= (size_t)kPanelSmemMax) {
+      p.pull = false;
+      p.maxr = maxr;
+      p.cs = cs;
+      p.ld = L.ld;
+      p.rows = 32 * maxr;
+      p.gs = v < 2;
+      p.bytes = L.bytes;
+      return true;
+    }
+  }
   return false;
 }
 
-// the column-by-column form: rows = ceil(m / cs) a CTA, at most 256
-// (complex64) or 128 (complex128)
+// the pulled form: rows = ceil(m / cs) a CTA, at most 256 (complex64) or
+// 128 (complex128)
 template <typename C>
 bool panel_fit_pull(int m, int n, int cs, PanelPlan& p) {
   const int rows = (m + cs - 1) / cs;
@@ -484,6 +1094,7 @@ bool panel_fit_pull(int m, int n, int cs, PanelPlan& p) {
   if (rows > max_rows) return false;
   const size_t b = panel_smem_pull<C>(rows, n);
   if (b > (size_t)kPanelSmemMax) return false;
+  p.pull = true;
   p.maxr = rows <= 64 ? 2 : (rows <= 128 ? 4 : 8);
   p.cs = cs;
   p.rows = rows;
@@ -503,13 +1114,36 @@ void maxr_list(const int*& list, int& nl) {
   }
 }
 
-// The column-by-column launch of an m x n panel: a given cluster, or the
-// fewest CTAs that fit, raised to about 256 (complex64) or 64 (complex128)
-// rows a CTA.
+// Launch plan of an m x n panel.  A given cluster size takes the fewest rows
+// per CTA that cover m; otherwise the fewest rows per CTA whose cluster has
+// at most 9 CTAs (complex64: two such clusters share one GPC's SMs, so
+// concurrent panels of different streams still place; the complex128 kernel
+// is bound by the FP64 rate of its SMs and spreads over up to 16), else up
+// to 16 CTAs.  Panels whose push buffers do not fit take the pulled form.
 template <typename C>
-bool panel_plan_pull(int m, int n, int cluster, PanelPlan& p) {
+bool panel_plan(int m, int n, bool want_q, int cluster, PanelPlan& p) {
   if (m < n || n < 1) return false;
-  if (cluster > 0) return cluster <= kPanelMaxCluster && panel_fit_pull<C>(m, n, cluster, p);
+  const int* list;
+  int nl;
+  maxr_list<C>(list, nl);
+  if (cluster > 0) {
+    if (cluster > kPanelMaxCluster) return false;
+    const int need = ((m + cluster - 1) / cluster + 31) / 32;
+    for (int a = 0; a < nl; ++a)
+      if (list[a] >= need) {
+        if (panel_fit<C>(n, list[a], cluster, want_q, p)) return true;
+        break;
+      }
+    return panel_fit_pull<C>(m, n, cluster, p);
+  }
+  const int pref = sizeof(C) == sizeof(float2) ? 9 : kPanelMaxCluster;
+  for (int lim : {pref, kPanelMaxCluster})
+    for (int a = 0; a < nl; ++a) {
+      const int cs = (m + 32 * list[a] - 1) / (32 * list[a]);
+      if (cs <= lim && panel_fit<C>(n, list[a], cs, want_q, p)) return true;
+    }
+  // pulled: the fewest CTAs that fit, raised to about 256 (complex64) or
+  // 64 (complex128) rows a CTA
   for (int cs = 1; cs <= kPanelMaxCluster; ++cs)
     if (panel_fit_pull<C>(m, n, cs, p)) {
       const int target = sizeof(C) == sizeof(float2) ? 256 : 64;
@@ -529,7 +1163,7 @@ int panel_min_cluster(int m, int n, bool want_q) {
   PanelPlan p;
   for (int a = nl - 1; a >= 0; --a) {
     const int cs = (m + 32 * list[a] - 1) / (32 * list[a]);
-    if (cs <= kPanelMaxCluster && panel_fit<C>(n, list[a], cs, want_q) && (best == 0 || cs < best)) best = cs;
+    if (cs <= kPanelMaxCluster && panel_fit<C>(n, list[a], cs, want_q, p) && (best == 0 || cs < best)) best = cs;
   }
   for (int cs = 1; cs <= kPanelMaxCluster && (best == 0 || cs < best); ++cs)
     if (panel_fit_pull<C>(m, n, cs, p)) {
@@ -543,8 +1177,8 @@ int panel_min_cluster(int m, int n, bool want_q) {
 
 cudaError_t init_panel_attributes() {
   cudaError_t e = panel_optin<float2>();
-  if (e == cudaSuccess) e = panel_optin<double2>();
-  return e == cudaSuccess ? init_bqr_attributes() : e;
+  if (e != cudaSuccess) return e;
+  return panel_optin<double2>();
 }
 
 int panel_cluster(int m, int n, size_t elem, bool want_q) {
@@ -553,17 +1187,13 @@ int panel_cluster(int m, int n, size_t elem, bool want_q) {
 
 template <typename C>
 static cudaError_t panel_t(const C* A, int m, int n, C* Q, C* R, int batch, long long stride, cudaStream_t s,
-                           int cluster) {
+                           int cluster, bool any_range = false) {
   if (batch < 1 || m < 1 || n < 1) return cudaSuccess;
-  if (m < n) return cudaErrorInvalidValue;
-  const bool want_q = Q != nullptr;
-  KTimerScope timer(KC_ORTH, s, batch * qr_flops(m, n));
-  if (bqr_fits(m, n, sizeof(C), want_q, cluster))
-    return launch_bqr(A, batch * m, n, m, stride, Q, R, cluster, s);
   PanelPlan p;
-  if (!panel_plan_pull<C>(m, n, cluster, p)) return cudaErrorInvalidValue;
+  if (!panel_plan<C>(m, n, Q != nullptr, cluster, p)) return cudaErrorInvalidValue;
   cudaError_t e = panel_optin<C>();
   if (e != cudaSuccess) return e;
+  KTimerScope timer(KC_ORTH, s, batch * qr_flops(m, n));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.cs * batch, 1, 1);
   cfg.blockDim = dim3(kPanelThreads, 1, 1);
@@ -576,10 +1206,32 @@ static cudaError_t panel_t(const C* A, int m, int n, C* Q, C* R, int batch, long
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (p.maxr == 2) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 2>, A, m, n, p.rows, Q, R, stride);
-  if (p.maxr == 4) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 4>, A, m, n, p.rows, Q, R, stride);
-  if constexpr (sizeof(C) == sizeof(float2))
-    if (p.maxr == 8) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 8>, A, m, n, p.rows, Q, R, stride);
+  if (p.pull) {
+    if (p.maxr == 2) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 2>, A, m, n, p.rows, Q, R, stride);
+    if (p.maxr == 4) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 4>, A, m, n, p.rows, Q, R, stride);
+    if constexpr (sizeof(C) == sizeof(float2))
+      if (p.maxr == 8) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 8>, A, m, n, p.rows, Q, R, stride);
+    return cudaErrorInvalidValue;
+  }
+  const int gsf = p.gs ? 1 : 0;
+  // (a panel that fills the shared memory has no room for the columns' scales)
+  const int scaled = any_range && sizeof(C) == sizeof(float2) && p.bytes + sizeof(float) * n <= (size_t)kPanelSmemMax;
+  if (scaled) cfg.dynamicSmemBytes += sizeof(float) * n;
+  switch (p.maxr) {
+    case 1: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 1>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+    case 2: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 2>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+    case 3: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 3>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+    case 4: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 4>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+    default: break;
+  }
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    switch (p.maxr) {
+      case 5: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 5>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+      case 6: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 6>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+      case 8: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 8>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+      default: break;
+    }
+  }
   return cudaErrorInvalidValue;
 }
 
@@ -642,12 +1294,12 @@ cudaError_t launch_panel_qr_chunked(const double2* A, int m, int n, double2* Q, 
 }
 
 cudaError_t launch_panel_qr(const float2* A, int m, int n, float2* Q, float2* R, int batch, long long stride,
-                            cudaStream_t s, int cluster) {
-  return panel_t(A, m, n, Q, R, batch, stride, s, cluster);
+                            cudaStream_t s, int cluster, bool any_range) {
+  return panel_t(A, m, n, Q, R, batch, stride, s, cluster, any_range);
 }
 cudaError_t launch_panel_qr(const double2* A, int m, int n, double2* Q, double2* R, int batch, long long stride,
-                            cudaStream_t s, int cluster) {
-  return panel_t(A, m, n, Q, R, batch, stride, s, cluster);
+                            cudaStream_t s, int cluster, bool any_range) {
+  return panel_t(A, m, n, Q, R, batch, stride, s, cluster, any_range);
 }
 
 }  // namespace bbp

@@ -250,31 +250,18 @@ inline double qr_flops(int m, int n) {
 // panel_cluster: the fewest CTAs whose shared memory holds an m x n panel of
 // elem-byte entries (with the reflector scalars Q needs when want_q; 0 when
 // even 16 do not).  cluster = 0 picks it; a given size must be at least
-// panel_cluster(m, n, elem) and at most kPanelMaxCluster.
+// panel_cluster(m, n, elem) and at most kPanelMaxCluster.  any_range: columns
+// of any magnitude of complex64 (else only what the squares of entries near
+// one and the products of two columns reach).
 constexpr int kPanelMaxCluster = 16;
 int panel_cluster(int m, int n, size_t elem, bool want_q = true);
 cudaError_t init_panel_attributes();
 cudaError_t launch_panel_qr(const float2* A, int m, int n, float2* Q, float2* R, int batch, long long stride,
-                            cudaStream_t s, int cluster = 0);
+                            cudaStream_t s, int cluster = 0, bool any_range = false);
 cudaError_t launch_panel_qr(const double2* A, int m, int n, double2* Q, double2* R, int batch, long long stride,
-                            cudaStream_t s, int cluster = 0);
-// The blocked factorisation behind it (k_qr.cu), for any shape: row blocks of
-// rb rows of A (m_all x n, the last one shorter), each k x n with k = min(rows,
-// n): Q (k columns a block, may alias A, may be null) at `stride` elements a
-// block, R k x n, or, of more than one block, n x n each with zero rows below
-// k.  bqr_fits: whether one block fits (cluster CTAs, 0: any number).
-bool bqr_fits(int m, int n, size_t elem, bool want_q, int cluster = 0);
-cudaError_t init_bqr_attributes();
-cudaError_t launch_bqr(const float2* A, int m_all, int n, int rb, long long stride, float2* Q, float2* R, int cluster,
-                       cudaStream_t s);
-cudaError_t launch_bqr(const double2* A, int m_all, int n, int rb, long long stride, double2* Q, double2* R,
-                       int cluster, cudaStream_t s);
-// T (n x m, row-major) = R^H Q^H from the QR of its conjugate transpose, T^H =
-// Q R: T is overwritten by Q^H (k x m), R is k x n, k = min(m, n).  qr_in_place:
-// whether launch_bqr and launch_blq take an m x n factorisation with Q over
-// its input (else launch_qr with separate buffers).
-cudaError_t launch_blq(float2* T, int n, int m, float2* R, cudaStream_t s);
-cudaError_t launch_blq(double2* T, int n, int m, double2* R, cudaStream_t s);
+                            cudaStream_t s, int cluster = 0, bool any_range = false);
+// Whether launch_qr takes an m x n matrix of elem-byte entries with Q over its
+// input (it is held in shared memory as a whole).
 bool qr_in_place(int m, int n, size_t elem);
 // Panels taller than one cluster holds (panel_cluster = 0): two-level TSQR
 // over row chunks that each fit one cluster; Q is required, R may be null.
