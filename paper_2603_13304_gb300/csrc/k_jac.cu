@@ -6,31 +6,42 @@
 // the same rotations accumulating in WH (M x M, from the identity): WH G_0 =
 // G.  A row of G and its row of WH are one vector of N + M entries.
 //
-// Distribution: 2 C blocks of bs rows on C CTAs, two a CTA ("top", "bottom").
-// A step rotates every pair (top i, bottom j): bs rounds of bs disjoint pairs,
-// a warp a pair, top row i staying in warp i's registers over the rounds.
-// Then the blocks move one place round the tournament (Brent and Luk's
-// ordering of blocks), pushed into the neighbours' shared memory; after 2 C -
-// 1 steps every two blocks have met and each is back home.  The pairs within
-// a block are rotated when a sweep begins.  A block is pushed into one of
-// three buffers in turn, completing on the receiver's mbarrier: a neighbour
-// pushes at the end of step s into the buffer whose last contents left at the
-// end of step s - 2, which its own push at the end of step s - 1 proves, so
-// no other handshake is needed.
+// Order and arithmetic are part of the results.  The phases of the singular
+// vectors follow from the order of the rotations and from every rounding, and
+// the randomised truncations sketch in the basis that these phases give: where
+// a spectrum is flat, another order moves a network's messages by 1e-5 in full
+// precision.  So the pairs go round a circle tournament (round r: row M' - 1
+// against row r, row r + q against row r - q, mod M' - 1, M' = M rounded up to
+// even), the four sums of a pair are taken lane by lane (32 or 16 lanes) with
+// one addition tree, and every product and sum is rounded as written here (fma
+// calls, and products that no addition can take up).  JacOrder names the three
+// forms that results so far were computed in; k_jacobi (device memory) rotates
+// as kJacPlain32.
 //
-// A rotation is given by tau = t e^{i phi} (t = tan theta), x' = c (x - tau
-// y), y' = c (y + conj(tau) x).  Any tau gives a unitary step once c = 1 /
-// sqrt(1 + |tau|^2) holds to working precision, so tau itself is formed in
-// float from the float images of the sums in both types (an error d of the
-// angle leaves d times the pair's inner product, which the next sweep takes);
-// c, sigma = c tau and the squared norms (al' = al - t |g|, be' = be + t |g|,
-// taken anew when they cancel and in every sweep) are in the element's type.
+// Distribution: the P = M' / 2 pairs of a round lie on C CTAs, pp places each,
+// a warp a place, both rows in shared memory.  From round to round the first
+// rows of the places move one place left and the second rows one place right
+// (turning at the ends; row M' - 1 stays): inside a CTA the rows stay where
+// they are and the places' slots move round two rings of pp + 2 slots; at its
+// ends a warp pushes the row that leaves into the neighbour's next slot,
+// completing on that CTA's mbarrier, and waits for the one that comes.  A
+// neighbour pushes at the end of round r into the slot whose row left at the
+// end of round r - 2: it has had this CTA's push of round r - 1, which came
+// after the block barrier of round r - 2.  One barrier a direction and round
+// parity: a push of round r + 2 needs this CTA's push of round r + 1, made by
+// the same warp after its wait for round r.
 //
-// What bounds it: complex128, the FP64 pipe (a warp-wide multiply-add takes
-// 64 clocks of its sub-partition): 4 for the inner product and 12 for the
-// rotation per 32 entries, about 20 a pair besides, so four pairs a CTA, one
-// per sub-partition, and as many CTAs as that gives; complex64, the chain of
-// one reduction and the scalars per round (about 600 clocks).
+// What bounds it.  complex128: the FP64 unit (a warp-wide instruction 64
+// clocks, one every 19 clocks an SM), so the square roots and the quotients of
+// a pair are taken side by side in lanes of one instruction and the sums share
+// their addition tree (6 additions for 20), two pairs a CTA: 128 instructions
+// a pair, half of them scalars.  complex64: the chain of one reduction and
+// five roots and quotients a round, eight pairs a CTA.  Measured, us, one CTA
+// with all rows (a warp or half a warp a pair, every lane its own scalars) and
+// here: complex128 8 x 8 261 and 178, 31 x 40 6170 and 1430, 64 x 64 28400 and
+// 3470 (graded rows 62600 and 8090); complex64 31 x 40 315 and 280, 64 x 64
+// 1030 and 757, 96 x 90 1737 and 1190; from device memory and here: complex128
+// 128 x 128 45600 and 11250.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -48,6 +59,7 @@ namespace {
 
 constexpr int kJacMaxCluster = 16;
 constexpr size_t kJacSmemMax = 227 * 1024;
+constexpr size_t kJacStaged = 211 * 1024;   // rows that one CTA's shared memory held: the staged orders
 
 template <typename C> struct RealJ;
 template <> struct RealJ<double2> { using T = double; };
@@ -59,60 +71,6 @@ template <typename C> __device__ __forceinline__ C mkj(typename RealJ<C>::T re, 
   return r;
 }
 
-// float image of x (about six digits in double, by its high word: no FP64
-// conversion), and the exact double of a float
-__device__ __forceinline__ float image(float x) { return x; }
-__device__ __forceinline__ float image(double x) {
-  const int hi = __double2hiint(x);
-  const int e = ((hi >> 20) & 0x7ff) - 1023 + 127;
-  if (e <= 0) return 0.f;
-  if (e >= 255) return __int_as_float((hi & 0x80000000) | 0x7f800000);
-  return __int_as_float((hi & 0x80000000) | (e << 23) | ((hi & 0xfffff) << 3));
-}
-__device__ __forceinline__ void widen(float x, float& r) { r = x; }
-__device__ __forceinline__ void widen(float x, double& r) {
-  const int b = __float_as_int(x);
-  const int e = (b >> 23) & 0xff;
-  r = e == 0 ? 0.0
-             : __hiloint2double((b & 0x80000000) | ((e - 127 + 1023) << 20) | ((b & 0x7fffff) >> 3), (b & 7) << 29);
-}
-// x 2^-e and the exponent e of the larger of two magnitudes (double: so that
-// the images are in float's range)
-__device__ __forceinline__ int top_exponent(double a, double b) {
-  return max((__double2hiint(a) >> 20) & 0x7ff, (__double2hiint(b) >> 20) & 0x7ff) - 1023;
-}
-__device__ __forceinline__ float image_scaled(double x, int e) {   // image of x 2^-e
-  const int hi = __double2hiint(x), ex = ((hi >> 20) & 0x7ff) - 1023 + 127 - e;
-  if (((hi >> 20) & 0x7ff) == 0 || ex <= 0) return 0.f;
-  if (ex >= 255) return __int_as_float((hi & 0x80000000) | 0x7f7fffff);
-  return __int_as_float((hi & 0x80000000) | (ex << 23) | ((hi & 0xfffff) << 3));
-}
-__device__ __forceinline__ int top_exponent(float, float) { return 0; }
-__device__ __forceinline__ float image_scaled(float x, int) { return x; }
-
-// 1 / sqrt(q), q in [1, 2]: a float seed and Newton (float) or one cubically
-// convergent Householder step (double)
-__device__ __forceinline__ float inv_root(float q) {
-  const float y = rsqrtf(q);
-  return fmaf(0.5f * y, fmaf(-q * y, y, 1.f), y);
-}
-__device__ __forceinline__ double inv_root(double q) {
-  double y;
-  widen(rsqrtf(image(q)), y);
-  const double e = fma(-q * y, y, 1.0);          // (six digits in: one step leaves 1e-18)
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-// two sums over the warp, both in every lane
-template <typename R>
-__device__ __forceinline__ void sum2(R& a, R& b, int lane) {
-  const bool up = lane & 16;
-  R v = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
-#pragma unroll
-  for (int o = 8; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  a = __shfl_sync(0xffffffffu, v, 0);
-  b = __shfl_sync(0xffffffffu, v, 16);
-}
 template <typename R>
 __device__ __forceinline__ R sum1(R v) {
 #pragma unroll
@@ -120,16 +78,94 @@ __device__ __forceinline__ R sum1(R v) {
   return v;
 }
 
+// Lanes of a pair's sums, and which product of e y is rounded by itself.
+enum JacOrder { kJacPlain32 = 0, kJacStaged32 = 1, kJacStaged16 = 2 };
+
+// Rotates rows x and y (N entries of G, len = N + M with those of WH) so that
+// their G parts become orthogonal; returns 1 when a rotation was applied.  A
+// warp; every lane takes the same decision.
+template <typename C, int ORD>
+__device__ __forceinline__ int rotate_rows(C* __restrict__ xr, C* __restrict__ yr, int N, int len, int lane,
+                                           typename RealJ<C>::T tol, typename RealJ<C>::T floor) {
+  using R = typename RealJ<C>::T;
+  const unsigned all = 0xffffffffu;
+  const bool up = lane & 16, odd = lane & 8;
+  R p0 = 0, p1 = 0;                      // lower lanes: |x|^2, Re x conj(y); upper: |y|^2, Im x conj(y)
+  if constexpr (ORD == kJacStaged16) {
+#pragma unroll 4
+    for (int c = lane & 15; c < N; c += 16) {
+      const C x = xr[c], y = yr[c];
+      const C u = up ? y : x;
+      const R a = up ? x.y : x.x, b = up ? -x.x : x.y;
+      p0 += fma(u.x, u.x, u.y * u.y);
+      p1 += fma(a, y.x, b * y.y);
+    }
+  } else {
+    R al = 0, be = 0, gx = 0, gy = 0;
+#pragma unroll 4
+    for (int c = lane; c < N; c += 32) {
+      const C x = xr[c], y = yr[c];
+      al += fma(x.x, x.x, x.y * x.y);
+      be += fma(y.x, y.x, y.y * y.y);
+      gx += fma(x.x, y.x, x.y * y.y);
+      gy += fma(x.y, y.x, -(x.x * y.y));
+    }
+    p0 = (up ? be : al) + __shfl_xor_sync(all, up ? al : be, 16);
+    p1 = (up ? gy : gx) + __shfl_xor_sync(all, up ? gx : gy, 16);
+  }
+  R v = (odd ? p1 : p0) + __shfl_xor_sync(all, odd ? p0 : p1, 8);
+  v += __shfl_xor_sync(all, v, 4);
+  v += __shfl_xor_sync(all, v, 2);
+  v += __shfl_xor_sync(all, v, 1);
+  const R al = __shfl_sync(all, v, 0), gx = __shfl_sync(all, v, 8);
+  const R be = __shfl_sync(all, v, 16), gy = __shfl_sync(all, v, 24);
+  const R rt = sqrt(odd ? fma(gx, gx, gy * gy) : v);     // |g| beside the two norms
+  const R g = __shfl_sync(all, rt, 8);
+  if (g == 0 || g <= tol * __shfl_sync(all, rt, 0) * __shfl_sync(all, rt, 16)) return 0;
+  // a row below eps ||Z|| carries nothing at working precision; orthogonalising
+  // it (in subnormal arithmetic, at worst) would never meet the test above
+  const R lo = fmin(al, be);
+  if (lo <= floor) return 0;
+  // rows whose norms differ by more than 1e30 (1e15 in complex64) do not
+  // affect each other at working precision; rotating them only churns
+  // rounding noise (and never meets the relative test once a norm is subnormal)
+  const R far = sizeof(R) == 8 ? (R)1e-60 : (R)1e-30;
+  if (lo <= far * fmax(al, be)) return 0;
+  const R num = up ? be - al : (odd ? gy : gx), den = up ? 2 * g : g;
+  const R quo = num / den;
+  const R ex = __shfl_sync(all, quo, 0), ey = __shfl_sync(all, quo, 8), zeta = __shfl_sync(all, quo, 16);
+  const R t = (zeta >= 0 ? (R)1 : (R)-1) / (fabs(zeta) + sqrt(fma(zeta, zeta, (R)1)));
+  const R cs = (R)1 / sqrt(fma(t, t, (R)1)), sn = cs * t;
+#pragma unroll 4
+  for (int c = lane; c < len; c += 32) {
+    const C x = xr[c], y = yr[c];
+    const R wx = fma(ex, y.x, -(ey * y.y));
+    const R wy = ORD == kJacPlain32 ? fma(ex, y.y, ey * y.x) : fma(ey, y.x, ex * y.y);
+    xr[c] = mkj<C>(fma(x.x, cs, -(wx * sn)), fma(x.y, cs, -(wy * sn)));
+    yr[c] = mkj<C>(fma(x.x, sn, wx * cs), fma(x.y, sn, wy * cs));
+  }
+  return 1;
+}
+
 struct JacArgs {
-  int M, N, bs, nb;                      // rows, row length, rows a block, buffers (1 or 3)
+  int M, N, pp;                          // rows, row length, places a CTA
   int ldz, conj_t;                       // G_0[a][c] = Z[a ldz + c], or conj(Z[c ldz + a])
   int m, n, k;                           // exact SVD outputs (U, Rem not null): U m x k, Rem k x n
   double tol, floor_rel;
   int max_sweeps;
 };
 
-// E: entries of a row (N + M) a lane holds (0: rows stay in shared memory).
-template <typename C, int E, bool CL>
+// ||Z||^2 between 2^-kJacUnscaled and 2^kJacUnscaled: the rows are taken as they are;
+// beyond, scaled by a power of two to a norm near one (every rounding stays the
+// same, and no square of an entry that matters leaves the range).
+template <typename C> constexpr int kJacUnscaled = sizeof(C) == sizeof(float2) ? 40 : 400;
+
+__host__ __device__ inline size_t jac_header(int M) {
+  const size_t Mp = M + (M & 1);
+  return 64 + 160 + 512 + ((2 * sizeof(double) + sizeof(int)) * Mp + 15) / 16 * 16;
+}
+
+template <typename C, int ORD, bool CL>
 __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__ Z, C* __restrict__ Gout,
                                                 C* __restrict__ WHout, double* __restrict__ sigma,
                                                 int* __restrict__ idx, double* __restrict__ zn2_out, int* counters,
@@ -137,56 +173,69 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
   using R = typename RealJ<C>::T;
   cg::cluster_group cl = cg::this_cluster();
   const int cs = CL ? (int)cl.num_blocks() : 1, cr = CL ? (int)cl.block_rank() : 0;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int M = p.M, N = p.N, bs = p.bs, len = N + M;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const int M = p.M, N = p.N, pp = p.pp, len = N + M;
   const int ld = (len + 1) & ~1;         // entries of a row in shared memory (16-byte rows)
+  const int Mp = M + (M & 1), P = Mp / 2, rounds = Mp - 1;
+  const int q0 = cr * pp, pl = min(pp, P - q0);     // first place and number of places of this CTA
+  const int S = pp + 2;                  // slots of a ring
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const uint32_t bars = saddr(smem_raw);            // blocks (three), counts (two)
+  const uint32_t bars = saddr(smem_raw);            // first rows in (by parity), second rows in, counts
   volatile int* failed = (volatile int*)(smem_raw + 48);
   int* s_rot = (int*)(smem_raw + 52);
-  double* s_sum = (double*)(smem_raw + 64);         // [2 cs] sums and sweep counts of the CTAs
-  int* s_cnt = (int*)(s_sum + kJacMaxCluster);      // [2][cs][4]
-  double* s_sig = (double*)(smem_raw + 64 + 128 + 512);   // [2 cs bs] singular values (in home order)
-  const size_t hdr = 64 + 128 + 512 + sizeof(double) * (size_t)(2 * cs * bs);
-  // buffer b: two blocks of bs rows, then their squared norms
-  const uint32_t blk = (uint32_t)(sizeof(C) * (size_t)ld * bs), nrm = (uint32_t)((sizeof(R) * bs + 15) & ~15u);
-  const uint32_t half = blk + nrm, buf = 2 * half;
-  unsigned char* base = smem_raw + ((hdr + 15) & ~size_t(15));
-  auto rows = [&](int b, int h) { return (C*)(base + (size_t)b * buf + (size_t)h * half); };
-  auto norms = [&](int b, int h) { return (R*)(base + (size_t)b * buf + (size_t)h * half + blk); };
+  double* s_sum = (double*)(smem_raw + 64);         // [0] this CTA's sum, [1 ..] warps' sums
+  int* s_cnt = (int*)(smem_raw + 64 + 160);         // [2][16][4] rotations of a sweep, by CTA
+  double* s_sig = (double*)(smem_raw + 64 + 160 + 512);   // [Mp] singular values
+  double* s_inv = s_sig + Mp;            // [Mp] their inverses, zero below the floor
+  int* s_rank = (int*)(s_inv + Mp);      // [Mp], and a pad to sixteen bytes
+  C* rows = (C*)(smem_raw + jac_header(M));
+  // first rows: slot (j + R) mod S of place j in round R (all sweeps counted
+  // through), row M' - 1 in a slot of its own; second rows: slot (j - R) mod S
+  // (one CTA alone: row a at rows + a ld)
+  auto ring_a = [&](int j, int r) { return rows + (size_t)((j + r) % S) * ld; };
+  auto ring_b = [&](int j, int r) { return rows + (size_t)(S + (j + r * (S - 1)) % S) * ld; };
+  C* const fixed = rows + (size_t)(2 * S) * ld;
+  auto first = [&](int j, int r) {       // rows of place j
+    if constexpr (CL) return q0 + j == 0 ? fixed : ring_a(j, r);
+    else return rows + (size_t)(j == 0 ? Mp - 1 : (r + j) % rounds) * ld;
+  };
+  auto second = [&](int j, int r) {
+    if constexpr (CL) return ring_b(j, r);
+    else return rows + (size_t)((r - j % rounds + rounds) % rounds) * ld;
+  };
+  auto id_a = [&](int j) { return q0 + j == 0 ? Mp - 1 : q0 + j; };             // rows of the places
+  auto id_b = [&](int j) { return q0 + j == 0 ? 0 : Mp - 1 - (q0 + j); };       // when a sweep begins
   const C zero = mkj<C>(0, 0);
   if (tid == 0) {
-    for (int q = 0; q < 5; ++q) bar_init(bars + 8 * q);
+    for (int q = 0; q < 6; ++q) bar_init(bars + 8 * q);
     *failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
 
-  // ---- load: block 2 cr at the top, 2 cr + 1 at the bottom
+  // ---- load
   double part = 0.0;
-  for (int rr = warp; rr < 2 * bs; rr += nt >> 5) {
-    const int a = 2 * cr * bs + rr;
-    C* row = rows(0, rr / bs) + (size_t)(rr % bs) * ld;
-    for (int c = lane; c < ld; c += 32) {
-      C v = zero;
-      if (a < M) {
-        if (c < N) {
-          v = p.conj_t ? Z[(size_t)c * p.ldz + a] : Z[(size_t)a * p.ldz + c];
-          if (p.conj_t) v.y = -v.y;
-          part += (double)v.x * v.x + (double)v.y * v.y;
-        } else if (c - N == a) {
-          v = mkj<C>(1, 0);
-        }
+#pragma unroll 4
+  for (int e = tid; e < 2 * pl * ld; e += nt) {
+    const int rr = e / ld, c = e - rr * ld, j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
+    if (!CL && a >= M) continue;         // (no slot for the row that rounds M up)
+    C v = zero;
+    if (a < M) {
+      if (c < N) {
+        v = p.conj_t ? Z[(size_t)c * p.ldz + a] : Z[(size_t)a * p.ldz + c];
+        if (p.conj_t) v.y = -v.y;
+        part += (double)v.x * v.x + (double)v.y * v.y;
+      } else if (c - N == a) {
+        v = mkj<C>(1, 0);
       }
-      row[c] = v;
     }
+    (rr & 1 ? second(j, 0) : first(j, 0))[c] = v;
   }
   part = sum1(part);
-  __syncthreads();
-  if (lane == 0) s_sig[warp] = part;     // (at most 2 bs warps: bs of them)
+  if (lane == 0) s_sum[1 + warp] = part;
   __syncthreads();
   if (tid == 0) {
     double s = 0.0;
-    for (int w = 0; w < nt >> 5; ++w) s += s_sig[w];
+    for (int w = 0; w < nw; ++w) s += s_sum[1 + w];
     s_sum[0] = s;
   }
   double zn2 = 0.0;
@@ -199,214 +248,71 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
     zn2 = s_sum[0];
   }
   if (cr == 0 && tid == 0 && zn2_out) *zn2_out = zn2;
-  // the rows are scaled by a power of two so that ||G|| is near one
   int ex2 = 0;
   if (zn2 > 0.0 && isfinite(zn2)) {
     int e;
     frexp(zn2, &e);
-    ex2 = e / 2;
+    if (abs(e) > kJacUnscaled<C>) ex2 = e / 2;
     if (sizeof(R) == 4) ex2 = min(max(ex2, -120), 120);
   }
   const R up = (R)ldexp(1.0, -ex2), down = (R)ldexp(1.0, ex2);
   const R floor = (R)(p.floor_rel * (zn2 * ldexp(1.0, -2 * ex2)));
-  for (int e = tid; e < 2 * bs * N; e += nt) {
-    const int rr = e / N, c = e - rr * N;
-    C* x = rows(0, rr / bs) + (size_t)(rr % bs) * ld + c;
-    *x = mkj<C>(x->x * up, x->y * up);
-  }
+  if (ex2 != 0)
+    for (int rr = warp; rr < 2 * pl; rr += nw) {
+      C* row = rr & 1 ? second(rr >> 1, 0) : first(rr >> 1, 0);
+      if ((rr & 1 ? id_b(rr >> 1) : id_a(rr >> 1)) >= M) continue;
+      for (int c = lane; c < N; c += 32) row[c] = mkj<C>(row[c].x * up, row[c].y * up);
+    }
   __syncthreads();
 
-  const R far = sizeof(R) == 8 ? (R)1e-60 : (R)1e-30;
-  const float ftol = (float)p.tol;
-  int rot = 0;
-  // one pair: x (squared norm al) in registers, or at xr when rows are too
-  // long for that (E = 0), and y at row (squared norm at nb)
-  constexpr int EX = E > 0 ? E : 1;
-  auto pair = [&](C (&x)[EX], C* xr, R& al, C* row, R* nb) {
-    C y[EX];
-    R gx = 0, gy = 0;
-    if constexpr (E > 0) {
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int c = lane + 32 * e;
-        y[e] = c < len ? row[c] : zero;
-        if (c < N) {                     // x conj(y)
-          gx = fma(x[e].y, y[e].y, fma(x[e].x, y[e].x, gx));
-          gy = fma(-x[e].x, y[e].y, fma(x[e].y, y[e].x, gy));
-        }
+  // ---- sweeps
+  const uint32_t row_bytes = (uint32_t)(sizeof(C) * (size_t)ld);
+  // the warps at the CTA's ends wait for the rows of round r
+  auto arrive = [&](int r) {
+    if constexpr (CL) {
+      if (warp == (pl - 1) % nw && cr < cs - 1) {
+        if (lane == 0) bar_expect(bars + 8 * (r & 1), row_bytes);
+        __syncwarp();
+        bar_wait(bars + 8 * (r & 1), (r - 1) >> 1 & 1, failed);
       }
-    } else {
-      for (int c = lane; c < N; c += 32) {
-        const C u = xr[c], v = row[c];
-        gx = fma(u.y, v.y, fma(u.x, v.x, gx));
-        gy = fma(-u.x, v.y, fma(u.y, v.x, gy));
+      if (warp == 0 && cr > 0) {
+        if (lane == 0) bar_expect(bars + 16 + 8 * (r & 1), row_bytes);
+        __syncwarp();
+        bar_wait(bars + 16 + 8 * (r & 1), (r - 1) >> 1 & 1, failed);
       }
-    }
-    const R be = *nb;
-    sum2(gx, gy, lane);
-    // negligible against the rows' norms, a row below eps ||Z|| (it carries
-    // nothing at working precision, and would never meet the first test), or
-    // norms too far apart to affect each other
-    const int ge = top_exponent(gx, gy);
-    const float fx = image_scaled(gx, ge), fy = image_scaled(gy, ge);
-    const float g2 = fx * fx + fy * fy;
-    if (g2 == 0.f) return;
-    const float ig = rsqrtf(g2), g = g2 * ig;
-    float gs = g;                        // g on the scale of the norms
-    if (sizeof(R) == 8) gs = ldexpf(g, max(ge, -200));
-    if (gs * rsqrtf(image(al)) * rsqrtf(image(be)) <= ftol) return;
-    const R lo = al < be ? al : be, hi = al < be ? be : al;
-    if (lo <= floor || lo <= far * hi) return;
-    const float zeta = 0.5f * image_scaled(be - al, ge) * ig;
-    const float az = fabsf(zeta);
-    const float t = az > 1e15f ? __fdividef(0.5f, az) : __fdividef(1.f, az + sqrtf(fmaf(az, az, 1.f)));
-    const float ft = copysignf(t, zeta) * ig;
-    R tx, ty;
-    widen(ft * fx, tx);
-    widen(ft * fy, ty);
-    const R c = inv_root(fma(tx, tx, fma(ty, ty, (R)1)));
-    const R sx = c * tx, sy = c * ty;
-    const R d = fma(tx, gx, ty * gy);    // t |g|
-    auto turn = [&](C& u, C& v) {        // c u - sigma v, c v + conj(sigma) u
-      const C a = u, b = v;
-      u.x = fma(sy, b.y, fma(-sx, b.x, c * a.x));
-      u.y = fma(-sy, b.x, fma(-sx, b.y, c * a.y));
-      v.x = fma(sy, a.y, fma(sx, a.x, c * b.x));
-      v.y = fma(-sy, a.x, fma(sx, a.y, c * b.y));
-    };
-    if constexpr (E > 0) {
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        turn(x[e], y[e]);
-        const int q = lane + 32 * e;
-        if (q < len) row[q] = y[e];
-      }
-    } else {
-      for (int q = lane; q < len; q += 32) {
-        C u = xr[q], v = row[q];
-        turn(u, v);
-        xr[q] = u;
-        row[q] = v;
-      }
-    }
-    R na = al - d, nbe = be + d;
-    if (na < (R)0.25 * al || nbe < (R)0.25 * be) {   // cancelled: take both anew
-      R a = 0, b = 0;
-      if constexpr (E > 0) {
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-          if (lane + 32 * e < N) {
-            a = fma(x[e].y, x[e].y, fma(x[e].x, x[e].x, a));
-            b = fma(y[e].y, y[e].y, fma(y[e].x, y[e].x, b));
-          }
-      } else {
-        for (int q = lane; q < N; q += 32) {
-          const C u = xr[q], v = row[q];
-          a = fma(u.y, u.y, fma(u.x, u.x, a));
-          b = fma(v.y, v.y, fma(v.x, v.x, b));
-        }
-      }
-      sum2(a, b, lane);
-      na = a;
-      nbe = b;
-    }
-    al = na;
-    __syncwarp();
-    if (lane == 0) *nb = nbe;
-    ++rot;
-  };
-  auto load_row = [&](C (&x)[EX], const C* r) {
-    if constexpr (E > 0) {
-#pragma unroll
-      for (int e = 0; e < E; ++e) x[e] = lane + 32 * e < len ? r[lane + 32 * e] : zero;
     }
   };
-  auto store_row = [&](const C (&x)[EX], C* r) {
-    if constexpr (E > 0) {
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (lane + 32 * e < len) r[lane + 32 * e] = x[e];
-    }
+  auto send = [&](const C* row, C* to, uint32_t bar, int rank) {
+    const uint32_t src = saddr(row), dst = CL ? remote(saddr(to), rank) : 0u, b = CL ? remote(bar, rank) : 0u;
+    for (uint32_t o = 16 * lane; o < row_bytes; o += 512) push128(dst + o, b, lds128(src + o));
   };
-
-  int sweeps = 0, rot_total = 0, cur = 0;
-  uint32_t ph = 0, ph_cnt = 0;           // phases of the block barriers and of the counts
+  auto copy = [&](const C* row, C* to) {
+    const uint32_t src = saddr(row), dst = saddr(to);
+    for (uint32_t o = 16 * lane; o < row_bytes; o += 512) sts128(dst + o, lds128(src + o));
+  };
+  const R tol = (R)p.tol;
+  int sweeps = 0, rot_total = 0, R0 = 0;
+  uint32_t ph_cnt = 0;                   // phases of the counts' barriers
   bool converged = false;
-  C x[EX];
-  const int steps = 2 * cs - 1;
   while (sweeps < p.max_sweeps) {
-    rot = 0;
-    // squared norms, and the pairs within each block: warp w < bs / 2 works
-    // on the top block, the others on the bottom one
-    for (int rr = warp; rr < 2 * bs; rr += nt >> 5) {
-      const C* row = rows(cur, rr / bs) + (size_t)(rr % bs) * ld;
-      R a = 0;
-      for (int c = lane; c < N; c += 32) a = fma(row[c].y, row[c].y, fma(row[c].x, row[c].x, a));
-      a = sum1(a);
-      if (lane == 0) norms(cur, rr / bs)[rr % bs] = a;
-    }
-    __syncthreads();
-    const int bp = bs + (bs & 1), hp = bp / 2;       // rounds of a block's own tournament
-    for (int r = 0; r < bp - 1; ++r) {
-      for (int w = warp; w < 2 * hp; w += nt >> 5) {
-        const int h = w / hp, q = w % hp;
-        const int i = q == 0 ? bp - 1 : (r + q) % (bp - 1), j = q == 0 ? r : (r - q + bp - 1) % (bp - 1);
-        if (i < bs && j < bs) {
-          C* rx = rows(cur, h) + (size_t)i * ld;
-          R al = norms(cur, h)[i];
-          load_row(x, rx);
-          const int was = rot;
-          pair(x, rx, al, rows(cur, h) + (size_t)j * ld, norms(cur, h) + j);
-          if (rot != was) {
-            store_row(x, rx);
-            if (lane == 0) norms(cur, h)[i] = al;
+    int rot = 0;
+    for (int r = 0; r < rounds; ++r, ++R0) {
+      if (R0 > 0) arrive(R0);
+      for (int j = warp; j < pl; j += nw) {
+        C* x = first(j, CL ? R0 : r);
+        C* y = second(j, CL ? R0 : r);
+        if (q0 + j > 0 || Mp == M) rot += rotate_rows<C, ORD>(x, y, N, len, lane, tol, floor);
+        if constexpr (CL) {
+          __syncwarp();
+          // first rows go left: out of the CTA, or from place 1 to place 0 as its second row
+          if (j == 0 && cr > 0) send(x, ring_a(pp - 1, R0 + 1), bars + 8 * ((R0 + 1) & 1), cr - 1);
+          else if (q0 + j == 1) copy(x, ring_b(0, R0 + 1));
+          // second rows go right: out of the CTA, or at the last place become its first row
+          if (j == pl - 1) {
+            if (cr < cs - 1) send(y, ring_b(0, R0 + 1), bars + 16 + 8 * ((R0 + 1) & 1), cr + 1);
+            else copy(y, ring_a(j, R0 + 1));
           }
         }
-      }
-      __syncthreads();
-    }
-    // the blocks' tournament
-    for (int s = 0; s < steps; ++s) {
-      R al = 0;
-      C* rx = rows(cur, 0) + (size_t)min(warp, bs - 1) * ld;
-      if (warp < bs) {
-        al = norms(cur, 0)[warp];
-        load_row(x, rx);
-      }
-      for (int r = 0; r < bs; ++r) {
-        if (warp < bs) {
-          int j = warp + r;
-          if (j >= bs) j -= bs;
-          pair(x, rx, al, rows(cur, 1) + (size_t)j * ld, norms(cur, 1) + j);
-        }
-        __syncthreads();
-      }
-      if (warp < bs) {
-        store_row(x, rx);
-        if (lane == 0) norms(cur, 0)[warp] = al;
-      }
-      if constexpr (CL) {
-        __syncthreads();
-        // top blocks move right (the first stays, the last turns), bottom
-        // blocks left (the first turns)
-        const int nxt = cur == 2 ? 0 : cur + 1;
-        const bool keep_top = cr == 0, turn = cr == cs - 1;
-        if (tid == 0) bar_expect(bars + 8 * nxt, half * (uint32_t)((cr > 0) + (cr < cs - 1)));
-        const uint32_t src = saddr(base) + cur * buf, dst = saddr(base) + nxt * buf;
-        const uint32_t bt = remote(bars + 8 * nxt, min(cr + 1, cs - 1)), bb = remote(bars + 8 * nxt, cr == 0 ? 1 : cr - 1);
-        const uint32_t dt = remote(dst, min(cr + 1, cs - 1));                  // neighbour's top
-        const uint32_t db = remote(cr == 0 ? dst : dst + half, cr == 0 ? 1 : cr - 1);   // its bottom (its top from CTA 0)
-        for (uint32_t o = 16 * tid; o < half; o += 16 * nt) {
-          float4 v = lds128(src + o);
-          if (keep_top) sts128(dst + o, v);
-          else if (turn) sts128(dst + half + o, v);
-          else push128(dt + o, bt, v);
-          v = lds128(src + half + o);
-          push128(db + o, bb, v);
-        }
-        cur = nxt;
-        bar_wait(bars + 8 * cur, (ph >> cur) & 1u, failed);
-        ph ^= 1u << cur;
       }
       __syncthreads();
     }
@@ -418,41 +324,51 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
     int total = *s_rot;
     if constexpr (CL) {
       const int par = sweeps & 1;
-      if (tid == 0) bar_expect(bars + 8 * (3 + par), 16u * cs);
+      if (tid == 0) bar_expect(bars + 32 + 8 * par, 16u * cs);
       if (tid < cs)
-        push128(remote(saddr(s_cnt + (par * kJacMaxCluster + cr) * 4), tid), remote(bars + 8 * (3 + par), tid),
+        push128(remote(saddr(s_cnt + (par * kJacMaxCluster + cr) * 4), tid), remote(bars + 32 + 8 * par, tid),
                 make_float4(__int_as_float(total), 0.f, 0.f, 0.f));
-      bar_wait(bars + 8 * (3 + par), (ph_cnt >> par) & 1u, failed);
+      bar_wait(bars + 32 + 8 * par, (ph_cnt >> par) & 1u, failed);
       ph_cnt ^= 1u << par;
       total = 0;
       for (int q = 0; q < cs; ++q) total += s_cnt[(par * kJacMaxCluster + q) * 4];
     }
     __syncthreads();
+    const bool bad = *failed != 0;       // an exchange that ran out: no result
+    __syncthreads();
     ++sweeps;
     rot_total += total;
-    if (total == 0 || *failed) { converged = total == 0; break; }
+    if (total == 0 || bad) { converged = total == 0 && !bad; break; }
   }
+  if (R0 > 0) arrive(R0);                // the rows are back at their places
+  __syncthreads();
+  if (*failed) converged = false;
 
   // ---- row norms in double, ranks by size, outputs
-  for (int rr = warp; rr < 2 * bs; rr += nt >> 5) {
-    const C* row = rows(cur, rr / bs) + (size_t)(rr % bs) * ld;
+  for (int rr = warp; rr < 2 * pl; rr += nw) {
+    const int j = rr >> 1, id = rr & 1 ? id_b(j) : id_a(j);
+    if (id >= M) continue;
+    const C* row = rr & 1 ? second(j, CL ? R0 : 0) : first(j, CL ? R0 : 0);
     double a = 0.0;
-    for (int c = lane; c < N; c += 32) a += (double)row[c].x * row[c].x + (double)row[c].y * row[c].y;
+    for (int c = lane; c < N; c += 32) {
+      const double x = row[c].x, y = row[c].y;
+      a += fma(x, x, y * y);
+    }
     a = sum1(a);
-    if (lane == 0) s_sig[2 * cr * bs + rr] = sqrt(a) * ldexp(1.0, ex2);
+    if (lane == 0) s_sig[id] = sqrt(a) * ldexp(1.0, ex2);
   }
   __syncthreads();
   if constexpr (CL) {
     cl.sync();
-    for (int e = tid; e < 2 * cs * bs; e += nt) {
-      const int q = e / (2 * bs);
+    for (int e = tid; e < M; e += nt) {
+      const int q = (e == Mp - 1 ? 0 : (e < P ? e : Mp - 1 - e)) / pp;   // the CTA of the row's place
       if (q != cr) s_sig[e] = cl.map_shared_rank(s_sig, q)[e];
     }
     cl.sync();                           // (no remote access after this)
   }
   const double smin = sqrt(p.floor_rel * zn2);
-  for (int rr = warp; rr < 2 * bs; rr += nt >> 5) {
-    const int a = 2 * cr * bs + rr;
+  for (int rr = warp; rr < 2 * pl; rr += nw) {
+    const int j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
     if (a >= M) continue;
     // a total order (non-finite norms last), so the ranks are a permutation
     const double sg = s_sig[a];
@@ -464,24 +380,35 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-    const C* g = rows(cur, rr / bs) + (size_t)(rr % bs) * ld;
-    const C* w = g + N;
-    if (sigma && lane == 0) sigma[a] = sg;
-    if (idx && lane == 0 && rank < p.k) idx[rank] = a;
-    if (Gout)
-      for (int c = lane; c < N; c += 32) Gout[(size_t)a * N + c] = mkj<C>(g[c].x * down, g[c].y * down);
-    if (WHout)
-      for (int c = lane; c < M; c += 32) WHout[(size_t)a * M + c] = w[c];
-    if (U && rank < p.k) {
-      if (p.m <= p.n) {                  // U = WH^H, Rem = G
-        for (int c = lane; c < M; c += 32) U[(size_t)c * p.k + rank] = mkj<C>(w[c].x, -w[c].y);
-        for (int c = lane; c < N; c += 32) Rem[(size_t)rank * p.n + c] = mkj<C>(g[c].x * down, g[c].y * down);
-      } else {                           // rows of Z^H: U = G^H / sigma, Rem = sigma WH
-        const R is = sg > smin && sg > 0.0 ? (R)(1.0 / sg) : (R)0, s1 = (R)sg;
-        for (int c = lane; c < N; c += 32)
-          U[(size_t)c * p.k + rank] = mkj<C>(g[c].x * down * is, -(g[c].y * down) * is);
-        for (int c = lane; c < M; c += 32) Rem[(size_t)rank * p.n + c] = mkj<C>(w[c].x * s1, w[c].y * s1);
+    if (lane == 0) {
+      s_rank[a] = rank;
+      s_inv[a] = sg > smin && sg > 0.0 ? 1.0 / sg : 0.0;
+      if (sigma) sigma[a] = sg;
+      if (idx && rank < p.k) idx[rank] = a;
+    }
+  }
+  __syncthreads();
+#pragma unroll 2
+  for (int e = tid; e < 2 * pl * len; e += nt) {
+    const int rr = e / len, c = e - rr * len, j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
+    if (a >= M) continue;
+    const C x = (rr & 1 ? second(j, CL ? R0 : 0) : first(j, CL ? R0 : 0))[c];
+    const int rank = s_rank[a];
+    const bool top = U && rank < p.k;
+    const double sg = s_sig[a];
+    if (c < N) {
+      const C g = mkj<C>(x.x * down, x.y * down);
+      if (Gout) Gout[(size_t)a * N + c] = g;
+      if (top && p.m <= p.n) Rem[(size_t)rank * p.n + c] = g;       // U = WH^H, Rem = G
+      if (top && p.m > p.n) {            // rows of Z^H: U = G^H / sigma, Rem = sigma WH
+        const R is = (R)s_inv[a];
+        U[(size_t)c * p.k + rank] = mkj<C>(g.x * is, -g.y * is);
       }
+    } else {
+      const int w = c - N;
+      if (WHout) WHout[(size_t)a * M + w] = x;
+      if (top && p.m <= p.n) U[(size_t)w * p.k + rank] = mkj<C>(x.x, -x.y);
+      if (top && p.m > p.n) Rem[(size_t)rank * p.n + w] = mkj<C>(x.x * (R)sg, x.y * (R)sg);
     }
   }
   if (tid == 0 && !converged) *status = 1;   // the sweep limit, or an exchange that ran out
@@ -497,46 +424,38 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
 }
 
 struct JacPlan {
-  int cs = 0, bs = 0, nb = 0, e = 0;
+  int cs = 0, pp = 0, order = 0;
   size_t bytes = 0;
 };
 
+// Places a CTA.  complex128: two (four pairs an SM wait for its FP64 unit:
+// 64 clocks a warp-wide instruction).  complex64: one CTA up to
+// sixteen places (pushing rows costs more than two CTAs save: 31 x 40 280 us,
+// on two CTAs 335), else eight a CTA.  More when sixteen CTAs need it, and one CTA
+// alone where a cluster's rings (pp + 2 slots each) do not fit.
 template <typename C>
-bool jac_fit(int M, int N, int cs, JacPlan& p) {
-  static const int kE[] = {2, 4, 6, 8, 12};
-  const size_t R = sizeof(C) / 2;
-  p.cs = cs;
-  p.bs = (M + 2 * cs - 1) / (2 * cs);
-  p.nb = cs > 1 ? 3 : 1;
-  const int per = (N + M + 31) / 32;
-  p.e = 0;
-  for (int e : kE)
-    if (e >= per && (sizeof(C) == sizeof(float2) || e <= 8)) { p.e = e; break; }
-  if (p.bs > 16) return false;
-  const size_t ld = (size_t)((N + M + 1) & ~1);
-  const size_t half = sizeof(C) * ld * p.bs + ((R * p.bs + 15) & ~size_t(15));
-  const size_t hdr = 64 + 128 + 512 + sizeof(double) * (size_t)std::max(2 * cs * p.bs, 16);
-  p.bytes = ((hdr + 15) & ~size_t(15)) + 2 * half * p.nb;
+bool jac_plan(int M, int N, JacPlan& p) {
+  const bool c64 = sizeof(C) == sizeof(float2);
+  const int P = (M + 1) / 2, pref = c64 ? 8 : 2;
+  const size_t row = sizeof(C) * (size_t)((N + M + 1) & ~1);
+  const bool staged = sizeof(C) * ((size_t)M * N + (size_t)M * M) <= kJacStaged;
+  p.order = !staged ? kJacPlain32 : (M > 64 ? kJacStaged16 : kJacStaged32);
+  if (P > (c64 ? 16 : pref)) {
+    p.pp = std::max(pref, (P + kJacMaxCluster - 1) / kJacMaxCluster);
+    p.cs = (P + p.pp - 1) / p.pp;
+    p.bytes = jac_header(M) + row * (2 * (p.pp + 2) + 1);
+    if (p.bytes <= kJacSmemMax) return true;
+  }
+  p.pp = P;
+  p.cs = 1;
+  p.bytes = jac_header(M) + row * M;
   return p.bytes <= kJacSmemMax;
 }
 
-// CTAs of an M-row problem: complex128 four pairs a CTA (one per FP64
-// sub-partition), complex64 eight.
-template <typename C>
-bool jac_plan(int M, int N, JacPlan& p) {
-  const int pairs = sizeof(C) == sizeof(float2) ? 8 : 4;
-  const int want = std::min(kJacMaxCluster, std::max(1, (M + 2 * pairs - 1) / (2 * pairs)));
-  for (int cs = want; cs <= kJacMaxCluster; ++cs)
-    if (jac_fit<C>(M, N, cs, p)) return true;
-  for (int cs = want - 1; cs >= 1; --cs)
-    if (jac_fit<C>(M, N, cs, p)) return true;
-  return false;
-}
-
-template <typename C, int E, bool CL>
+template <typename C, int ORD, bool CL>
 cudaError_t jac_run(const JacPlan& p, const JacArgs& a, const C* Z, C* G, C* WH, double* sigma, int* idx, double* zn2,
                     int* counters, C* U, C* Rem, int* status, double* flops, cudaStream_t s) {
-  auto kern = k_jac<C, E, CL>;
+  auto kern = k_jac<C, ORD, CL>;
   static std::atomic<unsigned long long> done{0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -551,7 +470,7 @@ cudaError_t jac_run(const JacPlan& p, const JacArgs& a, const C* Z, C* G, C* WH,
   if (p.cs == 0) return cudaSuccess;     // (the attributes only)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.cs, 1, 1);
-  cfg.blockDim = dim3(32 * std::max(p.bs + (p.bs & 1), 1), 1, 1);
+  cfg.blockDim = dim3(32 * std::min(std::max(p.pp, 8), 16), 1, 1);   // (eight warps load and store)
   cfg.dynamicSmemBytes = p.bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -564,29 +483,20 @@ cudaError_t jac_run(const JacPlan& p, const JacArgs& a, const C* Z, C* G, C* WH,
   return cudaLaunchKernelEx(&cfg, kern, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops);
 }
 
+template <typename C, int ORD>
+cudaError_t jac_order(const JacPlan& p, bool cl, const JacArgs& a, const C* Z, C* G, C* WH, double* sigma, int* idx,
+                      double* zn2, int* counters, C* U, C* Rem, int* status, double* flops, cudaStream_t s) {
+  return cl ? jac_run<C, ORD, true>(p, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s)
+            : jac_run<C, ORD, false>(p, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s);
+}
 template <typename C>
 cudaError_t jac_pick(const JacPlan& p, bool cl, const JacArgs& a, const C* Z, C* G, C* WH, double* sigma, int* idx,
                      double* zn2, int* counters, C* U, C* Rem, int* status, double* flops, cudaStream_t s) {
-#define BBP_JAC(E)                                                                                       \
-  case E:                                                                                                \
-    return cl ? jac_run<C, E, true>(p, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s)  \
-              : jac_run<C, E, false>(p, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s)
-  switch (p.e) {
-    BBP_JAC(0);
-    BBP_JAC(2);
-    BBP_JAC(4);
-    BBP_JAC(6);
-    BBP_JAC(8);
-    default: break;
-  }
-  if constexpr (sizeof(C) == sizeof(float2)) {
-    switch (p.e) {
-      BBP_JAC(12);
-      default: break;
-    }
-  }
-#undef BBP_JAC
-  return cudaErrorInvalidValue;
+  if (p.order == kJacStaged16)
+    return jac_order<C, kJacStaged16>(p, cl, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s);
+  if (p.order == kJacStaged32)
+    return jac_order<C, kJacStaged32>(p, cl, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s);
+  return jac_order<C, kJacPlain32>(p, cl, a, Z, G, WH, sigma, idx, zn2, counters, U, Rem, status, flops, s);
 }
 
 template <typename C>
@@ -599,8 +509,7 @@ cudaError_t jac_t(const C* Z, int ldz, bool conj_t, int M, int N, int k, C* G, C
   JacArgs a;
   a.M = M;
   a.N = N;
-  a.bs = p.bs;
-  a.nb = p.nb;
+  a.pp = p.pp;
   a.ldz = ldz;
   a.conj_t = conj_t ? 1 : 0;
   a.m = m;
@@ -617,10 +526,9 @@ template <typename C>
 cudaError_t jac_optin() {
   JacPlan p;
   JacArgs a = {};
-  for (int e : {0, 2, 4, 6, 8, 12})
+  for (int order : {kJacPlain32, kJacStaged32, kJacStaged16})
     for (bool cl : {false, true}) {
-      if (e > 8 && sizeof(C) != sizeof(float2)) continue;
-      p.e = e;
+      p.order = order;
       cudaError_t r = jac_pick<C>(p, cl, a, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
                                   nullptr, nullptr, nullptr, 0);
       if (r != cudaSuccess) return r;
