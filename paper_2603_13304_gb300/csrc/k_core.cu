@@ -152,15 +152,18 @@ __global__ void __launch_bounds__(256) k_fuse(const double2* __restrict__ t, int
 // entries of it (rows ty + i TM / RM, columns tx + j TN / RN, so that a warp
 // reads two rows and sixteen consecutive columns of a k slice from shared
 // memory), K in slices of kGemmK double-buffered in shared memory with the
-// next slice on its way in registers.  KG thread groups share a slice's k
-// (summed at the end).
+// next slice on its way in registers.
 //
-// complex64: 96 multiply-adds per ten shared-memory loads at 4 x 6 entries, so
-// that the FMA pipe and not the loads bounds it; every product is a chain of
-// fused multiply-adds (a complex product added to the sum takes half as many
-// instructions again).  complex128 is bound by the FP64 rate (two
-// multiply-adds a clock and SM) at any tile, so its tiles are small: padding
-// to a tile costs FP64 time, and a product must spread over many SMs.
+// An entry is the sum over k in order of rounded products (cmac): with these
+// roundings any tile gives the same bits.  The order and the rounding are part
+// of the results (k_jac.cu says why); chains of four fused multiply-adds a
+// product in place of two products, two fused multiply-adds and two additions
+// would take a third off the arithmetic.
+//
+// complex64: 72 to 144 instructions per seven to ten shared-memory loads, so
+// that the FMA pipe and not the loads bounds it.  complex128 is bound by the
+// FP64 rate at any tile, so its tiles are small: padding to a tile costs FP64
+// time, and a product must spread over many SMs.
 constexpr int kGemmK = 16;
 
 template <typename C>
@@ -170,24 +173,28 @@ __device__ __forceinline__ C load_op(const C* P, int ld, char op, int r, int c, 
   C v = P[(long long)c * ld + r];
   return op == 'C' ? cconj(v) : v;
 }
-template <typename C> __device__ __forceinline__ void cfma(C& s, C a, C b) {   // s += a b
-  s.x = fma(-a.y, b.y, fma(a.x, b.x, s.x));
-  s.y = fma(a.y, b.x, fma(a.x, b.y, s.y));
+// a b and s + a b, each product rounded once before it is added
+template <typename C> __device__ __forceinline__ C cprod(C a, C b) {
+  C r;
+  r.x = fma(a.x, b.x, -(a.y * b.y));
+  r.y = fma(a.y, b.x, a.x * b.y);
+  return r;
 }
+template <typename C> __device__ __forceinline__ void cmac(C& s, C a, C b) { s = cadd(s, cprod(a, b)); }
 
 // With part != null the grid's z index is a slice of K (kchunk entries,
 // batch 1): each CTA writes its raw partial tile to part[z][M][N] and
 // k_gemm_reduce adds the slices in order (split K for skinny products).
-template <typename C, int TM, int TN, int RM, int RN, int KG>
-__global__ void __launch_bounds__((TM / RM) * (TN / RN) * KG, 2)
+template <typename C, int TM, int TN, int RM, int RN>
+__global__ void __launch_bounds__((TM / RM) * (TN / RN), 2)
     k_gemm(char opA, char opB, int M, int N, int K, C alpha, const C* __restrict__ A, int lda, long long sA,
            const C* __restrict__ B, int ldb, long long sB, C beta, C* __restrict__ Cm, int ldc, long long sC,
            int kchunk, C* __restrict__ part) {
-  constexpr int TX = TN / RN, TY = TM / RM, NT = TX * TY * KG;
+  constexpr int TX = TN / RN, TY = TM / RM, NT = TX * TY;
   constexpr int PA = (TM * kGemmK + NT - 1) / NT, PB = (TN * kGemmK + NT - 1) / NT;
   __shared__ C As[2][kGemmK][TM + 1];
   __shared__ C Bs[2][kGemmK][TN + 1];
-  const int tid = threadIdx.x, g = tid / (TX * TY), tx = tid % TX, ty = (tid / TX) % TY;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int bz = blockIdx.z;
   int kb = 0, ke = K;
   if (part) {
@@ -244,10 +251,8 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN) * KG, 2)
   for (int k0 = kb; k0 < ke; k0 += kGemmK) {
     const bool more = k0 + kGemmK < ke;
     if (more) fetch(k0 + kGemmK);
-    constexpr int KK = kGemmK / KG;
 #pragma unroll 4
-    for (int q = 0; q < KK; ++q) {
-      const int kk = KG > 1 ? g * KK + q : q;
+    for (int kk = 0; kk < kGemmK; ++kk) {
       C a[RM], b[RN];
 #pragma unroll
       for (int i = 0; i < RM; ++i) a[i] = As[buf][kk][ty + TY * i];
@@ -256,20 +261,11 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN) * KG, 2)
 #pragma unroll
       for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < RN; ++j) cfma(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < RN; ++j) cmac(acc[i][j], a[i], b[j]);
     }
     if (more) stage(buf ^ 1);
     __syncthreads();
     buf ^= 1;
-  }
-  if constexpr (KG > 1) {                // the groups' sums, in order
-    C* sum = &As[0][0][0];
-    static_assert(RM * RN == 1 && TX * TY * KG <= 2 * kGemmK * (TM + 1), "the sums fit the staging buffer");
-    sum[tid] = acc[0][0];
-    __syncthreads();
-    if (g > 0) return;
-#pragma unroll
-    for (int q = 1; q < KG; ++q) acc[0][0] = cadd(acc[0][0], sum[q * TX * TY + tid]);
   }
 #pragma unroll
   for (int i = 0; i < RM; ++i)
@@ -281,8 +277,8 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN) * KG, 2)
           part[((long long)bz * M + r) * N + c] = acc[i][j];
           continue;
         }
-        C v = cmul(alpha, acc[i][j]);
-        if (beta.x != 0 || beta.y != 0) v = cadd(v, cmul(beta, Cm[(long long)r * ldc + c]));
+        C v = cprod(alpha, acc[i][j]);
+        if (beta.x != 0 || beta.y != 0) cmac(v, beta, Cm[(long long)r * ldc + c]);
         Cm[(long long)r * ldc + c] = v;
       }
     }
@@ -1421,25 +1417,36 @@ cudaError_t launch_fuse(const double2* t, int d, int D, const int n[4], const do
 }
 
 // K slices of a skinny product (few output tiles, long K) when a scratch of
-// kSplitMax x M x N entries is given
+// kSplitMax x M x N entries is given.  Their number goes by 32 x 32 tiles,
+// whatever tile is launched: it is part of the order of the sums.
 constexpr int kSplitMax = 8;
+template <typename C>
+static int gemm_slices(int M, int N, int K, int batch, const void* work, size_t work_bytes) {
+  const long long tiles = ((long long)(N + 31) / 32) * ((M + 31) / 32);
+  if (batch != 1 || !work || tiles >= 2 * 152 || K < 8 * kGemmK) return 1;
+  int S = std::min(kSplitMax, std::max(2, (6 * 152) / (int)tiles));
+  S = std::min(S, K / (4 * kGemmK));
+  while (S > 1 && (size_t)S * M * N * sizeof(C) > work_bytes) --S;
+  if (S <= 1) return 1;
+  const int kchunk = ((K + S - 1) / S + kGemmK - 1) / kGemmK * kGemmK;
+  return (K + kchunk - 1) / kchunk;
+}
 
-template <typename C, int TM, int TN, int RM, int RN, int KG>
+template <typename C, int TM, int TN, int RM, int RN>
 static cudaError_t gemm_tile(char opA, char opB, int M, int N, int K, C alpha, const C* A, int lda, long long sA,
                              const C* B, int ldb, long long sB, C beta, C* Cm, int ldc, long long sC, int batch,
                              int S, C* part, cudaStream_t s) {
-  constexpr int NT = (TM / RM) * (TN / RN) * KG;
+  constexpr int NT = (TM / RM) * (TN / RN);
   const long long tiles = ((long long)(N + TN - 1) / TN) * ((M + TM - 1) / TM);
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   if (S > 1) {
     const int kchunk = ((K + S - 1) / S + kGemmK - 1) / kGemmK * kGemmK;
-    S = (K + kchunk - 1) / kchunk;
-    k_gemm<C, TM, TN, RM, RN, KG><<<dim3((unsigned)tiles, 1, S), NT, 0, s>>>(opA, opB, M, N, K, alpha, A, lda, sA, B,
-                                                                            ldb, sB, beta, Cm, ldc, sC, kchunk, part);
+    k_gemm<C, TM, TN, RM, RN><<<dim3((unsigned)tiles, 1, S), NT, 0, s>>>(opA, opB, M, N, K, alpha, A, lda, sA, B, ldb,
+                                                                        sB, beta, Cm, ldc, sC, kchunk, part);
     k_gemm_reduce<C><<<grid_for((long long)M * N, 256), 256, 0, s>>>(part, S, M, N, alpha, beta, Cm, ldc);
     return cudaGetLastError();
   }
-  k_gemm<C, TM, TN, RM, RN, KG><<<dim3((unsigned)tiles, 1, batch), NT, 0, s>>>(
+  k_gemm<C, TM, TN, RM, RN><<<dim3((unsigned)tiles, 1, batch), NT, 0, s>>>(
       opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, 0, nullptr);
   return cudaGetLastError();
 }
@@ -1450,37 +1457,28 @@ static cudaError_t gemm_t(char opA, char opB, int M, int N, int K, C alpha, cons
                           cudaStream_t s, void* work = nullptr, size_t work_bytes = 0) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   KTimerScope timer(KC_GEMM, s, 8.0 * M * N * (double)K * batch);
-  // slices that bring `tiles` tiles to `want` CTAs, at least four k steps each
-  auto slices = [&](long long tiles, long long want) {
-    if (batch != 1 || !work || tiles >= want || K < 8 * kGemmK) return 1;
-    int S = (int)std::min<long long>(kSplitMax, (want + tiles - 1) / tiles);
-    S = std::max(1, std::min(S, K / (4 * kGemmK)));
-    while (S > 1 && (size_t)S * M * N * sizeof(C) > work_bytes) --S;
-    return S;
-  };
-  auto tiles_of = [&](int tm, int tn) { return ((long long)(M + tm - 1) / tm) * ((N + tn - 1) / tn) * batch; };
-#define BBP_GEMM(TM, TN, RM, RN, KG, S)                                                                      \
-  return gemm_tile<C, TM, TN, RM, RN, KG>(opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, \
-                                          batch, S, (C*)work, s)
+  const int S = gemm_slices<C>(M, N, K, batch, work, work_bytes);
+  // CTAs of a tile
+  auto ctas = [&](int tm, int tn) { return ((long long)(M + tm - 1) / tm) * ((N + tn - 1) / tn) * batch * S; };
+#define BBP_GEMM(TM, TN, RM, RN)                                                                                       \
+  return gemm_tile<C, TM, TN, RM, RN>(opA, opB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, Cm, ldc, sC, batch, S, \
+                                      (C*)work, s)
   if constexpr (sizeof(C) == sizeof(float2)) {
-    // 64-row tiles of the width that pads N least, once they and the slices
-    // of K fill the SMs; else 32 x 32
+    // 64-row tiles of the width that pads N least where they give every SM
+    // nearly two CTAs, 48 columns where only those do; else 32 x 32
     int tn = 96;
     for (int w : {64, 48})
       if ((N + w - 1) / w * w < (N + tn - 1) / tn * tn) tn = w;
-    const long long tiles = tiles_of(64, tn);
-    const int S = slices(tiles, 2 * 152);
-    if (M > 32 && tiles * S >= 152) {
-      if (tn == 96) { BBP_GEMM(64, 96, 4, 6, 1, S); }
-      if (tn == 64) { BBP_GEMM(64, 64, 4, 4, 1, S); }
-      BBP_GEMM(64, 48, 4, 3, 1, S);
+    if (ctas(64, tn) < 256 && (N + 47) / 48 * 48 <= (N + tn - 1) / tn * tn) tn = 48;
+    if (M > 32 && ctas(64, tn) >= 152) {
+      if (tn == 96) { BBP_GEMM(64, 96, 4, 6); }
+      if (tn == 64) { BBP_GEMM(64, 64, 4, 4); }
+      BBP_GEMM(64, 48, 4, 3);
     }
-    BBP_GEMM(32, 32, 2, 2, 1, slices(tiles_of(32, 32), 6 * 152));
+    BBP_GEMM(32, 32, 2, 2);
   } else {
-    const long long tiles = tiles_of(16, 16);
-    const int S = slices(tiles, 5 * 152);
-    if (tiles * S >= 2 * 152) { BBP_GEMM(16, 16, 1, 2, 1, S); }
-    BBP_GEMM(8, 8, 1, 1, 2, slices(tiles_of(8, 8), 5 * 152));
+    if (ctas(16, 16) >= 2 * 152) { BBP_GEMM(16, 16, 1, 2); }
+    BBP_GEMM(8, 8, 1, 1);
   }
 #undef BBP_GEMM
 }
