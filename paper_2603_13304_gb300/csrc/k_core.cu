@@ -1178,217 +1178,108 @@ __global__ void k_omega(C* O, int n, int b) {
 
 // FP64 finish of the reduced SVD (complex64 modes).  After the complex64
 // Jacobi, the rows of G' = WH L (b x b) are orthogonal to complex64 accuracy
-// and idx holds the k largest.  In complex128 every pair (kept x, discarded y)
-// is rotated once more, x' = x - tau y, y' = y + conj(tau) x with the Jacobi
-// tau of the pair, which makes the kept rows orthogonal to the discarded ones;
-// then the row norms and the choice of the k largest rows are taken in double.
-//
-// All tau are small (the complex64 Jacobi left inner products of about 1e-6 of
-// the norms), so the k (b - k) rotations are applied at once: a CTA per row
-// takes the tau of its row against the opposite set and the sum of their
-// rows, and rescales the row so that its WH part has unit norm.  What that
-// leaves is of second order in tau, as one sequential sweep leaves.  A pair
-// whose tau is not small (norms equal to about 1e-3 of themselves) is left out
-// here and marked; k_cut_select rotates the marked pairs one after another.
-// Rows below eps ||Z|| of complex64 (the floor of the complex64 Jacobi) hold
-// only the rounding of Z, with norms all alike: their pairs are not marked
-// (on the BlockBP splits every pair with a large tau is of that kind).
-// Against one cluster that rotated pair after pair (64 rounds of a cluster
-// barrier, remote rows and FP64 scalars): 653 us and 75 us (both kernels) at b = 96, k = 64;
-// bound by the FP64 rate of each row's SM.
-constexpr double kCutSmall = 1e-6;   // |tau|^2 of a rotation applied with all others
-constexpr double kCutNoise = floor_rel_of<float2>();
+// and idx holds the k largest.  The rows of G' and WH are promoted to
+// complex128 and every pair (kept, discarded) is rotated once more in double
+// arithmetic, which makes the kept rows orthogonal to the discarded ones to
+// double accuracy (the rotations within either set do not change the kept
+// subspace); then the row norms and the choice of the k largest rows are
+// taken in double.  The FP64 units of one SM are the bottleneck, so the rows
+// of G' are spread over the shared memory of a cluster of kCutCluster CTAs
+// (row r on CTA r % kCutCluster) and every round's disjoint pairs over all
+// their warps, with one cluster barrier per round; WH stays in global memory.
+constexpr int kCutCluster = 16;   // (a non-portable cluster size, opted in)
 
-struct CutLayout {
-  size_t row, opp, gx, gy, n2, red, bytes;
-};
-__host__ __device__ inline CutLayout cut_layout(int b) {
-  CutLayout L;
-  size_t o = 0;
-  L.row = o; o += sizeof(double2) * b;
-  L.gx = o; o += sizeof(double) * b;
-  L.gy = o; o += sizeof(double) * b;
-  L.n2 = o; o += sizeof(double) * b;
-  L.red = o; o += sizeof(double) * 40;
-  L.opp = o; o += sizeof(int) * (size_t)(2 * b + 2);
-  L.bytes = o;
-  return L;
-}
-
-// the Jacobi tau of rows x, y: squared norms al, be, inner product g = x y^H;
-// zero when the pair needs no rotation (the tests of rotate_pair)
-__device__ __forceinline__ double2 cut_tau(double al, double be, double gx, double gy, double floor) {
-  const double g = sqrt(gx * gx + gy * gy);
-  if (g == 0 || g <= 1e-15 * sqrt(al) * sqrt(be) || fmin(al, be) <= floor || fmin(al, be) <= 1e-60 * fmax(al, be))
-    return make_double2(0.0, 0.0);
-  const double zeta = (be - al) / (2 * g);
-  const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta)) / g;
-  return make_double2(t * gx, t * gy);
-}
-
-constexpr int kCutThreads = 256;
-__global__ void __launch_bounds__(kCutThreads) k_cut_rows(const float2* __restrict__ G, const float2* __restrict__ WH,
-                                                          const int* __restrict__ idx, int b, int k,
-                                                          const double* __restrict__ zn2, double2* __restrict__ G64,
-                                                          double2* __restrict__ WH64, double* __restrict__ sig64,
-                                                          int* __restrict__ big, int* __restrict__ nbig) {
+__global__ void __launch_bounds__(1024) k_jacobi_cut64(SvdWork<float2> w, int b, int k, double2* __restrict__ G64,
+                                                       double2* __restrict__ WH64, double* __restrict__ sig64,
+                                                       int* __restrict__ idx64) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), cr = (int)cl.block_rank();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const CutLayout L = cut_layout(b);
-  double2* row = (double2*)(smem_raw + L.row);
-  double* s_gx = (double*)(smem_raw + L.gx);
-  double* s_gy = (double*)(smem_raw + L.gy);
-  double* s_n2 = (double*)(smem_raw + L.n2);
-  double* red = (double*)(smem_raw + L.red);
-  int* opp = (int*)(smem_raw + L.opp);
-  int* mark = opp + b;
-  const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  for (int e = tid; e < b; e += blockDim.x) {
-    mark[e] = 0;
-    big[(size_t)r * b + e] = 0;
-    row[e] = c128(G[(size_t)r * b + e]);
+  const int rpc = (b + cs - 1) / cs;          // rows per CTA
+  double2* G = (double2*)smem_raw;            // local rows: r = cr + cs * t at G + t * b
+  int* kept = (int*)(G + (size_t)rpc * b);    // k
+  int* disc = kept + k;                       // b - k
+  int* mark = disc + (b - k);                 // b
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int e = threadIdx.x; e < rpc * b; e += blockDim.x) {
+    const int t = e / b, c = e % b, r = cr + cs * t;
+    if (r < b) G[e] = c128(w.G[(size_t)r * b + c]);
+  }
+  for (int e = threadIdx.x; e < b * b; e += blockDim.x)
+    if ((e / b) % cs == cr) __stcg(WH64 + e, c128(w.WH[e]));
+  for (int e = threadIdx.x; e < b; e += blockDim.x) mark[e] = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < k; e += blockDim.x) {
+    const int a = min(max(w.idx[e], 0), b - 1);
+    kept[e] = a;
+    mark[a] = 1;
   }
   __syncthreads();
-  for (int e = tid; e < k; e += blockDim.x) mark[min(max(idx[e], 0), b - 1)] = 1;
-  __syncthreads();
-  const bool kept = mark[r] != 0;
-  if (warp == 0) {                       // the opposite set, in order
-    int n = 0;
-    for (int e0 = 0; e0 < b; e0 += 32) {
-      const bool in = e0 + lane < b && (mark[min(e0 + lane, b - 1)] != 0) != kept;
-      const unsigned m = __ballot_sync(0xffffffffu, in);
-      if (in) opp[n + __popc(m & ((1u << lane) - 1))] = e0 + lane;
-      n += __popc(m);
-    }
-    if (lane == 0) mark[b] = n;
+  if (threadIdx.x == 0) {
+    int q = 0;
+    for (int a = 0; a < b; ++a)
+      if (!mark[a] && q < b - k) disc[q++] = a;
+    for (; q < b - k; ++q) disc[q] = -1;     // duplicate indices in idx (never expected)
   }
-  double al = 0.0;                       // the row's own squared norm, in every warp
-  for (int c = lane; c < b; c += 32) al = fma(row[c].y, row[c].y, fma(row[c].x, row[c].x, al));
-  al = warp_sum(al);
-  __syncthreads();
-  const int no = mark[b];
-  // inner products (kept row times conj discarded row, the same order of
-  // terms in both rows' CTAs) and norms
-  for (int o = warp; o < no; o += nw) {
-    const float2* other = G + (size_t)opp[o] * b;
-    double gx = 0.0, gy = 0.0, n2 = 0.0;
-    for (int c = lane; c < b; c += 32) {
-      const double2 z = c128(other[c]), x = kept ? row[c] : z, y = kept ? z : row[c];
-      gx = fma(x.y, y.y, fma(x.x, y.x, gx));
-      gy = fma(-x.x, y.y, fma(x.y, y.x, gy));
-      n2 = fma(z.y, z.y, fma(z.x, z.x, n2));
-    }
-    gx = warp_sum(gx);
-    gy = warp_sum(gy);
-    n2 = warp_sum(n2);
-    if (lane == 0) {
-      s_gx[o] = gx;
-      s_gy[o] = gy;
-      s_n2[o] = n2;
-    }
-  }
-  __syncthreads();
-  const double floor = 1e-32 * *zn2;     // eps^2 of double, as in the complex128 Jacobi
-  for (int o = tid; o < no; o += blockDim.x) {
-    double2 t = kept ? cut_tau(al, s_n2[o], s_gx[o], s_gy[o], floor) : cut_tau(s_n2[o], al, s_gx[o], s_gy[o], floor);
-    const bool far = !(t.x * t.x + t.y * t.y <= kCutSmall);
-    if (kept && far && !(fmin(al, s_n2[o]) <= kCutNoise * *zn2)) {
-      big[(size_t)r * b + opp[o]] = 1;
-      atomicAdd(nbig, 1);
-    }
-    if (far) t = make_double2(0.0, 0.0);
-    // x' = x - tau y, y' = y + conj(tau) x
-    s_gx[o] = kept ? -t.x : t.x;
-    s_gy[o] = -t.y;
-  }
-  __syncthreads();
-  double wn = 0.0, gn = 0.0;
-  double2* out_g = G64 + (size_t)r * b;
-  double2* out_w = WH64 + (size_t)r * b;
-  for (int c = tid; c < 2 * b; c += blockDim.x) {
-    const float2* src = c < b ? G + c : WH + (c - b);
-    double2 v = c128(src[(size_t)r * b]);
-    for (int o = 0; o < no; ++o) {
-      const double2 z = c128(__ldg(src + (size_t)opp[o] * b));
-      const double tx = s_gx[o], ty = s_gy[o];
-      v.x = fma(-ty, z.y, fma(tx, z.x, v.x));
-      v.y = fma(ty, z.x, fma(tx, z.y, v.y));
-    }
-    const double q = fma(v.x, v.x, v.y * v.y);
-    if (c < b) { gn += q; out_g[c] = v; }
-    else { wn += q; out_w[c - b] = v; }
-  }
-  gn = block_sum(gn, red);
-  __syncthreads();
-  wn = block_sum(wn, red);
-  const double s = wn > 0.0 ? 1.0 / sqrt(wn) : 1.0;
-  for (int c = tid; c < 2 * b; c += blockDim.x) {   // (a thread's own entries)
-    double2* p = c < b ? out_g + c : out_w + (c - b);
-    *p = make_double2(p->x * s, p->y * s);
-  }
-  if (tid == 0) sig64[r] = sqrt(gn) * s;
-}
-
-// The marked pairs rotated in order, the k largest rows by their norms, and
-// those rows of WH and G' in complex64 (one CTA).
-__global__ void __launch_bounds__(1024) k_cut_select(double2* __restrict__ G64, double2* __restrict__ WH64,
-                                                            double* __restrict__ sig64, const int* __restrict__ big,
-                                                            const int* __restrict__ nbig, int b, int k,
-                                                            const double* __restrict__ zn2, float2* __restrict__ Wt,
-                                                            float2* __restrict__ Gt) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* sig = (double*)smem_raw;       // b
-  int* top = (int*)(sig + b);            // k
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  if (*nbig > 0) {
-    if (warp == 0)
-      for (int p = 0; p < b * b; ++p) {
-        if (!big[p]) continue;           // (uniform: every lane reads the same mark)
-        const int i = p / b, j = p % b;
-        rotate_pair<true, double2, true>(G64 + (size_t)i * b, G64 + (size_t)j * b, b, WH64 + (size_t)i * b,
-                                         WH64 + (size_t)j * b, b, lane, 1e-15, 1e-32 * *zn2);
-        __syncwarp();
+  cl.sync();                                  // every CTA's rows and WH rows are in place
+  auto grow = [&](int r) { return cl.map_shared_rank(G, r % cs) + (size_t)(r / cs) * b; };
+  const int nd = b - k;
+  const double floor = 1e-32 * (double)*w.zn2;   // eps^2 of double, as in the complex128 Jacobi
+  if (nd > 0 && k > 0) {
+    const int nbig = k >= nd ? k : nd, nsmall = k >= nd ? nd : k;
+    const int* big = k >= nd ? kept : disc;
+    const int* small = k >= nd ? disc : kept;
+    for (int r = 0; r < nbig; ++r) {          // round r: pairs (big[(p + r) % nbig], small[p]), disjoint
+      for (int p = cr + cs * warp; p < nsmall; p += cs * nw) {   // pairs dealt round-robin over the CTAs
+        const int a = big[(p + r) % nbig], c = small[p];
+        if (a < 0 || c < 0) continue;
+        // rows of G' in (distributed) shared memory, rows of WH in global
+        // memory past L1 (other CTAs of the cluster rotate them too)
+        rotate_pair<false, double2, true>(grow(a), grow(c), b, WH64 + (size_t)a * b, WH64 + (size_t)c * b, b, lane,
+                                          1e-15, floor);
       }
-    __threadfence_block();
-    __syncthreads();
-    for (int r = warp; r < b; r += nw) {
-      double sq = 0.0;
-      for (int c = lane; c < b; c += 32) sq += cabs2d(__ldcg(G64 + (size_t)r * b + c));
-      sq = warp_sum(sq);
-      if (lane == 0) sig64[r] = sqrt(sq);
+      cl.sync();
     }
-    __syncthreads();
   }
-  for (int a = tid; a < b; a += blockDim.x) {       // a total order, non-finite norms last
-    const double s = sig64[a];
-    sig[a] = s >= 0.0 && isfinite(s) ? s : -1.0;
+  // row norms and the selection in double (CTA 0), rows written back
+  for (int t = warp; t < rpc; t += nw) {
+    const int row = cr + cs * t;
+    if (row >= b) continue;
+    double sq = 0.0;
+    for (int c = lane; c < b; c += 32) sq += cabs2d(G[(size_t)t * b + c]);
+    sq = warp_sum(sq);
+    if (lane == 0) __stcg(sig64 + row, sqrt(sq));
   }
-  for (int a = tid; a < k; a += blockDim.x) top[a] = 0;
-  __syncthreads();
-  for (int a = tid; a < b; a += blockDim.x) {
-    const double sa = sig[a];
+  for (int e = threadIdx.x; e < rpc * b; e += blockDim.x) {
+    const int t = e / b, c = e % b, r = cr + cs * t;
+    if (r < b) G64[(size_t)r * b + c] = G[e];
+  }
+  cl.sync();                                  // sig64 complete; no remote reads after this
+  if (cr != 0) return;
+  for (int a = threadIdx.x; a < b; a += blockDim.x) {   // total order, non-finite norms last
+    double sa = __ldcg(sig64 + a);
+    if (!(sa >= 0.0) || !isfinite(sa)) sa = -1.0;
     int rank = 0;
-    for (int c = 0; c < b; ++c) rank += sig[c] > sa || (sig[c] == sa && c < a);
-    if (rank < k) top[rank] = a;
-  }
-  __syncthreads();
-#pragma unroll 4
-  for (int e = tid; e < k * b; e += blockDim.x) {
-    const int a = top[e / b], c = e % b;
-    const double2 w = __ldcg(WH64 + (size_t)a * b + c), g = __ldcg(G64 + (size_t)a * b + c);
-    Wt[e] = make_float2((float)w.x, (float)w.y);
-    Gt[e] = make_float2((float)g.x, (float)g.y);
+    for (int c = 0; c < b; ++c) {
+      double sc = __ldcg(sig64 + c);
+      if (!(sc >= 0.0) || !isfinite(sc)) sc = -1.0;
+      rank += (sc > sa) || (sc == sa && c < a);
+    }
+    if (rank < k) idx64[rank] = a;
   }
 }
 
-// The kept rows of WH and G' of the reduced SVD, in order (complex128), for
-// U = Q WH[top]^H (m x k) and Rem = G'[top] W^H (k x n).
+// The kept rows of WH and G' of the reduced SVD, in order and in the path's
+// element type, for U = Q WH[top]^H (m x k) and Rem = G'[top] W^H (k x n).
+// (complex64: the complex128 factors are rounded once; products in FP64 would
+// cost 64 times the FP32 rate and add nothing to what Q and W carry.)
 template <typename C>
-__global__ void k_gather_top(const C* __restrict__ WH, const C* __restrict__ G, const int* __restrict__ idx, int k,
-                             int b, C* __restrict__ Wt, C* __restrict__ Gt) {
+__global__ void k_gather_top(const double2* __restrict__ WH, const double2* __restrict__ G,
+                             const int* __restrict__ idx, int k, int b, C* __restrict__ Wt, C* __restrict__ Gt) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < k * b; e += gridDim.x * blockDim.x) {
     const int a = min(max(idx[e / b], 0), b - 1), c = e % b;
-    Wt[e] = WH[a * b + c];
-    Gt[e] = G[a * b + c];
+    Wt[e] = cx<C>(WH[a * b + c].x, WH[a * b + c].y);
+    Gt[e] = cx<C>(G[a * b + c].x, G[a * b + c].y);
   }
 }
 
@@ -1665,12 +1556,9 @@ size_t svd_work_bound_rand64(int max_min, int max_max, int chi) {
                   jacobi_bytes<double2>(jm, max_max) + jacobi_reduce_bytes<double2>(jm, max_max));
 }
 
-// The largest reduced factor of a complex64 truncation: b x b complex128 over
-// sixteen CTAs' shared memory (the rows of the FP64 finish lay there once; the
-// bound on chi that it set is part of the interface).
-static bool cut64_fits(int b) {
-  const size_t rows = (size_t)(b + 15) / 16;
-  return sizeof(double2) * rows * b + sizeof(int) * (size_t)(2 * b + 8) <= (size_t)kSmemMax;
+static size_t cut64_smem(int b, int k) {
+  const size_t rpc = (size_t)(b + kCutCluster - 1) / kCutCluster;
+  return sizeof(double2) * rpc * b + sizeof(int) * (size_t)(2 * b + 8);
 }
 
 // Orthonormalise the columns of Y (rows x b) in place; R (b x b) too when R
@@ -1691,7 +1579,7 @@ static cudaError_t orth_panel(C* Y, int rows, int b, C* R, void* chunk_scratch, 
 // Z^H Q = W R_W, so that B = Q^H Z = R_W^H W^H and the SVD runs on the b x b
 // factor L = R_W^H.  Its one-sided Jacobi gives G' = WH L (rows sigma_i v_i^H
 // in the W basis); U = Q WH[top]^H and Rem = G'[top] W^H.  complex64: the
-// Jacobi runs in complex64 and is finished in complex128 (k_cut_rows);
+// Jacobi runs in complex64 and is finished in complex128 (k_jacobi_cut64);
 // complex128: the Jacobi runs in complex128.
 template <typename C>
 static cudaError_t rand_svd(const C* Z, int m, int n, int chi, int b, C* U, C* Rem, void* work, int* status,
@@ -1699,7 +1587,7 @@ static cudaError_t rand_svd(const C* Z, int m, int n, int chi, int b, C* U, C* R
   const int M = m < n ? m : n;
   const int k = chi < M ? chi : M;
   const bool c64 = sizeof(C) == sizeof(float2);
-  if (c64 && !cut64_fits(b)) return cudaErrorInvalidValue;
+  if (c64 && cut64_smem(b, k) > (size_t)kSmemMax) return cudaErrorInvalidValue;
   const size_t z = sizeof(C), zd = sizeof(double2);
   char* p = (char*)work;
   C* W = (C*)p; p += align256(z * (size_t)n * b);
@@ -1710,7 +1598,7 @@ static cudaError_t rand_svd(const C* Z, int m, int n, int chi, int b, C* U, C* R
   double2* G64 = (double2*)p; p += align256(zd * (size_t)b * b);
   double2* WH64 = (double2*)p; p += align256(zd * (size_t)b * b);
   double* sig64 = (double*)p; p += align256(sizeof(double) * b);
-  p += align256(sizeof(int) * b) + 256;
+  int* idx64 = (int*)p; p += align256(sizeof(int) * b) + 256;
   void* chunk = p; p += orth_scratch_bytes<C>(m, n, b);
   const size_t split_bytes = align256(sizeof(C) * (size_t)kSplitMax * std::max(m, n) * b);
   void* split = p; p += split_bytes;
@@ -1775,11 +1663,21 @@ static cudaError_t rand_svd(const C* Z, int m, int n, int chi, int b, C* U, C* R
   }
   // the kept rows of WH into Rw, of G' into L (k x b)
   if constexpr (sizeof(C) == sizeof(float2)) {
-    int* big = (int*)split;              // (b x b marks; the products are done)
-    k_cut_rows<<<b, kCutThreads, cut_layout(b).bytes, s>>>(w.G, w.WH, w.idx, b, k, w.zn2, G64, WH64, sig64, big,
-                                                          w.counters);
-    k_cut_select<<<1, 1024, (sizeof(double) + sizeof(int)) * (size_t)b, s>>>(G64, WH64, sig64, big, w.counters,
-                                                                                   b, k, w.zn2, Rw, L);
+    if ((e = smem_optin<k_jacobi_cut64>()) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kCutCluster, 1, 1);
+    cfg.blockDim = dim3(std::min(1024, 32 * std::max(1, (b + 1) / 2)), 1, 1);
+    cfg.dynamicSmemBytes = cut64_smem(b, k);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kCutCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if ((e = cudaLaunchKernelEx(&cfg, k_jacobi_cut64, w, b, k, G64, WH64, sig64, idx64)) != cudaSuccess) return e;
+    k_gather_top<C><<<grid_for((long long)k * b, 256), 256, 0, s>>>(WH64, G64, idx64, k, b, Rw, L);
   } else {
     k_gather_top<C><<<grid_for((long long)k * b, 256), 256, 0, s>>>(w.WH, w.G, w.idx, k, b, Rw, L);
   }
@@ -2293,8 +2191,10 @@ cudaError_t init_kernel_attributes() {
   if ((e = smem_optin<k_tsqr_reg<4>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_tsqr_reg<8>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_tsqr_reg<16>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_jacobi_cut64>()) != cudaSuccess) return e;
   for (const void* f : {(const void*)k_msg_normalise<double2>, (const void*)k_msg_normalise<float2>,
-                        (const void*)k_mps_dot<double2>, (const void*)k_mps_dot<float2>})
+                        (const void*)k_mps_dot<double2>, (const void*)k_mps_dot<float2>,
+                        (const void*)k_jacobi_cut64})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
   if ((e = init_panel_attributes()) != cudaSuccess) return e;
   if ((e = init_jac_attributes()) != cudaSuccess) return e;
