@@ -17,11 +17,15 @@
 // GEMM: X^T and S are scaled by a power of two (largest magnitude about 1)
 // and split into limbs of the operand type, and the K dimension concatenates
 // segments that pair a limb of A with a limb of B:
-//   A = [ Re a, -Im a ]  (rows q),  [ Im a, Re a ]  (rows Q + q)  per segment
-//   B = [ Re b ; Im b ]                                           per segment
+//   A = [ Re a, -Im a ]  (rows 2 q),  [ Im a, Re a ]  (rows 2 q + 1)  per segment
+//   B = [ Re b ; Im b ]                                               per segment
 // TF32: limbs hi, lo and the segments hi*hi, hi*lo, lo*hi; BF16 (8 bits a
 // limb): limbs h, m, l and the segments hh, hm, mh, hl, mm, lh.  Both
-// accumulate in FP32 in one pass to about FP32 accuracy.
+// accumulate in FP32 in one pass to about FP32 accuracy.  The sums run over
+// the segments as one K dimension, one MMA (32 bytes of K) after the other:
+// which entries share an MMA is part of the result.  Where a segment is whole
+// MMAs, each limb is stored once and read as often as it occurs; else a row
+// holds every segment (kOnce).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -473,18 +477,25 @@ __device__ __forceinline__ float limb(float x, int which) {
   return O::round(r1 - m);
 }
 
-// Operands of the absorb contraction.  A row holds, limb after limb, a segment
-// of `pitch` entries: [Re block of P | Im block of P | zeros], the pitch a
-// whole number of pipeline stages (128 bytes).  Each limb is stored once.  A 32
-// x 32 tile of the source is read along its rows and written transposed.
-//
+// Operands of the absorb contraction: rows of `row` entries.  kOnce: limb after
+// limb, `pitch` entries each, [Re block of P | Im block of P | zeros], the
+// pitch a whole number of pipeline stages (128 bytes).  Else segment after
+// segment without gaps (pitch = 2 P), zeros at the row's end.  A 32 x 32 tile of
+// the source is read along its rows and written transposed.
+template <bool kBF16, bool kOnce> constexpr int kCopies = kOnce ? Split<kBF16>::kLimbs : Split<kBF16>::kSegs;
+template <bool kBF16>
+__device__ __forceinline__ void limbs(float x, float (&v)[3]) {
+#pragma unroll
+  for (int w = 0; w < Split<kBF16>::kLimbs; ++w) v[w] = limb<kBF16>(x, w);
+}
 // A from X (P x Q complex, row-major): row 2 q holds [Re, -Im] of column q,
 // row 2 q + 1 [Im, Re].
-template <bool kBF16, typename C>
+template <bool kBF16, bool kOnce, typename C>
 __global__ void __launch_bounds__(256) k_pack_a(const C* __restrict__ X, int P, int Q, const int* amax,
-                                                typename Op<kBF16>::T* __restrict__ A, int pitch) {
+                                                typename Op<kBF16>::T* __restrict__ A, int pitch, int row) {
   using O = Op<kBF16>;
-  constexpr int NL = Split<kBF16>::kLimbs;
+  using Sp = Split<kBF16>;
+  constexpr int NC = kCopies<kBF16, kOnce>;
   __shared__ float2 tile[32][33];
   const float sc = pow2_scale(amax);
   const int q0 = blockIdx.x * 32;
@@ -507,31 +518,37 @@ __global__ void __launch_bounds__(256) k_pack_a(const C* __restrict__ X, int P, 
 #pragma unroll
     for (int i = ty; i < 32; i += 8) {
       if (q0 + i >= Q) break;
-      typename O::T* re = A + (long long)(2 * (q0 + i)) * NL * pitch;
-      typename O::T* im = re + (long long)NL * pitch;
+      typename O::T* re = A + (long long)(2 * (q0 + i)) * row;
+      typename O::T* im = re + row;
       const float2 z = tile[tx][i];
+      float xr[3], xi[3];
+      limbs<kBF16>(z.x, xr);
+      limbs<kBF16>(z.y, xi);
 #pragma unroll
-      for (int w = 0; w < NL; ++w) {
+      for (int w = 0; w < NC; ++w) {
+        const int l = kOnce ? w : Sp::limb_a(w);
         if (p < P) {
-          const float xr = limb<kBF16>(z.x, w), xi = limb<kBF16>(z.y, w);
-          re[w * pitch + p] = O::store(xr);
-          re[w * pitch + P + p] = O::store(-xi);
-          im[w * pitch + p] = O::store(xi);
-          im[w * pitch + P + p] = O::store(xr);
+          re[w * pitch + p] = O::store(xr[l]);
+          re[w * pitch + P + p] = O::store(-xi[l]);
+          im[w * pitch + p] = O::store(xi[l]);
+          im[w * pitch + P + p] = O::store(xr[l]);
         }
-        if (last)
+        if (last && kOnce)
           for (int k = 2 * P + tx; k < pitch; k += 32) re[w * pitch + k] = im[w * pitch + k] = O::store(0.f);
       }
+      if (last && !kOnce)
+        for (int k = NC * pitch + tx; k < row; k += 32) re[k] = im[k] = O::store(0.f);
     }
   }
 }
 
 // B^T from S (l x P x r complex): row n = a r + c holds [Re, Im] of (a, ., c).
-template <bool kBF16, typename C>
+template <bool kBF16, bool kOnce, typename C>
 __global__ void __launch_bounds__(256) k_pack_b(const C* __restrict__ S, int P, int r, const int* amax,
-                                                typename Op<kBF16>::T* __restrict__ B, int pitch) {
+                                                typename Op<kBF16>::T* __restrict__ B, int pitch, int row) {
   using O = Op<kBF16>;
-  constexpr int NL = Split<kBF16>::kLimbs;
+  using Sp = Split<kBF16>;
+  constexpr int NC = kCopies<kBF16, kOnce>;
   __shared__ float2 tile[32][33];
   const float sc = pow2_scale(amax);
   const int ct = (r + 31) / 32, a = blockIdx.x / ct, c0 = (blockIdx.x % ct) * 32;
@@ -554,17 +571,23 @@ __global__ void __launch_bounds__(256) k_pack_b(const C* __restrict__ S, int P, 
 #pragma unroll
     for (int i = ty; i < 32; i += 8) {
       if (c0 + i >= r) break;
-      typename O::T* row = B + ((long long)a * r + c0 + i) * NL * pitch;
+      typename O::T* out = B + ((long long)a * r + c0 + i) * row;
       const float2 z = tile[tx][i];
+      float xr[3], xi[3];
+      limbs<kBF16>(z.x, xr);
+      limbs<kBF16>(z.y, xi);
 #pragma unroll
-      for (int w = 0; w < NL; ++w) {
+      for (int w = 0; w < NC; ++w) {
+        const int l = kOnce ? w : Sp::limb_b(w);
         if (p < P) {
-          row[w * pitch + p] = O::store(limb<kBF16>(z.x, w));
-          row[w * pitch + P + p] = O::store(limb<kBF16>(z.y, w));
+          out[w * pitch + p] = O::store(xr[l]);
+          out[w * pitch + P + p] = O::store(xi[l]);
         }
-        if (last)
-          for (int k = 2 * P + tx; k < pitch; k += 32) row[w * pitch + k] = O::store(0.f);
+        if (last && kOnce)
+          for (int k = 2 * P + tx; k < pitch; k += 32) out[w * pitch + k] = O::store(0.f);
       }
+      if (last && !kOnce)
+        for (int k = NC * pitch + tx; k < row; k += 32) out[k] = O::store(0.f);
     }
   }
 }
@@ -946,10 +969,20 @@ cudaError_t launch_tc_gemm(bool bf16, const void* A, long long lda, const void* 
 }
 
 long long tc_ld(int P) { return ((6LL * P + 31) / 32) * 32; }
-// columns of one limb of the absorb operands: 2 P reals in whole 128-byte stages
-int tc_absorb_pitch(bool bf16, int P) {
-  const int ke = bf16 ? 64 : 32;
-  return (2 * P + ke - 1) / ke * ke;
+// A row of the absorb operands: kOnce of the packing, entries from copy to copy
+// and of the whole row, and the K dimension of the product (all segments).
+struct AbsorbRow {
+  bool once;
+  int pitch, row, K;
+};
+static AbsorbRow absorb_row(bool bf16, int P) {
+  const int es = bf16 ? 2 : 4, ke = 128 / es, segs = bf16 ? 6 : 3, limbs = bf16 ? 3 : 2;
+  AbsorbRow a;
+  a.once = (2 * P * es) % 32 == 0;
+  a.pitch = a.once ? (2 * P + ke - 1) / ke * ke : 2 * P;
+  a.K = (segs * 2 * P + 31) / 32 * 32;
+  a.row = a.once ? limbs * a.pitch : a.K;
+  return a;
 }
 
 // ------------------------------------------------ general complex GEMM (c64)
@@ -998,31 +1031,28 @@ cudaError_t tc_zgemm_packed(bool bf16, int M, int N, int K, const void* Ap, cons
 // operands; or the operands as they are, where their padding takes more)
 size_t tc_absorb_bytes(bool bf16, int P, int Q, int l, int r) {
   const size_t es = bf16 ? 2 : 4;
-  const size_t ld = ((2 * (size_t)(bf16 ? 6 : 3) * P + 31) / 32) * 32;
-  const size_t row = (size_t)(bf16 ? 3 : 2) * tc_absorb_pitch(bf16, P) * es;
+  const AbsorbRow a = absorb_row(bf16, P);
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  return std::max(al(2 * (size_t)Q * ld * es) + al((size_t)l * r * ld * es) + al(sizeof(float) * 2 * (size_t)Q * l * r),
-                  al(2 * (size_t)Q * row) + al((size_t)l * r * row)) +
-         256;
+  auto operands = [&](size_t row) { return al(2 * (size_t)Q * row * es) + al((size_t)l * r * row * es); };
+  return std::max(operands(a.K) + al(sizeof(float) * 2 * (size_t)Q * l * r), operands(a.row)) + 256;
 }
 
 // Largest magnitudes, the two packed operands, and one product whose epilogue
 // writes R.  At P = Q = 1296, l = r = 64: the limbs stored once are 85 MB of B
 // and 54 MB of A (each segment's copy took 127 and 81 MB, and the real product
 // another 42 MB written, read and written again as R).
-template <bool kBF16, typename C>
+template <bool kBF16, bool kOnce, typename C>
 static cudaError_t tc_absorb_t(const C* X, int P, int Q, const C* S, int l, int r, C* R, void* work, int* err,
-                               cudaStream_t s) {
+                               cudaStream_t s, const AbsorbRow& w) {
   using T = typename Op<kBF16>::T;
   using Sp = Split<kBF16>;
-  const int pitch = tc_absorb_pitch(kBF16, P), ke = 128 / (int)sizeof(T);
-  const size_t row = (size_t)Sp::kLimbs * pitch * sizeof(T);
+  constexpr int ke = 128 / (int)sizeof(T), EPI = sizeof(C) == sizeof(float2) ? 1 : 2;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   char* p = (char*)work;
   T* A = (T*)p;
-  p += al(2 * (size_t)Q * row);
+  p += al(2 * (size_t)Q * w.row * sizeof(T));
   T* B = (T*)p;
-  p += al((size_t)l * r * row);
+  p += al((size_t)l * r * w.row * sizeof(T));
   int* amax = (int*)p;   // [0] X, [1] S
   cudaError_t e;
   if ((e = cudaMemsetAsync(amax, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
@@ -1031,24 +1061,33 @@ static cudaError_t tc_absorb_t(const C* X, int P, int Q, const C* S, int l, int 
   const long long nx = (long long)P * Q, ns = (long long)l * P * r;
   k_absmax<C><<<ctas(nx) + ctas(ns), 256, 0, s>>>(X, nx, ctas(nx), S, ns, amax);
   const unsigned pt = std::min((P + 31) / 32, 65535);
-  k_pack_a<kBF16, C><<<dim3((Q + 31) / 32, pt), 256, 0, s>>>(X, P, Q, amax, A, pitch);
-  k_pack_b<kBF16, C><<<dim3((unsigned)l * ((r + 31) / 32), pt), 256, 0, s>>>(S, P, r, amax + 1, B, pitch);
-  const int N = l * r, M = 2 * Q, Kt = Sp::kSegs * pitch;
-  const TcTile t = tile_of(kBF16, M, N, Kt);
-  const TcK ks = {Sp::kSegs, pitch / ke, pitch};
+  k_pack_a<kBF16, kOnce, C><<<dim3((Q + 31) / 32, pt), 256, 0, s>>>(X, P, Q, amax, A, w.pitch, w.row);
+  k_pack_b<kBF16, kOnce, C><<<dim3((unsigned)l * ((r + 31) / 32), pt), 256, 0, s>>>(S, P, r, amax + 1, B, w.pitch, w.row);
+  const int N = l * r, M = 2 * Q;
+  const TcTile t = tile_of(kBF16, M, N, w.K);
+  const TcK ks = kOnce ? TcK{Sp::kSegs, w.pitch / ke, w.pitch} : TcK{1, (w.row + ke - 1) / ke, 0};
   const TcOut out = {R, Q, r, r % 4 == 0 && ((uintptr_t)R & 15) == 0 ? 1 : 0, amax, amax + 1};
-  constexpr int EPI = sizeof(C) == sizeof(float2) ? 1 : 2;
-  return tc_dispatch<EPI>(kBF16, A, Sp::kLimbs * pitch, B, Sp::kLimbs * pitch, nullptr, 0, M, N, Sp::kLimbs * pitch,
-                          1.0f, err, s, t.bn, t.group_m, 8.0 * Q * N * (double)P, ks, out);
+  return tc_dispatch<EPI>(kBF16, A, w.row, B, w.row, nullptr, 0, M, N, w.row, 1.0f, err, s, t.bn, t.group_m,
+                          8.0 * Q * N * (double)P, ks, out);
+}
+template <typename C>
+static cudaError_t tc_absorb(bool bf16, const C* X, int P, int Q, const C* S, int l, int r, C* R, void* work, int* err,
+                             cudaStream_t s) {
+  const AbsorbRow w = absorb_row(bf16, P);
+  if (bf16)
+    return w.once ? tc_absorb_t<true, true>(X, P, Q, S, l, r, R, work, err, s, w)
+                  : tc_absorb_t<true, false>(X, P, Q, S, l, r, R, work, err, s, w);
+  return w.once ? tc_absorb_t<false, true>(X, P, Q, S, l, r, R, work, err, s, w)
+                : tc_absorb_t<false, false>(X, P, Q, S, l, r, R, work, err, s, w);
 }
 
 cudaError_t launch_tc_absorb(bool bf16, const double2* X, int P, int Q, const double2* S, int l, int r, double2* R,
                              void* work, int* err, cudaStream_t s) {
-  return bf16 ? tc_absorb_t<true>(X, P, Q, S, l, r, R, work, err, s) : tc_absorb_t<false>(X, P, Q, S, l, r, R, work, err, s);
+  return tc_absorb(bf16, X, P, Q, S, l, r, R, work, err, s);
 }
 cudaError_t launch_tc_absorb(bool bf16, const float2* X, int P, int Q, const float2* S, int l, int r, float2* R,
                              void* work, int* err, cudaStream_t s) {
-  return bf16 ? tc_absorb_t<true>(X, P, Q, S, l, r, R, work, err, s) : tc_absorb_t<false>(X, P, Q, S, l, r, R, work, err, s);
+  return tc_absorb(bf16, X, P, Q, S, l, r, R, work, err, s);
 }
 
 }  // namespace bbp
