@@ -1718,61 +1718,87 @@ cudaError_t svd_stats(const void* work, int m, int n, int* sweeps, long long* ro
 // --------------------------------------------------------------- normalise
 
 namespace {
-// Up to 32768 entries, held in registers between the sum and the scaling: one
-// CTA up to 2048, a cluster of eight above (sums exchanged through distributed
-// shared memory, added in rank order).  One CTA of 1024 threads read them twice
-// and took all the FP64 sums on one SM: 15.5 us at some 20000 entries and 11.2
-// at a few hundred (with the logarithm), against 10.7 and 8.8 without it.
-constexpr int kNormCluster = 8, kNormThreads = 256, kNormPer = 16;
+// Up to 32768 entries, held in registers between the sum and the scaling: 1024
+// partial sums (entries t, t + 1024, ...) and one tree over the lanes of their
+// 32 warps, then over the warps - the order of one CTA of 1024 threads, which
+// the results keep - on one CTA of 256 threads (four partial sums a thread, one
+// tree for the four) or, above 2048 entries, a cluster of eight CTAs of 128.
+// One thread takes the root and the quotient; the logarithm is left out where
+// nobody reads it.  One CTA read the entries twice and took every thread's root
+// and quotient on one SM's FP64 unit.
+constexpr int kNormSums = 1024, kNormCluster = 8, kNormMax = 32768;
 template <typename C, bool CL>
-__global__ void __launch_bounds__(kNormThreads) k_normalise(C* A, int n, double* logscale) {   // logscale may be null
-  __shared__ double sh[40], mine;
+__global__ void __launch_bounds__(CL ? kNormSums / kNormCluster : 256) k_normalise(C* A, int n,
+                                                                                  double* logscale) {   // may be null
+  constexpr int NT = CL ? kNormSums / kNormCluster : 256, V = CL ? 1 : kNormSums / NT;   // sums a thread
+  constexpr int E = CL ? kNormMax / kNormSums : 2;                                       // entries a sum
+  __shared__ double sh[32], s_inv;
   cg::cluster_group cl = cg::this_cluster();
-  const int cr = CL ? (int)cl.block_rank() : 0, step = (CL ? kNormCluster : 1) * kNormThreads;
-  C v[kNormPer];
-  double part = 0.0;
+  const int cr = CL ? (int)cl.block_rank() : 0, t0 = cr * NT + threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  C v[V][E];
+  double part[V];
 #pragma unroll
-  for (int e = 0; e < kNormPer; ++e) {
-    const int i = cr * kNormThreads + threadIdx.x + e * step;
-    if (i < n) {
-      v[e] = A[i];
-      part += cabs2d(v[e]);
+  for (int u = 0; u < V; ++u) {
+    part[u] = 0.0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = t0 + u * NT + e * kNormSums;
+      if (i < n) v[u][e] = A[i];
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (t0 + u * NT + e * kNormSums < n) part[u] += cabs2d(v[u][e]);
+  }
+  if constexpr (CL) {
+    const double s = warp_sum(part[0]);
+    if (lane == 0) sh[warp] = s;
+  } else {                               // lane L: sum u = L >> 3 of the warp's four
+    const bool up = lane & 16, odd = lane & 8;
+    const double a = (up ? part[1] : part[0]) + __shfl_xor_sync(0xffffffffu, up ? part[0] : part[1], 16);
+    const double b = (up ? part[3] : part[2]) + __shfl_xor_sync(0xffffffffu, up ? part[2] : part[3], 16);
+    double s = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if ((lane & 7) == 0) sh[warp + (NT / 32) * ((up ? 1 : 0) + (odd ? 2 : 0))] = s;   // (warp of entry t0 + u NT)
+  }
+  if constexpr (CL) cl.sync();
+  else __syncthreads();
+  if (warp == 0) {
+    double s;
+    if constexpr (CL) s = cl.map_shared_rank(sh, lane >> 2)[lane & 3];
+    else s = sh[lane];
+    s = warp_sum(s);
+    const double nrm = sqrt(s);
+    if (lane == 0) s_inv = nrm > 0.0 ? 1.0 / nrm : -1.0;
+    if (logscale && cr == 0 && lane == 0) {
+      if (nrm > 0.0) *logscale += log(nrm);
+      else *logscale = -INFINITY;
     }
   }
-  double s = block_sum(part, sh);
-  if constexpr (CL) {
-    if (threadIdx.x == 0) mine = s;
-    cl.sync();
-    s = 0.0;
-    for (int q = 0; q < kNormCluster; ++q) s += *cl.map_shared_rank(&mine, q);
-    cl.sync();                           // every CTA's sum is read: none leaves or reuses it before
-  }
-  // one thread's square root and division, another's logarithm beside them
-  // (in every thread they would take the SM's FP64 units for microseconds)
-  if (threadIdx.x == 0) mine = s > 0.0 ? rsqrt(s) : 0.0;
-  if (logscale && cr == 0 && threadIdx.x == 32) {
-    if (s > 0.0) *logscale += 0.5 * log(s);
-    else *logscale = -INFINITY;
-  }
-  __syncthreads();
-  const double inv = mine;
-  if (inv == 0.0) return;
+  if constexpr (CL) cl.sync();           // every CTA's sums are read: none leaves before
+  else __syncthreads();
+  const double inv = s_inv;
+  if (inv < 0.0) return;                 // (zero or NaN norm)
 #pragma unroll
-  for (int e = 0; e < kNormPer; ++e) {
-    const int i = cr * kNormThreads + threadIdx.x + e * step;
-    if (i < n) A[i] = cscale(v[e], inv);
-  }
+  for (int u = 0; u < V; ++u)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = t0 + u * NT + e * kNormSums;
+      if (i < n) A[i] = cscale(v[u][e], inv);
+    }
 }
 
 template <typename C>
 cudaError_t normalise_small(C* A, int n, double* logscale, cudaStream_t s) {
-  if (n <= 2048) {
-    k_normalise<C, false><<<1, kNormThreads, 0, s>>>(A, n, logscale);
+  if (n <= 2 * kNormSums) {
+    k_normalise<C, false><<<1, 256, 0, s>>>(A, n, logscale);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kNormCluster, 1, 1);
-  cfg.blockDim = dim3(kNormThreads, 1, 1);
+  cfg.blockDim = dim3(kNormSums / kNormCluster, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2092,7 +2118,7 @@ __global__ void __launch_bounds__(256) k_mps_dot(ChainDesc A, ChainDesc B, doubl
 
 #define BBP_INSTANTIATE(C)                                                                                          \
   cudaError_t launch_normalise(C* A, long long n, double* logscale, bool want_log, cudaStream_t s) {               \
-    if (n <= kNormCluster * kNormThreads * kNormPer)                                                               \
+    if (n <= kNormMax)                                                               \
       return normalise_small(A, (int)n, want_log ? logscale : nullptr, s);                                         \
     /* logscale[1]: the accumulator of the many-CTA form */                                                        \
     cudaError_t e = cudaMemsetAsync(logscale + 1, 0, sizeof(double), s);                                          \
