@@ -1132,8 +1132,8 @@ cudaError_t jacobi_svd(const C* Z, int m, int n, int chi, C* U, C* Rem, void* wo
       tall = GH;
     }
     if ((e = launch_panel_qr(tall, N, M, QT, RT, 1, 0, s)) != cudaSuccess) return e;
-    // L = R_T^H rotated into LR = WH L, its row norms, their order and ||Z||^2
-    if ((e = launch_jac(RT, M, true, M, M, k, LR, w.WH, w.sigma, w.idx, w.zn2, w.counters, 0, 0, (C*)nullptr,
+    // L = R_T^H rotated into LR = WH L, and ||Z||^2
+    if ((e = launch_jac(RT, M, true, M, M, k, LR, w.WH, nullptr, nullptr, w.zn2, w.counters, 0, 0, (C*)nullptr,
                         (C*)nullptr, tol, floor_rel_of<C>(), max_sweeps, status, s)) != cudaSuccess)
       return e;
     // rotated rows of G: (WH L) Q_T^H (M x N)
@@ -1147,9 +1147,10 @@ cudaError_t jacobi_svd(const C* Z, int m, int n, int chi, C* U, C* Rem, void* wo
     if ((e = cudaMemsetAsync(w.counters, 0, 64, s)) != cudaSuccess) return e;
     k_svd_init<C><<<grid_for((long long)M * N + (long long)M * M, 256), 256, 0, s>>>(Z, m, n, w);
     if ((e = launch_jacobi(w, M, N, tol, max_sweeps, status, s)) != cudaSuccess) return e;
-    k_row_norms<C><<<(M * 32 + 255) / 256, 256, 0, s>>>(w, M, N);
-    k_select<C><<<1, 256, 0, s>>>(w, M, k);
   }
+  // (the singular values are the norms of the rotated rows of G, not of LR)
+  k_row_norms<C><<<(M * 32 + 255) / 256, 256, 0, s>>>(w, M, N);
+  k_select<C><<<1, 256, 0, s>>>(w, M, k);
   k_svd_out<C><<<grid_for((long long)m * k + (long long)k * n, 256), 256, 0, s>>>(w, m, n, k, floor_rel_of<C>(), U,
                                                                                  Rem);
   return cudaGetLastError();
