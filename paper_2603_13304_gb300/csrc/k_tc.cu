@@ -191,17 +191,20 @@ struct TcOut {
   int Q, r, vec;
   const int *amax_a, *amax_b;
 };
-template <typename C2> __device__ __forceinline__ void store_pair(C2* p, float x0, float y0, float x1, float y1);
-template <> __device__ __forceinline__ void store_pair(float2* p, float x0, float y0, float x1, float y1) {
+// (complex128: times s; complex64 entries are scaled before)
+template <typename C2> __device__ __forceinline__ void store_pair(C2* p, float x0, float y0, float x1, float y1, double s);
+template <> __device__ __forceinline__ void store_pair(float2* p, float x0, float y0, float x1, float y1, double) {
   *reinterpret_cast<float4*>(p) = make_float4(x0, y0, x1, y1);
 }
-template <> __device__ __forceinline__ void store_pair(double2* p, float x0, float y0, float x1, float y1) {
-  p[0] = make_double2(x0, y0);
-  p[1] = make_double2(x1, y1);
+template <> __device__ __forceinline__ void store_pair(double2* p, float x0, float y0, float x1, float y1, double s) {
+  p[0] = make_double2(x0 * s, y0 * s);
+  p[1] = make_double2(x1 * s, y1 * s);
 }
-template <typename C2> __device__ __forceinline__ void store_one(C2* p, float x, float y);
-template <> __device__ __forceinline__ void store_one(float2* p, float x, float y) { *p = make_float2(x, y); }
-template <> __device__ __forceinline__ void store_one(double2* p, float x, float y) { *p = make_double2(x, y); }
+template <typename C2> __device__ __forceinline__ void store_one(C2* p, float x, float y, double s);
+template <> __device__ __forceinline__ void store_one(float2* p, float x, float y, double) { *p = make_float2(x, y); }
+template <> __device__ __forceinline__ void store_one(double2* p, float x, float y, double s) {
+  *p = make_double2(x * s, y * s);
+}
 
 // EPI: 0 the real product (C = alpha A B^T), 1 complex64 entries of R, 2
 // complex128 ones (straight from TMEM: no real product in memory).
@@ -314,8 +317,10 @@ __global__ void __launch_bounds__(128, 1)
     const bool odd = lane & 1;
     const int q = row >> 1, r = out_c.r;
     const int ex = -(scale_exp(out_c.amax_a) + scale_exp(out_c.amax_b));
-    const bool plain = ex > -120 && ex < 120;
+    // (complex128 entries are scaled in double: they reach past float's range)
+    const bool plain = EPI == 1 && ex > -120 && ex < 120;
     const float inv = plain ? exp2f((float)ex) : 1.f;
+    const double inv2 = EPI == 2 ? ldexp(1.0, ex) : 1.0;
 #pragma unroll 1
     for (int c0 = 0; c0 < BN && n0 + c0 < N; c0 += 32) {
       uint32_t v[32];
@@ -327,7 +332,7 @@ __global__ void __launch_bounds__(128, 1)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           x[u] = __uint_as_float(v[j + u]);
-          x[u] = plain ? x[u] * inv : ldexpf(x[u], ex);
+          if constexpr (EPI == 1) x[u] = plain ? x[u] * inv : ldexpf(x[u], ex);
         }
         const float ra = __shfl_xor_sync(0xffffffffu, odd ? x[0] : x[2], 1);
         const float rb = __shfl_xor_sync(0xffffffffu, odd ? x[1] : x[3], 1);
@@ -335,10 +340,11 @@ __global__ void __launch_bounds__(128, 1)
         if (row < M) {
           C2* p = R + ((long long)a * out_c.Q + q) * r + c;
           if (out_c.vec) {
-            if (n < N) store_pair(p, re0, im0, re1, im1);
+            if (n < N) store_pair(p, re0, im0, re1, im1, inv2);
           } else {
-            if (n < N) store_one(p, re0, im0);
-            if (n + 1 < N) store_one(c + 1 < r ? p + 1 : R + ((long long)(a + 1) * out_c.Q + q) * r, re1, im1);
+            if (n < N) store_one(p, re0, im0, inv2);
+            if (n + 1 < N) store_one(c + 1 < r ? p + 1 : R + ((long long)(a + 1) * out_c.Q + q) * r, re1, im1,
+                                        inv2);
           }
         }
         n += 4;
