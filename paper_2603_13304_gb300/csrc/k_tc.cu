@@ -774,20 +774,28 @@ cudaError_t launch_tc_gemm_tile(bool bf16, const void* A, long long lda, const v
 //
 // The tile of a launch (BN, the width of a CTA's output tile, and group_m,
 // the M tiles a wave sweeps together) is looked up by the exact GEMM shape
-// (precision, M, N, K); shapes not in the table take the size rule
-// (rule_tile; group_m 16).  While recording is on, unknown shapes
-// are collected; tc_autotune times every candidate tile of each collected
-// shape on scratch operands (CUDA events, outside any capture) and keeps
-// the fastest.  The table can be written to and read from a text cache.
+// (precision, M, N, K, and the form of the launch: a real product, or an
+// absorb's, whose operand rows and epilogue differ); shapes not in the table
+// take the size rule (rule_tile; group_m 16).  While recording is on, unknown
+// shapes are collected; tc_autotune times every candidate tile of each
+// collected shape, in its form, on scratch operands (CUDA events, outside any
+// capture) and keeps the fastest.  The table can be written to and read from a
+// text cache; an absorb without an entry of its own takes that of the real
+// product of its shape (the only form that earlier caches hold).
 namespace {
 
+// forms: 0 a real product; an absorb into complex64 (1) or complex128 (2), its
+// operand rows holding every segment; the same with each limb stored once
+constexpr int kFormOnce = 2;
+
 struct TcKey {
-  int bf16, M, N, K;
+  int bf16, M, N, K, form;
   bool operator<(const TcKey& o) const {
     if (bf16 != o.bf16) return bf16 < o.bf16;
     if (M != o.M) return M < o.M;
     if (N != o.N) return N < o.N;
-    return K < o.K;
+    if (K != o.K) return K < o.K;
+    return form < o.form;
   }
 };
 struct TcTile {
@@ -822,10 +830,10 @@ TcTile rule_tile(int M, int N) {
 bool write_cache(const char* path) {
   FILE* f = std::fopen(path, "w");
   if (!f) return false;
-  std::fprintf(f, "# bbp tensor-core GEMM tiles: tc bf16 M N K bn group_m microseconds\n");
+  std::fprintf(f, "# bbp tensor-core GEMM tiles: tc bf16 M N K bn group_m microseconds form\n");
   for (const auto& kv : g_tiles)
-    std::fprintf(f, "tc %d %d %d %d %d %d %.3f\n", kv.first.bf16, kv.first.M, kv.first.N, kv.first.K, kv.second.bn,
-                 kv.second.group_m, kv.second.us);
+    std::fprintf(f, "tc %d %d %d %d %d %d %.3f %d\n", kv.first.bf16, kv.first.M, kv.first.N, kv.first.K, kv.second.bn,
+                 kv.second.group_m, kv.second.us, kv.first.form);
   return std::fclose(f) == 0;
 }
 
@@ -865,15 +873,19 @@ cudaError_t tc_autotune(const char* cache_path, int* tuned) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   int* err = nullptr;
-  cudaMalloc(&err, sizeof(int));
+  cudaMalloc(&err, 3 * sizeof(int));     // the error word, and an absorb's two magnitudes (zero: scale one)
   int n_done = 0;
   for (const TcKey& k : todo) {
-    const size_t es = k.bf16 ? 2 : 4;
-    const long long ld = ((long long)k.K + 31) / 32 * 32;
-    void *A = nullptr, *B = nullptr;
-    float* C = nullptr;
+    const int es = k.bf16 ? 2 : 4, ke = 128 / es, segs = k.bf16 ? 6 : 3;
+    const bool absorb = k.form > 0, once = k.form > kFormOnce, c128 = absorb && (k.form - 1) % kFormOnce == 1;
+    // stored entries of an operand row (an absorb's limbs once: K is segs times
+    // 2 P, rounded up to 32)
+    const int pitch = once ? (k.K / segs / 8 * 8 + ke - 1) / ke * ke : 0;
+    const long long ld = once ? (long long)(k.bf16 ? 3 : 2) * pitch : ((long long)k.K + 31) / 32 * 32;
+    const TcK ks = once ? TcK{segs, pitch / ke, pitch} : TcK{1, (k.K + ke - 1) / ke, 0};
+    void *A = nullptr, *B = nullptr, *C = nullptr;
     if (cudaMalloc(&A, (size_t)k.M * ld * es) != cudaSuccess || cudaMalloc(&B, (size_t)k.N * ld * es) != cudaSuccess ||
-        cudaMalloc(&C, sizeof(float) * (size_t)k.M * k.N) != cudaSuccess) {
+        cudaMalloc(&C, (c128 ? 8 : 4) * (size_t)k.M * k.N) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(A);
       cudaFree(B);
@@ -882,7 +894,16 @@ cudaError_t tc_autotune(const char* cache_path, int* tuned) {
     }
     cudaMemsetAsync(A, 0, (size_t)k.M * ld * es, s);
     cudaMemsetAsync(B, 0, (size_t)k.N * ld * es, s);
-    cudaMemsetAsync(err, 0, sizeof(int), s);
+    cudaMemsetAsync(err, 0, 3 * sizeof(int), s);
+    // an absorb's output: M / 2 rows, the columns as one row of R (whatever r)
+    const TcOut out = {C, k.M / 2, k.N, k.N % 4 == 0 ? 1 : 0, err + 1, err + 2};
+    auto run = [&](int bn, int gm) {
+      const bool bf = k.bf16 != 0;
+      if (!absorb)
+        return launch_tc_gemm_tile(bf, A, ld, B, ld, (float*)C, k.N, k.M, k.N, k.K, 1.f, err, s, bn, gm, 0.0);
+      return c128 ? tc_dispatch<2>(bf, A, ld, B, ld, nullptr, 0, k.M, k.N, (int)ld, 1.f, err, s, bn, gm, 0.0, ks, out)
+                  : tc_dispatch<1>(bf, A, ld, B, ld, nullptr, 0, k.M, k.N, (int)ld, 1.f, err, s, bn, gm, 0.0, ks, out);
+    };
     TcTile best;
     best.us = 1e30f;
     const int tiles_m = (k.M + kBM - 1) / kBM;
@@ -892,11 +913,9 @@ cudaError_t tc_autotune(const char* cache_path, int* tuned) {
       for (int gm : {1, 8, 16}) {
         // groups of at least tiles_m M tiles all give one group (the same order)
         if ((gm == 16 && tiles_m <= 8) || (gm == 8 && tiles_m <= 1)) continue;
-        if (launch_tc_gemm_tile(k.bf16 != 0, A, ld, B, ld, C, k.N, k.M, k.N, k.K, 1.f, err, s, bn, gm, 0.0) !=
-            cudaSuccess)
-          continue;
+        if (run(bn, gm) != cudaSuccess) continue;
         cudaEventRecord(e0, s);
-        for (int r = 0; r < 3; ++r) launch_tc_gemm_tile(k.bf16 != 0, A, ld, B, ld, C, k.N, k.M, k.N, k.K, 1.f, err, s, bn, gm, 0.0);
+        for (int r = 0; r < 3; ++r) run(bn, gm);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -946,7 +965,10 @@ int tc_autotune_load(const char* cache_path) {
   while (std::fgets(line, sizeof(line), f)) {
     TcKey k;
     TcTile t;
-    if (std::sscanf(line, "tc %d %d %d %d %d %d %f", &k.bf16, &k.M, &k.N, &k.K, &t.bn, &t.group_m, &t.us) != 7) continue;
+    k.form = 0;
+    if (std::sscanf(line, "tc %d %d %d %d %d %d %f %d", &k.bf16, &k.M, &k.N, &k.K, &t.bn, &t.group_m, &t.us, &k.form) < 7)
+      continue;
+    if (k.form < 0 || k.form > 4) continue;
     if ((t.bn != 64 && t.bn != 128 && t.bn != 256) || t.group_m < 1 || k.M < 1 || k.N < 1 || k.K < 1) continue;
     g_tiles[k] = t;
     ++n;
@@ -957,10 +979,12 @@ int tc_autotune_load(const char* cache_path) {
 }
 
 // the tile of a shape: the table's, else the size rule's (recorded on request)
-static TcTile tile_of(bool bf16, int M, int N, int K) {
-  const TcKey key{bf16 ? 1 : 0, M, N, K};
+static TcTile tile_of(bool bf16, int M, int N, int K, int form) {
+  TcKey key{bf16 ? 1 : 0, M, N, K, form};
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tiles.find(key);
+  if (it == g_tiles.end() && form && !g_recording.load(std::memory_order_relaxed))
+    it = g_tiles.find(TcKey{key.bf16, M, N, K, 0});
   if (it != g_tiles.end()) return it->second;
   if (g_recording.load(std::memory_order_relaxed)) g_pending.insert(key);
   return rule_tile(M, N);
@@ -970,7 +994,7 @@ cudaError_t launch_tc_gemm(bool bf16, const void* A, long long lda, const void* 
                            long long ldc, int M, int N, int K, float alpha, int* err, cudaStream_t s,
                            double algo_flops) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  const TcTile t = tile_of(bf16, M, N, K);
+  const TcTile t = tile_of(bf16, M, N, K, 0);
   return launch_tc_gemm_tile(bf16, A, lda, Bt, ldb, C, ldc, M, N, K, alpha, err, s, t.bn, t.group_m, algo_flops);
 }
 
@@ -1070,7 +1094,7 @@ static cudaError_t tc_absorb_t(const C* X, int P, int Q, const C* S, int l, int 
   k_pack_a<kBF16, kOnce, C><<<dim3((Q + 31) / 32, pt), 256, 0, s>>>(X, P, Q, amax, A, w.pitch, w.row);
   k_pack_b<kBF16, kOnce, C><<<dim3((unsigned)l * ((r + 31) / 32), pt), 256, 0, s>>>(S, P, r, amax + 1, B, w.pitch, w.row);
   const int N = l * r, M = 2 * Q;
-  const TcTile t = tile_of(kBF16, M, N, w.K);
+  const TcTile t = tile_of(kBF16, M, N, w.K, kOnce ? kFormOnce + EPI : EPI);
   const TcK ks = kOnce ? TcK{Sp::kSegs, w.pitch / ke, w.pitch} : TcK{1, (w.row + ke - 1) / ke, 0};
   const TcOut out = {R, Q, r, r % 4 == 0 && ((uintptr_t)R & 15) == 0 ? 1 : 0, amax, amax + 1};
   return tc_dispatch<EPI>(kBF16, A, w.row, B, w.row, nullptr, 0, M, N, w.row, 1.0f, err, s, t.bn, t.group_m,
