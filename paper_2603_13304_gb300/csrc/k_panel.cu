@@ -12,8 +12,8 @@
 // those raw sums and row j, so one cluster-wide exchange per column
 // suffices.  The exchange is pushed: every CTA stores its partial sums (and
 // the owner of row j stores row j) straight into every CTA's receive buffer
-// in distributed shared memory before the cluster barrier, so that after it
-// every CTA reads only its own shared memory and forms the same reflector
+// in distributed shared memory, completing on that CTA's mbarrier, so that
+// every CTA then reads only its own shared memory and forms the same reflector
 // from the same values in the same order (bitwise identical in every CTA).
 // Q = H_0 ... H_{k-1} [I; 0] is then formed in place backwards with one
 // exchange per reflector.
@@ -31,6 +31,7 @@
 #include <initializer_list>
 
 #include "kernels.h"
+#include "push.h"
 
 namespace cg = cooperative_groups;
 
@@ -60,6 +61,15 @@ template <typename C> __device__ __forceinline__ C pmulc(C a, C b) {   // conj(a
   r.x = a.x * b.x + a.y * b.y;
   r.y = a.x * b.y - a.y * b.x;
   return r;
+}
+// the same rounded as written, wherever they are inlined (which product of the
+// imaginary part is rounded by itself: one way with one row a lane, the other
+// with more)
+template <int MAXR, typename C> __device__ __forceinline__ C fmul(C a, C b) {
+  return mkc<C>(fma(a.x, b.x, -(a.y * b.y)), MAXR == 1 ? fma(a.y, b.x, a.x * b.y) : fma(a.x, b.y, a.y * b.x));
+}
+template <typename C> __device__ __forceinline__ C fmulc(C a, C b) {   // conj(a) b
+  return mkc<C>(fma(a.x, b.x, a.y * b.y), fma(a.x, b.y, -(a.y * b.x)));
 }
 template <typename C> __device__ __forceinline__ C padd(C a, C b) { a.x += b.x; a.y += b.y; return a; }
 template <typename C> __device__ __forceinline__ C psub(C a, C b) { a.x -= b.x; a.y -= b.y; return a; }
@@ -100,40 +110,27 @@ __device__ __forceinline__ double2 pick(const double2 (&y)[MAXR], int q) {
 
 constexpr int kPanelThreads = 512;
 constexpr int kPanelSmemMax = 227 * 1024;
+constexpr int kPanelWork = kPanelThreads / 32 - 1;   // warps that work on columns
+constexpr int kPanelExtra = 48 + 10 * 16;            // bytes behind the layout: barriers, the last reflectors
 constexpr int kQBlock = 8;               // reflectors a block of the Q formation
-
-// distributed shared memory through 32-bit shared-window addresses
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t dsmem_addr(uint32_t a, int rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void st_dsmem(uint32_t a, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
-}
-__device__ __forceinline__ void st_dsmem(uint32_t a, double2 v) {
-  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
-}
 
 // Shared memory of one CTA, in elements: the slice (n columns of ld >= 32
 // MAXR entries), the receive buffers of the partial sums ([2][cs][n], by
-// step parity and source CTA), row j ([2][n]), the gathered sums (n, when
-// staged), the partial norms ([2][cs]), tau of every step (n, when Q is
-// formed) and tau, sc and the new diagonal of the last two steps.
+// step parity and source CTA), row j ([2][n]), the partial norms ([2][cs]), tau
+// of every step (n, when Q is formed) and six entries to spare; behind it
+// kPanelExtra bytes and the columns' scales.
 struct PanelLayout {
   int ld;
-  size_t recv, rowb, gs, pp, tau, ring, bytes;
+  size_t recv, rowb, pp, tau, bytes;
 };
 template <typename C>
-__host__ __device__ inline PanelLayout panel_layout(int maxr, int n, int cs, bool want_q, bool odd_ld, bool gs) {
+__host__ __device__ inline PanelLayout panel_layout(int maxr, int n, int cs, bool want_q, bool odd_ld) {
   PanelLayout L;
   L.ld = 32 * maxr + (odd_ld ? 1 : 0);
   size_t o = (size_t)L.ld * n;
   const size_t ex0 = o;
   L.recv = o; o += 2 * (size_t)cs * n;
   L.rowb = o; o += 2 * (size_t)n;
-  L.gs = o; o += gs ? (size_t)n : 0;
   L.pp = o; o += 2 * (size_t)cs;
   // the same area holds the block buffers of the Q formation
   if (want_q) {
@@ -141,30 +138,52 @@ __host__ __device__ inline PanelLayout panel_layout(int maxr, int n, int cs, boo
     o = o > qb ? o : qb;
   }
   L.tau = o; o += want_q ? (size_t)n : 0;
-  L.ring = o; o += 6;
+  o += 6;
   L.bytes = sizeof(C) * o;
   return L;
 }
 
-// Householder step j, with the partial sums of step j already received:
-//  gather   threads c > j sum the received partial dots of column c (in
-//           source order); one thread forms the reflector from the partial
-//           norms and row j
-//  pass     every warp forms the updated column j + 1 in registers from the
-//           step's reflector and factor (x' = x - v f_{j+1}), updates its
-//           columns c > j + 1 and, from the same registers, takes the
-//           partial dots x'^H a_c of step j + 1 and pushes them (and row
-//           j + 1, from its owner CTA) to every CTA; the warp of column j + 1
-//           pushes its partial norm and stores the column after the cluster
-//           barrier, when no warp reads the old one any more
-// (one block barrier and one cluster barrier per step).  Column c is always
-// worked on by warp c mod nw, so a warp's own deferred stores and later loads
-// of a column are ordered by program order.  Column j stays unscaled while it
-// is read as the reflector of step j; its warp scales it in the next step.
+// Householder step j.  Fifteen warps work on columns, column c always by warp c
+// mod 15 (so that a warp's own deferred stores and later loads of a column are
+// ordered by program order); the last warp forms the reflectors.
+//  factors  the threads sum the received partial dots of column c in source
+//           order and form its factor f_c from them, row j and the reflector
+//  pass     every working warp forms the updated column j + 1 in registers
+//           (x' = x - v f_{j+1}), updates its columns c > j + 1 and, from the
+//           same registers, takes the partial dots x'^H a_c of step j + 1.  The
+//           warp of column j + 1 first pushes its partial norm and stores the
+//           column behind the block barrier that ends the pass, when no warp
+//           reads the old one any more.  Beside the pass the last warp waits
+//           for the norms and forms the reflector of step j + 1: the chain
+//           norm, exchange, reflector and the pass overlap.
+//  exchange complex64: behind that barrier the dots go to every CTA, a warp's
+//           stores to contiguous places of one CTA (instead of a store per
+//           column and CTA out of the pass: 2304 x 96, R alone, 338 us and
+//           310); row j + 1 went ahead with the factors, from its owner CTA.
+//           complex128, whose pass waits for the FP64 unit anyway, pushes dots
+//           and row out of the pass (512 x 64 with Q 1280 us and 1223).
+// The pushes complete on mbarriers (norm and alpha; dots and row; by step
+// parity), two block barriers a step.  A CTA pushes the sums of step j + 2 over
+// those of step j only after every CTA's sums of step j + 1, which are sent
+// behind the block barrier that follows the last read of the sums of step j
+// (and of the factors and dots staged over them).
+// Column j stays unscaled while it is read as the reflector of step j; its
+// warp scales it in the next step.
+//
+// Measured with Q, us, against a cluster barrier a step with the reflector
+// formed ahead of the pass and every factor formed by every warp: complex64
+// 2304 x 96 645 and 550, 2304 x 64 358 and 315, 512 x 48 158 and 144; complex128
+// 512 x 64 1526 and 1226, 512 x 32 594 and 502.  What is left of a step (2.9 us
+// at 2304 x 64) is the chain column, norm, push, reflector, factors; the Q part
+// takes two fifths.
+//
+// Order and rounding are part of the results (k_jac.cu says why): rows a CTA,
+// rows a lane, the tree over the lanes, the CTAs in rank order, and every
+// product and sum as written.
 template <typename C, int MAXR>
 __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restrict__ Ag, int m, int n,
                                                             C* __restrict__ Qg, C* __restrict__ Rg, long long stride,
-                                                            int ld, int use_gs, int scaled) {
+                                                            int ld, int scaled) {
   using R = typename Real<C>::T;
   cg::cluster_group cl = cg::this_cluster();
   const int cs = (int)cl.num_blocks(), cr = (int)cl.block_rank();
@@ -173,14 +192,18 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
   if (Qg) Qg += panel * stride;
   if (Rg) Rg += panel * (long long)n * n;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const PanelLayout L = panel_layout<C>(MAXR, n, cs, Qg != nullptr, (ld & 1) != 0, use_gs != 0);
+  const PanelLayout L = panel_layout<C>(MAXR, n, cs, Qg != nullptr, (ld & 1) != 0);
   C* A = (C*)smem_raw;                   // local row t of column c at A[c * ld + t]
   C* recv = A + L.recv;
   C* rowb = A + L.rowb;
-  C* gs = A + L.gs;
   C* pp = A + L.pp;                      // (scale, scaled sum of squares)
   C* s_tau = A + L.tau;
-  C* ring = A + L.ring;                  // [2][3]: tau, sc, diagonal
+  // barriers (norm, sums; by step parity), the failure mark, the factor of
+  // column j + 1, and tau, sc and the new diagonal of the last steps, [3][3]
+  const uint32_t bar_n = saddr(smem_raw + L.bytes), bar_s = bar_n + 16;
+  volatile int* failed = (volatile int*)(smem_raw + L.bytes + 32);
+  C* f_next = (C*)(smem_raw + L.bytes + 48);
+  C* ring = f_next + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   constexpr int rows = 32 * MAXR;
   const int r0 = cr * rows;
@@ -188,19 +211,41 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
   const int k = min(m, n);
   const C zero = mkc<C>(0, 0), one = mkc<C>(1, 0);
   // lane q < cs pushes to CTA q
-  const uint32_t recv_q = lane < cs ? dsmem_addr(smem_addr(recv), lane) : 0u;
-  const uint32_t rowb_q = lane < cs ? dsmem_addr(smem_addr(rowb), lane) : 0u;
-  const uint32_t pp_q = lane < cs ? dsmem_addr(smem_addr(pp), lane) : 0u;
+  constexpr bool kStaged = sizeof(R) == 4;   // the exchange of the dots behind the pass
+  const uint32_t bar_q = lane < cs ? remote(bar_n, lane) : 0u;
+  const uint32_t pp_q = lane < cs ? remote(saddr(pp), lane) : 0u;
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 4; ++q) bar_init(bar_n + 8 * q);
+    *failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
 
+  int wide = 0;                          // an entry beyond 2^-50 .. 2^50
   for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
     const int t = e / n, c = e % n;
-    A[(size_t)c * ld + t] = t < mr ? Ag[(long long)(r0 + t) * n + c] : zero;
+    const C x = t < mr ? Ag[(long long)(r0 + t) * n + c] : zero;
+    A[(size_t)c * ld + t] = x;
+    if constexpr (sizeof(R) == 4) {
+      const unsigned a = __float_as_uint(fmaxf(fabsf(x.x), fabsf(x.y)));
+      wide |= a != 0 && a - (77u << 23) > (100u << 23);
+    }
+  }
+  int* s_wide = (int*)(smem_raw + L.bytes + 36);
+  if constexpr (sizeof(R) == 4) {
+    if (scaled) {
+      wide = __syncthreads_or(wide);
+      if (threadIdx.x == 0) *s_wide = wide;
+    }
   }
   cl.sync();                             // every CTA of the cluster runs before the first push
-  // complex64 columns of any magnitude: each is scaled by the power of two near
+  if (scaled) {
+    scaled = 0;
+    for (int q = 0; q < cs; ++q) scaled |= *cl.map_shared_rank(s_wide, q);
+  }
+  // complex64 columns of other magnitudes: each is scaled by the power of two near
   // its largest entry (exact, so every factor and every bit of Q stays what it
   // is), or the product of two large columns would overflow; R is scaled back
-  float* s_scale = (float*)(smem_raw + L.bytes);
+  float* s_scale = (float*)(smem_raw + L.bytes + kPanelExtra);
   if constexpr (sizeof(R) == 4) {
     if (scaled) {
       for (int c = warp; c < n; c += nw) {
@@ -257,9 +302,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
       if (r0 + lane + 32 * i <= g0) x[i] = zero;
   };
   auto dot = [&](const C (&x)[MAXR], const C (&y)[MAXR]) {   // sum over the slice of conj(x) y
-    C acc = pmulc(x[0], y[0]);
+    C acc = fmulc(x[0], y[0]);
 #pragma unroll
-    for (int i = 1; i < MAXR; ++i) acc = padd(acc, pmulc(x[i], y[i]));
+    for (int i = 1; i < MAXR; ++i) acc = padd(acc, fmulc(x[i], y[i]));
     acc.x = wsum(acc.x);
     acc.y = wsum(acc.y);
     return acc;
@@ -269,40 +314,63 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
     if constexpr (sizeof(R) == 8) {
       R s2 = 0;
 #pragma unroll
-      for (int i = 0; i < MAXR; ++i) s2 += x[i].x * x[i].x + x[i].y * x[i].y;
+      for (int i = 0; i < MAXR; ++i) s2 += fma(x[i].x, x[i].x, x[i].y * x[i].y);
       return mkc<C>(1, wsum(s2));
     } else {
       R amax = 0;
 #pragma unroll
       for (int i = 0; i < MAXR; ++i) amax = fmaxf(amax, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
-      amax = wmax(amax);
-      if (amax == 0) return zero;
-      int ex;
-      frexpf(amax, &ex);                 // amax < 2^ex; 2^-ex in two in-range factors
-      const R s1 = ldexpf(1.f, -(ex / 2)), s2 = ldexpf(1.f, -(ex - ex / 2));
+      const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+      if (bits == 0) return zero;
+      int ex = (int)(bits >> 23) - 126;  // amax < 2^ex; 2^-ex in two in-range factors
+      if (ex == -126) frexpf(__uint_as_float(bits), &ex);
+      const R s1 = __uint_as_float((unsigned)(127 - ex / 2) << 23);
+      const R s2 = __uint_as_float((unsigned)(127 - (ex - ex / 2)) << 23);
       R ss = 0;
 #pragma unroll
       for (int i = 0; i < MAXR; ++i) {
         const R a = x[i].x * s1 * s2, b = x[i].y * s1 * s2;
-        ss += a * a + b * b;
+        ss += fma(a, a, b * b);
       }
       return mkc<C>(ldexpf(1.f, ex), wsum(ss));
     }
   };
-  auto push_recv = [&](int par, int c, C d) {
-    if (lane < cs) st_dsmem(recv_q + (uint32_t)(sizeof(C) * ((size_t)(par * cs + cr) * n + c)), d);
-  };
   auto push_norm = [&](int par, C np) {
-    if (lane < cs) st_dsmem(pp_q + (uint32_t)(sizeof(C) * (size_t)(par * cs + cr)), np);
+    if (lane < cs) push(pp_q + (uint32_t)(sizeof(C) * (size_t)(par * cs + cr)), bar_q + 8 * par, np.x, np.y);
   };
-  // row g of column values y, from the CTA that holds it, into every CTA
-  auto push_row = [&](const C (&y)[MAXR], int g, int par, int c) {
+  // entry c of row g = the step's row, to every CTA (the diagonal entry with the
+  // norms): a thread a column, so that a warp's stores to a CTA are contiguous
+  auto push_entry = [&](int g, int c, C val) {
+    const uint32_t a = saddr(rowb) + (uint32_t)(sizeof(C) * ((size_t)(g & 1) * n + c));
+    const uint32_t b = bar_n + (c == g ? 0 : 16) + 8 * (g & 1);
+    for (int q = 0; q < cs; ++q) push(remote(a, q), remote(b, q), val.x, val.y);
+  };
+  // the partial dot of column c of step g to every CTA: lane q to CTA q
+  auto push_dot = [&](int g, int c, C d) {
+    if (lane < cs)
+      push(remote(saddr(recv) + (uint32_t)(sizeof(C) * ((size_t)((g & 1) * cs + cr) * n + c)), lane),
+           remote(bar_s + 8 * (g & 1), lane), d.x, d.y);
+  };
+  // row g of column values y, from the CTA that holds it, to every CTA
+  auto push_row = [&](const C (&y)[MAXR], int g, int c) {
     const int t = g - r0;
     if (t < 0 || t >= mr) return;        // uniform over the CTA
     C val = pick(y, t >> 5);
     val.x = __shfl_sync(0xffffffffu, val.x, t & 31);
     val.y = __shfl_sync(0xffffffffu, val.y, t & 31);
-    if (lane < cs) st_dsmem(rowb_q + (uint32_t)(sizeof(C) * ((size_t)par * n + c)), val);
+    if (lane < cs)
+      push(remote(saddr(rowb) + (uint32_t)(sizeof(C) * ((size_t)(g & 1) * n + c)), lane),
+           remote(bar_n + (c == g ? 0 : 16) + 8 * (g & 1), lane), val.x, val.y);
+  };
+  // the partial dots of step g (columns c > g, staged at dots[c]) to every CTA
+  auto push_dots = [&](int g, const C* dots) {
+    const int cols = n - g - 1;
+    const uint32_t a = saddr(recv) + (uint32_t)(sizeof(C) * (size_t)((g & 1) * cs + cr) * n);
+    for (int e = threadIdx.x; e < cs * cols; e += kPanelThreads) {
+      const int q = e / cols, c = g + 1 + e - q * cols;
+      const C d = dots[c];
+      push(remote(a + (uint32_t)(sizeof(C) * c), q), remote(bar_s + 8 * (g & 1), q), d.x, d.y);
+    }
   };
   auto sum_recv = [&](int par, int c) {   // the cluster sum of column c, in source order
     C s = zero;
@@ -311,80 +379,121 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
   };
 
   // ---- factorisation
-  if (k > 0) {                           // sums of step 0
+  const bool works = warp < kPanelWork;
+  {                                      // sums of step 0
+    C* d0 = recv + (size_t)cs * n;       // (staged where those of step 1 will be received)
     C x[MAXR];
     load_col(0, x);
-    if (warp == 0) push_row(x, 0, 0, 0);
     mask_below(x, 0);
     if (warp == 0) push_norm(0, norm_part(x));
-    for (int c = warp == 0 ? nw : warp; c < n; c += nw) {
+    for (int c = 1 + warp; c < n; c += kPanelThreads / 32) {
       C y[MAXR];
       load_col(c, y);
-      push_recv(0, c, dot(x, y));
-      push_row(y, 0, 0, c);
+      const C d = dot(x, y);
+      if (lane == 0) d0[c] = d;
     }
+    if (cr == 0)
+      for (int c = threadIdx.x; c < n; c += kPanelThreads) push_entry(0, c, A[(size_t)c * ld]);
+    __syncthreads();
+    push_dots(0, d0);
   }
-  cl.sync();
-  for (int j = 0; j < k; ++j) {
+  // the reflector of step j from the norm of x and alpha = A[j][j] (one warp)
+  auto reflector = [&](int j) {
     const int par = j & 1;
-    if (use_gs)
-      for (int c = j + 1 + threadIdx.x; c < n; c += blockDim.x) gs[c] = sum_recv(par, c);
-    if (threadIdx.x == blockDim.x - 1) {
-      // the reflector of step j from the norm of x and alpha = A[j][j]
-      R M = 0, S = 0;
-      for (int q = 0; q < cs; ++q) M = fmax(M, pp[par * cs + q].x);
-      if (M > 0) {
-        const R iM = (R)1 / M;           // (the scales are powers of two: exact)
-        for (int q = 0; q < cs; ++q) {
-          const C np = pp[par * cs + q];
-          const R rq = np.x * iM;
-          S += np.y * rq * rq;
+    if (lane == 0) bar_expect(bar_n + 8 * par, (uint32_t)(sizeof(C) * (cs + 1)));
+    __syncwarp();
+    bar_wait(bar_n + 8 * par, j >> 1 & 1, failed);
+    R M = 0, S = 0;
+    C np[kPanelMaxCluster];              // (loaded together, used in rank order)
+#pragma unroll
+    for (int q = 0; q < kPanelMaxCluster; ++q) np[q] = q < cs ? pp[par * cs + q] : zero;
+#pragma unroll
+    for (int q = 0; q < kPanelMaxCluster; ++q)
+      if (q < cs) M = fmax(M, np[q].x);
+    if (M > 0) {
+      const R iM = (R)1 / M;             // (the scales are powers of two: exact)
+#pragma unroll
+      for (int q = 0; q < kPanelMaxCluster; ++q)
+        if (q < cs) {
+          const R rq = np[q].x * iM;
+          S = fma(np[q].y * rq, rq, S);
         }
+    }
+    const R xnorm = M * sqrt(S);
+    const C alpha = rowb[(size_t)par * n + j];
+    const R ar = alpha.x, ai = alpha.y;
+    R taur = 0, taui = 0, scr = 0, sci = 0, beta = ar;
+    if (!(xnorm == 0 && ai == 0)) {
+      // beta = -sign(ar) |(alpha, x)| from scaled terms; alpha - beta
+      // scaled by 1 / |beta| (|alpha - beta| >= |beta|), so that nothing
+      // overflows or underflows
+      const R mx = fmax(fmax(fabs(ar), fabs(ai)), xnorm), imx = (R)1 / mx;
+      const R u = ar * imx, w = ai * imx, z = xnorm * imx;
+      beta = -copysign(mx * sqrt(fma(z, z, fma(u, u, w * w))), ar);
+      const R ib = (R)1 / beta, sb = fabs(ib);
+      const R dx = (ar - beta) * sb, dy = ai * sb, idd = sb / fma(dx, dx, dy * dy);
+      taur = (beta - ar) * ib;
+      taui = -ai * ib;
+      scr = dx * idd;
+      sci = -dy * idd;
+      // (the element type must hold sc too: columns near the bottom of its
+      // range leave the column as it is)
+      const R smax = sizeof(R) == 4 ? (R)1e37 : (R)1e300;
+      if (!(isfinite(taur) && isfinite(taui) && isfinite(scr) && isfinite(sci) && isfinite(beta)) ||
+          fabs(scr) > smax || fabs(sci) > smax || beta == (R)0) {
+        taur = taui = scr = sci = 0;
+        beta = ar;
       }
-      const R xnorm = M * sqrt(S);
-      const C alpha = rowb[(size_t)par * n + j];
-      const R ar = alpha.x, ai = alpha.y;
-      R taur = 0, taui = 0, scr = 0, sci = 0, beta = ar;
-      if (!(xnorm == 0 && ai == 0)) {
-        // beta = -sign(ar) |(alpha, x)| from scaled terms; alpha - beta
-        // scaled by 1 / |beta| (|alpha - beta| >= |beta|), so that nothing
-        // overflows or underflows
-        const R mx = fmax(fmax(fabs(ar), fabs(ai)), xnorm), imx = (R)1 / mx;
-        const R u = ar * imx, w = ai * imx, z = xnorm * imx;
-        beta = -copysign(mx * sqrt(u * u + w * w + z * z), ar);
-        const R ib = (R)1 / beta, sb = fabs(ib);
-        const R dx = (ar - beta) * sb, dy = ai * sb, idd = sb / (dx * dx + dy * dy);
-        taur = (beta - ar) * ib;
-        taui = -ai * ib;
-        scr = dx * idd;
-        sci = -dy * idd;
-        // (the element type must hold sc too: columns near the bottom of its
-        // range leave the column as it is)
-        const R smax = sizeof(R) == 4 ? (R)1e37 : (R)1e300;
-        if (!(isfinite(taur) && isfinite(taui) && isfinite(scr) && isfinite(sci) && isfinite(beta)) ||
-            fabs(scr) > smax || fabs(sci) > smax || beta == (R)0) {
-          taur = taui = scr = sci = 0;
-          beta = ar;
-        }
-      }
+    }
+    if (lane == 0) {
       const bool act = !(taur == 0 && taui == 0);
-      ring[par * 3 + 0] = mkc<C>(taur, taui);
-      ring[par * 3 + 1] = mkc<C>(scr, sci);
-      ring[par * 3 + 2] = mkc<C>(beta, act ? (R)0 : ai);
+      C* out = ring + 3 * (j % 3);
+      out[0] = mkc<C>(taur, taui);
+      out[1] = mkc<C>(scr, sci);
+      out[2] = mkc<C>(beta, act ? (R)0 : ai);
       if (Qg) s_tau[j] = mkc<C>(taur, taui);
     }
-    __syncthreads();
-    const C tj = ring[par * 3 + 0], sc = ring[par * 3 + 1], ctau = mkc<C>(tj.x, -tj.y);
+  };
+  if (!works) reflector(0);
+  __syncthreads();
+  for (int j = 0; j < k; ++j) {
+    const int par = j & 1;
+    const C* now = ring + 3 * (j % 3);
+    const C tj = now[0], sc = now[1], ctau = mkc<C>(tj.x, -tj.y);
     const bool active = !(tj.x == 0 && tj.y == 0);
+    // the factors, over the sums of CTA 0
+    C* fj = recv + (size_t)(par * cs) * n;
+    if (j + 1 < n) {
+      if (threadIdx.x == 0) bar_expect(bar_s + 8 * par, (uint32_t)(sizeof(C) * (size_t)(cs + 1) * (n - j - 1)));
+      bar_wait(bar_s + 8 * par, j >> 1 & 1, failed);
+      for (int c = j + 1 + threadIdx.x; c < n; c += blockDim.x) {
+        const C s = sum_recv(par, c);
+        const C f = active ? fmul<2>(ctau, padd(rowb[(size_t)par * n + c], fmulc(sc, s))) : zero;
+        fj[c] = f;
+        if (c == j + 1) *f_next = f;
+        // row j + 1 after step j, from the CTA that holds it
+        const int t = j + 1 - r0;
+        if (kStaged && j + 1 < k && t >= 0 && t < mr)
+          push_entry(j + 1, c, psub(A[(size_t)c * ld + t], fmul<MAXR>(fmul<MAXR>(A[(size_t)j * ld + t], sc), f)));
+      }
+    }
+    __syncthreads();
+    if (!works) {
+      if (j + 1 < k) reflector(j + 1);
+      __syncthreads();
+      if (kStaged && j + 1 < k) push_dots(j + 1, fj);
+      continue;
+    }
     // scale the reflector of step j - 1 (no longer read)
-    if (j > 0 && warp == (j - 1) % nw) {
+    if (j > 0 && warp == (j - 1) % kPanelWork) {
       C x[MAXR];
       load_col(j - 1, x);
-      const C scp = ring[(par ^ 1) * 3 + 1], dg = ring[(par ^ 1) * 3 + 2];
+      const C* was = ring + 3 * ((j - 1) % 3);
+      const C scp = was[1], dg = was[2];
 #pragma unroll
       for (int i = 0; i < MAXR; ++i) {
         const int g = r0 + lane + 32 * i;
-        if (g > j - 1) x[i] = pmul(x[i], scp);
+        if (g > j - 1) x[i] = fmul<2>(x[i], scp);
         else if (g == j - 1) x[i] = dg;
       }
       store_col(j - 1, x);
@@ -394,20 +503,16 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
 #pragma unroll
     for (int i = 0; i < MAXR; ++i) {
       const int g = r0 + lane + 32 * i;
-      v[i] = g > j ? pmul(v[i], sc) : (g == j ? one : zero);
+      v[i] = g > j ? fmul<MAXR>(v[i], sc) : (g == j ? one : zero);
     }
-    auto fac = [&](int c) {
-      const C s = use_gs ? gs[c] : sum_recv(par, c);
-      return active ? pmul(ctau, padd(rowb[(size_t)par * n + c], pmulc(sc, s))) : zero;
-    };
-    const bool own = j + 1 < n && warp == (j + 1) % nw;
+    const bool own = j + 1 < n && warp == (j + 1) % kPanelWork;
     C xm[MAXR];                          // column j + 1 after step j, then its rows > j + 1
     C keep_j = zero, keep_j1 = zero;     // (owner) its rows j and j + 1, in the lanes that hold them
     if (j + 1 < n) {
       load_col(j + 1, xm);
-      const C f1 = fac(j + 1);
+      const C f1 = *f_next;
 #pragma unroll
-      for (int i = 0; i < MAXR; ++i) xm[i] = psub(xm[i], pmul(v[i], f1));
+      for (int i = 0; i < MAXR; ++i) xm[i] = psub(xm[i], fmul<MAXR>(v[i], f1));
       if (own) {
 #pragma unroll
         for (int i = 0; i < MAXR; ++i) {
@@ -415,34 +520,34 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
           if (g == j) keep_j = xm[i];
           if (g == j + 1) keep_j1 = xm[i];
         }
-        if (j + 1 < k) push_row(xm, j + 1, par ^ 1, j + 1);
+        if (!kStaged && j + 1 < k) push_row(xm, j + 1, j + 1);
       }
       mask_below(xm, j + 1);
       if (own && j + 1 < k) push_norm(par ^ 1, norm_part(xm));
-      int c = j + 2 + ((warp - (j + 2)) % nw + nw) % nw;
+      int c = j + 2 + ((warp - (j + 2)) % kPanelWork + kPanelWork) % kPanelWork;
       if constexpr ((sizeof(R) == 4 && MAXR <= 6) || (sizeof(R) == 8 && MAXR <= 2)) {
         // two columns at a time (two independent chains, one reduction
         // tree for both dots: lanes 0-7 end with the first real part, 8-15
         // its imaginary part, 16-31 the second column's)
-        for (; c + nw < n; c += 2 * nw) {
-          const int c2 = c + nw;
+        for (; c + kPanelWork < n; c += 2 * kPanelWork) {
+          const int c2 = c + kPanelWork;
           C y[MAXR], y2[MAXR];
           load_col(c, y);
           load_col(c2, y2);
-          const C f = fac(c), f2 = fac(c2);
+          const C f = fj[c], f2 = fj[c2];
 #pragma unroll
           for (int i = 0; i < MAXR; ++i) {
-            y[i] = psub(y[i], pmul(v[i], f));
-            y2[i] = psub(y2[i], pmul(v[i], f2));
+            y[i] = psub(y[i], fmul<MAXR>(v[i], f));
+            y2[i] = psub(y2[i], fmul<MAXR>(v[i], f2));
           }
           store_col(c, y);
           store_col(c2, y2);
           if (j + 1 < k) {
-            C d = pmulc(xm[0], y[0]), d2 = pmulc(xm[0], y2[0]);
+            C d = fmulc(xm[0], y[0]), d2 = fmulc(xm[0], y2[0]);
 #pragma unroll
             for (int i = 1; i < MAXR; ++i) {
-              d = padd(d, pmulc(xm[i], y[i]));
-              d2 = padd(d2, pmulc(xm[i], y2[i]));
+              d = padd(d, fmulc(xm[i], y[i]));
+              d2 = padd(d2, fmulc(xm[i], y2[i]));
             }
             const bool h4 = lane & 16, h3 = lane & 8;
             R a0 = h4 ? d2.x : d.x, a1 = h4 ? d2.y : d.y;     // kept halves
@@ -454,27 +559,40 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
             b += __shfl_xor_sync(0xffffffffu, b, 1);
             const C s1 = mkc<C>(__shfl_sync(0xffffffffu, b, 0), __shfl_sync(0xffffffffu, b, 8));
             const C s2 = mkc<C>(__shfl_sync(0xffffffffu, b, 16), __shfl_sync(0xffffffffu, b, 24));
-            push_recv(par ^ 1, c, s1);
-            push_recv(par ^ 1, c2, s2);
-            push_row(y, j + 1, par ^ 1, c);
-            push_row(y2, j + 1, par ^ 1, c2);
+            if constexpr (kStaged) {
+              if (lane == 0) {           // (over the factors, which this warp has read)
+                fj[c] = s1;
+                fj[c2] = s2;
+              }
+            } else {
+              push_dot(j + 1, c, s1);
+              push_dot(j + 1, c2, s2);
+              push_row(y, j + 1, c);
+              push_row(y2, j + 1, c2);
+            }
           }
         }
       }
-      for (; c < n; c += nw) {
+      for (; c < n; c += kPanelWork) {
         C y[MAXR];
         load_col(c, y);
-        const C f = fac(c);
+        const C f = fj[c];
 #pragma unroll
-        for (int i = 0; i < MAXR; ++i) y[i] = psub(y[i], pmul(v[i], f));
+        for (int i = 0; i < MAXR; ++i) y[i] = psub(y[i], fmul<MAXR>(v[i], f));
         store_col(c, y);
         if (j + 1 < k) {
-          push_recv(par ^ 1, c, dot(xm, y));
-          push_row(y, j + 1, par ^ 1, c);
+          const C d = dot(xm, y);
+          if constexpr (kStaged) {
+            if (lane == 0) fj[c] = d;
+          } else {
+            push_dot(j + 1, c, d);
+            push_row(y, j + 1, c);
+          }
         }
       }
     }
-    cl.sync();
+    __syncthreads();
+    if (kStaged && j + 1 < k) push_dots(j + 1, fj);
     if (own) {                           // column j + 1, rows >= j (rows above are unchanged)
       C* p = A + (size_t)(j + 1) * ld + lane;
 #pragma unroll
@@ -486,14 +604,14 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
       }
     }
   }
-  if (k > 0 && warp == (k - 1) % nw) {   // scale the last reflector
+  if (k > 0 && warp == (k - 1) % kPanelWork) {   // scale the last reflector
     C x[MAXR];
     load_col(k - 1, x);
-    const C scp = ring[((k - 1) & 1) * 3 + 1], dg = ring[((k - 1) & 1) * 3 + 2];
+    const C scp = ring[3 * ((k - 1) % 3) + 1], dg = ring[3 * ((k - 1) % 3) + 2];
 #pragma unroll
     for (int i = 0; i < MAXR; ++i) {
       const int g = r0 + lane + 32 * i;
-      if (g > k - 1) x[i] = pmul(x[i], scp);
+      if (g > k - 1) x[i] = fmul<2>(x[i], scp);
       else if (g == k - 1) x[i] = dg;
     }
     store_col(k - 1, x);
@@ -509,7 +627,19 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
         if (scaled) x = mkc<C>(x.x * s_scale[c], x.y * s_scale[c]);
       if (g < k) Rg[(long long)g * n + c] = x;
     }
-  if (!Qg) return;     // nothing is pushed after the last cluster barrier above
+  // an exchange that ran out leaves a NaN
+  auto leave = [&](C* out) {
+    __syncthreads();
+    if (threadIdx.x == 0 && *failed && out && r0 < m) {
+      const R bad = (R)__int_as_float(0x7fffffff);
+      out[0] = mkc<C>(bad, bad);
+    }
+  };
+  if (!Qg) {
+    leave(Rg ? Rg + (size_t)(r0 < k ? r0 : 0) * n : nullptr);
+    cl.sync();
+    return;
+  }
 
   // ---- Q = H_0 ... H_{k-1} [I; 0] by blocks of NB reflectors, the last
   // block first, in place: H_{b0} ... H_{b1-1} = I - V T V^H (compact WY;
@@ -598,7 +728,11 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
         x[i] = vb(b0, a, lane + 32 * i);
         y[i] = vb(b0, b, lane + 32 * i);
       }
-      const C d = dot(x, y);
+      C d = pmulc(x[0], y[0]);
+#pragma unroll
+      for (int i = 1; i < MAXR; ++i) d = padd(d, pmulc(x[i], y[i]));
+      d.x = wsum(d.x);
+      d.y = wsum(d.y);
       if (lane == 0) Pw[(size_t)a * W + k + b] = d;
     }
     cl.sync();
@@ -662,6 +796,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
     const int t = e / k, c = e % k;
     Qg[(long long)(r0 + t) * k + c] = A[(size_t)c * ld + t];
   }
+  leave(Qg + (size_t)r0 * k);
 }
 
 // sum of slot[off] over the cluster's CTAs in rank order (the same grouping
@@ -1061,24 +1196,27 @@ cudaError_t panel_optin() {
 struct PanelPlan {
   bool pull = false;
   int maxr = 0, cs = 0, ld = 0, rows = 0;
-  bool gs = true;
   size_t bytes = 0;
 };
 
-// the first layout that fits: odd column stride (no bank conflicts in the
-// row-major copies) with staged sums, even stride, then sums taken in place
+// Whether a panel's slices fit (the published smallest cluster goes by this),
+// and the layout taken: odd column stride (no bank conflicts in the row-major
+// copies), else even; false when the barriers behind it do not fit.
+template <typename C>
+bool panel_holds(int n, int maxr, int cs, bool want_q) {
+  return panel_layout<C>(maxr, n, cs, want_q, false).bytes <= (size_t)kPanelSmemMax;
+}
 template <typename C>
 bool panel_fit(int n, int maxr, int cs, bool want_q, PanelPlan& p) {
-  for (int v = 0; v < 3; ++v) {
-    const PanelLayout L = panel_layout<C>(maxr, n, cs, want_q, v == 0, v < 2);
-    if (L.bytes <= (size_t)kPanelSmemMax) {
+  for (bool odd : {true, false}) {
+    const PanelLayout L = panel_layout<C>(maxr, n, cs, want_q, odd);
+    if (L.bytes + kPanelExtra <= (size_t)kPanelSmemMax) {
       p.pull = false;
       p.maxr = maxr;
       p.cs = cs;
       p.ld = L.ld;
       p.rows = 32 * maxr;
-      p.gs = v < 2;
-      p.bytes = L.bytes;
+      p.bytes = L.bytes + kPanelExtra;
       return true;
     }
   }
@@ -1134,7 +1272,9 @@ bool panel_plan(int m, int n, bool want_q, int cluster, PanelPlan& p) {
         if (panel_fit<C>(n, list[a], cluster, want_q, p)) return true;
         break;
       }
-    return panel_fit_pull<C>(m, n, cluster, p);
+    if (panel_fit_pull<C>(m, n, cluster, p)) return true;
+    // (110 columns, R alone, fill three CTAs to the last bytes: one CTA more)
+    return panel_plan<C>(m, n, want_q, cluster + 1, p);
   }
   const int pref = sizeof(C) == sizeof(float2) ? 9 : kPanelMaxCluster;
   for (int lim : {pref, kPanelMaxCluster})
@@ -1163,7 +1303,7 @@ int panel_min_cluster(int m, int n, bool want_q) {
   PanelPlan p;
   for (int a = nl - 1; a >= 0; --a) {
     const int cs = (m + 32 * list[a] - 1) / (32 * list[a]);
-    if (cs <= kPanelMaxCluster && panel_fit<C>(n, list[a], cs, want_q, p) && (best == 0 || cs < best)) best = cs;
+    if (cs <= kPanelMaxCluster && panel_holds<C>(n, list[a], cs, want_q) && (best == 0 || cs < best)) best = cs;
   }
   for (int cs = 1; cs <= kPanelMaxCluster && (best == 0 || cs < best); ++cs)
     if (panel_fit_pull<C>(m, n, cs, p)) {
@@ -1213,22 +1353,22 @@ static cudaError_t panel_t(const C* A, int m, int n, C* Q, C* R, int batch, long
       if (p.maxr == 8) return cudaLaunchKernelEx(&cfg, k_panel_qr_pull<C, 8>, A, m, n, p.rows, Q, R, stride);
     return cudaErrorInvalidValue;
   }
-  const int gsf = p.gs ? 1 : 0;
   // (a panel that fills the shared memory has no room for the columns' scales)
-  const int scaled = any_range && sizeof(C) == sizeof(float2) && p.bytes + sizeof(float) * n <= (size_t)kPanelSmemMax;
+  const int scaled = any_range && sizeof(C) == sizeof(float2) &&
+                     cfg.dynamicSmemBytes + sizeof(float) * n <= (size_t)kPanelSmemMax;
   if (scaled) cfg.dynamicSmemBytes += sizeof(float) * n;
   switch (p.maxr) {
-    case 1: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 1>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
-    case 2: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 2>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
-    case 3: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 3>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
-    case 4: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 4>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+    case 1: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 1>, A, m, n, Q, R, stride, p.ld, scaled);
+    case 2: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 2>, A, m, n, Q, R, stride, p.ld, scaled);
+    case 3: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 3>, A, m, n, Q, R, stride, p.ld, scaled);
+    case 4: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 4>, A, m, n, Q, R, stride, p.ld, scaled);
     default: break;
   }
   if constexpr (sizeof(C) == sizeof(float2)) {
     switch (p.maxr) {
-      case 5: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 5>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
-      case 6: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 6>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
-      case 8: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 8>, A, m, n, Q, R, stride, p.ld, gsf, scaled);
+      case 5: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 5>, A, m, n, Q, R, stride, p.ld, scaled);
+      case 6: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 6>, A, m, n, Q, R, stride, p.ld, scaled);
+      case 8: return cudaLaunchKernelEx(&cfg, k_panel_qr<C, 8>, A, m, n, Q, R, stride, p.ld, scaled);
       default: break;
     }
   }

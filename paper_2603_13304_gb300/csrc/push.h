@@ -16,9 +16,15 @@ __device__ __forceinline__ uint32_t remote(uint32_t a, int rank) {
   return r;
 }
 
-// Sixteen-byte pushes into another CTA's shared memory that complete on that
-// CTA's mbarrier, and the bounded wait for them: a wait that runs out marks
-// the CTA, whose outputs become NaN.
+// Pushes of eight or sixteen bytes into another CTA's shared memory that
+// complete on that CTA's mbarrier, and the bounded wait for them: a wait that
+// runs out marks the CTA (the kernels report it: NaN in the panels, the status
+// word in the Jacobi).
+__device__ __forceinline__ void push(uint32_t a, uint32_t bar, float v0, float v1) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a),
+               "f"(v0), "f"(v1), "r"(bar)
+               : "memory");
+}
 __device__ __forceinline__ void push(uint32_t a, uint32_t bar, float v0, float v1, float v2, float v3) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a),
                "f"(v0), "f"(v1), "f"(v2), "f"(v3), "r"(bar)
