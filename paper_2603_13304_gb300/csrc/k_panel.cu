@@ -111,7 +111,7 @@ __device__ __forceinline__ double2 pick(const double2 (&y)[MAXR], int q) {
 constexpr int kPanelThreads = 512;
 constexpr int kPanelSmemMax = 227 * 1024;
 constexpr int kPanelWork = kPanelThreads / 32 - 1;   // warps that work on columns
-constexpr int kPanelExtra = 48 + 10 * 16;            // bytes behind the layout: barriers, the last reflectors
+constexpr int kPanelExtra = 48 + 11 * 16;            // bytes behind the layout: barriers, the last reflectors
 constexpr int kQBlock = 8;               // reflectors a block of the Q formation
 
 // Shared memory of one CTA, in elements: the slice (n columns of ld >= 32
@@ -199,11 +199,14 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
   C* pp = A + L.pp;                      // (scale, scaled sum of squares)
   C* s_tau = A + L.tau;
   // barriers (norm, sums; by step parity), the failure mark, the factor of
-  // column j + 1, and tau, sc and the new diagonal of the last steps, [3][3]
+  // column j + 1, the entry of column j in row j + 1 (from its owner: the column
+  // itself is stored behind the block barrier that ends a pass, with no barrier
+  // before the factors), and tau, sc and the new diagonal of the last steps, [3][3]
   const uint32_t bar_n = saddr(smem_raw + L.bytes), bar_s = bar_n + 16;
   volatile int* failed = (volatile int*)(smem_raw + L.bytes + 32);
   C* f_next = (C*)(smem_raw + L.bytes + 48);
-  C* ring = f_next + 1;
+  C* x_next = f_next + 1;
+  C* ring = f_next + 2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   constexpr int rows = 32 * MAXR;
   const int r0 = cr * rows;
@@ -394,6 +397,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
     }
     if (cr == 0)
       for (int c = threadIdx.x; c < n; c += kPanelThreads) push_entry(0, c, A[(size_t)c * ld]);
+    if (threadIdx.x == 0 && 1 - r0 >= 0 && 1 - r0 < mr) *x_next = A[1 - r0];
     __syncthreads();
     push_dots(0, d0);
   }
@@ -474,7 +478,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
         // row j + 1 after step j, from the CTA that holds it
         const int t = j + 1 - r0;
         if (kStaged && j + 1 < k && t >= 0 && t < mr)
-          push_entry(j + 1, c, psub(A[(size_t)c * ld + t], fmul<MAXR>(fmul<MAXR>(A[(size_t)j * ld + t], sc), f)));
+          push_entry(j + 1, c, psub(A[(size_t)c * ld + t], fmul<MAXR>(fmul<MAXR>(*x_next, sc), f)));
       }
     }
     __syncthreads();
@@ -519,6 +523,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel_qr(const C* __restri
           const int g = r0 + lane + 32 * i;
           if (g == j) keep_j = xm[i];
           if (g == j + 1) keep_j1 = xm[i];
+          if (kStaged && g == j + 2 && lane + 32 * i < mr) *x_next = xm[i];
         }
         if (!kStaged && j + 1 < k) push_row(xm, j + 1, j + 1);
       }

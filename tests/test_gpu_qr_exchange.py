@@ -1,10 +1,9 @@
-"""Exchanges of the blocked QR in which a CTA of the cluster owns no column.
+"""Exchanges of the panel QR under load.
 
-A panel narrower than twice its cluster has passes over fewer columns than
-CTAs: the CTAs without a column receive no partial product and send no factor.
-Many panels a launch, so that the CTAs of a cluster start apart, and many
-launches: every panel has to be factorised (a wait that runs out leaves a NaN)
-and every launch has to give the same bits.  Tolerance as for the other panels.
+Panels narrower than their cluster, and ordinary ones.  Many panels a launch, so
+that the CTAs of a cluster start apart, and many launches: every panel has to be
+factorised (a wait that runs out leaves a NaN) and every launch has to give the
+same bits.  Tolerance as for the other panels.
 """
 import numpy as np
 import pytest
@@ -23,10 +22,7 @@ def built():
     P.lib()
 
 
-@pytest.mark.parametrize("c64", [True, False])
-@pytest.mark.parametrize("m,n,cluster", [(300, 9, 16), (300, 16, 16), (300, 17, 9), (1100, 24, 16), (260, 12, 5)])
-def test_fewer_columns_than_ctas(c64, m, n, cluster):
-    batch = 40
+def check(c64, m, n, cluster, batch):
     rng = np.random.default_rng(m + n)
     A = (rng.standard_normal((batch, m, n)) + 1j * rng.standard_normal((batch, m, n)))
     A = A.astype(np.complex64 if c64 else np.complex128)
@@ -44,3 +40,18 @@ def test_fewer_columns_than_ctas(c64, m, n, cluster):
     eye = torch.eye(n, dtype=torch.complex128, device="cuda")
     assert (q.mH @ q - eye).abs().max().item() < tol
     assert ((q @ r - a.to(torch.complex128)).norm(dim=1) / a.to(torch.complex128).norm(dim=1)).max().item() < tol
+
+
+@pytest.mark.parametrize("c64", [True, False])
+@pytest.mark.parametrize("m,n,cluster", [(300, 9, 16), (300, 16, 16), (300, 17, 9), (1100, 24, 16), (260, 12, 5)])
+def test_fewer_columns_than_ctas(c64, m, n, cluster):
+    check(c64, m, n, cluster, 40)
+
+
+@pytest.mark.parametrize("c64", [True, False])
+@pytest.mark.parametrize("m,n,cluster", [(1300, 40, 6), (2000, 33, 9), (520, 48, 0), (1000, 47, 16)])
+def test_many_at_once(c64, m, n, cluster):
+    """Every SM busy with panels, so that the warps of a CTA drift apart: a column
+    or a row read before it is stored shows as other bits."""
+    cmin = P.bbp_k_panel_cluster(c64, m, n)
+    check(c64, m, n, max(cluster, cmin) if cluster else 0, 48)
