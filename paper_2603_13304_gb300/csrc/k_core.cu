@@ -447,6 +447,11 @@ cudaError_t smem_optin() {
 // prefetched into a double buffer, again one barrier per step.  Same
 // convention as cta_householder: R has a real diagonal beta_j,
 // Q = H_0 ... H_{k-1}, H = I - tau v v^H.
+// What bounds it: complex128, the FP64 unit (a warp-wide instruction 64 clocks,
+// one every 19 clocks an SM), most of a step being the reflector's chain of a
+// root and two quotients; complex64 (k_tsqr_reg) the same chain and the trees of
+// one column.  A warp a column and no more: 32 x 8 complex128 53 us (63 with 32
+// warps at every barrier and the quotients one after the other).
 template <typename C>
 struct TsqrSmem {
   static size_t bytes(int m, int n) {   // column-major (m + 1) x n or row-major m x (n + 1) panel
@@ -455,37 +460,58 @@ struct TsqrSmem {
   }
 };
 
+// largest of the lanes' non-negative values, on their bits (a NaN counts as
+// largest: the column is left as it is either way)
+__device__ __forceinline__ float lanes_max(float v) {
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ double lanes_max(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
+  return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
+}
+__device__ __forceinline__ float abs_max(float m, float2 a) { return fmaxf(m, fmaxf(fabsf(a.x), fabsf(a.y))); }
+__device__ __forceinline__ double abs_max(double m, double2 a) {   // (integer compares: none on the FP64 unit)
+  const long long x = __double_as_longlong(a.x) & 0x7fffffffffffffffll, y = __double_as_longlong(a.y) & 0x7fffffffffffffffll;
+  const long long b = __double_as_longlong(m);
+  return __longlong_as_double(max(b, max(x, y)));
+}
+
+// reflector of column j (rows j..m-1), by one warp in the element's real type,
+// with the column scaled by its largest magnitude first so that tiny columns
+// neither underflow nor divide by zero.  The two quotients at the end share one
+// instruction sequence (the FP64 unit takes a warp as long as a lane).
 template <typename C>
 __device__ void tsqr_params(const C* col, int j, int m, C* s_tau, C* s_sc, C* s_beta) {
-  // reflector of column j (rows j..m-1); computed by one warp in the
-  // element's real type, with the column scaled by its largest magnitude
-  // first so that tiny columns neither underflow nor divide by zero
   using R = typename RealOf<C>::T;
   const int lane = threadIdx.x & 31;
   const C alpha = col[j];
-  R amax = fmax(fabs(alpha.x), fabs(alpha.y));
-  for (int r = j + 1 + lane; r < m; r += 32) amax = fmax(amax, fmax(fabs(col[r].x), fabs(col[r].y)));
-  for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  R amax = abs_max((R)0, alpha);
+  for (int r = j + 1 + lane; r < m; r += 32) amax = abs_max(amax, col[r]);
+  amax = lanes_max(amax);
   const R sa = (amax > (R)0 && isfinite(amax)) ? (R)1 / amax : (R)0;
   R xn2 = 0;
   for (int r = j + 1 + lane; r < m; r += 32) xn2 += cabs2(cscale(col[r], sa));
   xn2 = warp_sum(xn2);
-  if (lane == 0) {
-    C tau = cx<C>(0, 0), sc = cx<C>(0, 0), beta = alpha;
-    if (sa > (R)0 && !(xn2 == (R)0 && alpha.y == (R)0)) {
-      const R ax = alpha.x * sa, ay = alpha.y * sa;          // scaled, |.| <= 1
-      const R bs = -copysign(sqrt(ax * ax + ay * ay + xn2), ax);
-      const R dx = ax - bs, dy = ay, dd = dx * dx + dy * dy;
-      const R ib = (R)1 / bs, idd = sa / dd;                 // 1 / (alpha - beta) = sa conj(d') / |d'|^2
-      tau = cx<C>((bs - ax) * ib, -ay * ib);
-      sc = cx<C>(dx * idd, -dy * idd);
-      beta = cx<C>(bs * amax, 0.0);
-      if (!(isfinite(tau.x) && isfinite(tau.y) && isfinite(sc.x) && isfinite(sc.y) && isfinite(beta.x))) {
-        tau = cx<C>(0, 0);                                     // leave the column as it is
-        sc = cx<C>(0, 0);
-        beta = alpha;
-      }
+  C tau = cx<C>(0, 0), sc = cx<C>(0, 0), beta = alpha;
+  if (sa > (R)0 && !(xn2 == (R)0 && alpha.y == (R)0)) {
+    const R ax = alpha.x * sa, ay = alpha.y * sa;          // scaled, |.| <= 1
+    const R bs = -copysign(sqrt(ax * ax + ay * ay + xn2), ax);
+    const R dx = ax - bs, dy = ay, dd = dx * dx + dy * dy;
+    const R quo = (lane & 1 ? sa : (R)1) / (lane & 1 ? dd : bs);
+    const R ib = __shfl_sync(0xffffffffu, quo, 0);
+    const R idd = __shfl_sync(0xffffffffu, quo, 1);        // 1 / (alpha - beta) = sa conj(d') / |d'|^2
+    tau = cx<C>((bs - ax) * ib, -ay * ib);
+    sc = cx<C>(dx * idd, -dy * idd);
+    beta = cx<C>(bs * amax, 0.0);
+    if (!(isfinite(tau.x) && isfinite(tau.y) && isfinite(sc.x) && isfinite(sc.y) && isfinite(beta.x))) {
+      tau = cx<C>(0, 0);                                     // leave the column as it is
+      sc = cx<C>(0, 0);
+      beta = alpha;
     }
+  }
+  if (lane == 0) {
     s_tau[j] = tau;
     s_sc[j] = sc;
     s_beta[j] = beta;
@@ -621,7 +647,7 @@ __device__ __forceinline__ void tsqr_params_reg(const float2* A, int ldr, int c,
   float amax = fmaxf(fabsf(alpha.x), fabsf(alpha.y));
 #pragma unroll
   for (int i = 0; i < MAXR; ++i) amax = fmaxf(amax, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  amax = lanes_max(amax);
   const float sa = (amax > 0.f && isfinite(amax)) ? 1.f / amax : 0.f;
   float xn2 = 0.f;
 #pragma unroll
@@ -664,7 +690,7 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
   Ag += (size_t)row0 * n;
   if (gridDim.x > 1) Rm += (size_t)blockIdx.x * n * n;
   const int k = m < n ? m : n;
-  const int ldr = n + 1;
+  const int ldr = n | 1;                     // odd: the rows of a column lie in different banks
   C* A = (C*)smem_raw;                       // (r, c) at A[r * ldr + c]
   C* vbuf = A + (size_t)m * ldr;
   C* s_tau = vbuf + 2 * (size_t)m;
@@ -828,12 +854,14 @@ cudaError_t tsqr_launch(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, cuda
   if constexpr (sizeof(C) == sizeof(float2)) {
     const size_t sr = tsqr_reg_bytes(rb, n);
     if (sr <= (size_t)kSmemMax) {
-      if (rb <= 128) return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, 512, sr, s);
-      if (rb <= 256) return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, 512, sr, s);
-      if (rb <= 512) return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, 512, sr, s);
+      const int threads = 32 * std::min(16, std::max(4, n));
+      if (rb <= 128) return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+      if (rb <= 256) return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+      if (rb <= 512) return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
     }
   }
-  return tsqr_run<k_tsqr_smem<C>>(Ag, m_all, n, Q, Rm, rb, 1024, TsqrSmem<C>::bytes(rb, n), s);
+  const int threads = 32 * std::min(32, std::max({4, n, rb / 64}));   // (a warp a column)
+  return tsqr_run<k_tsqr_smem<C>>(Ag, m_all, n, Q, Rm, rb, threads, TsqrSmem<C>::bytes(rb, n), s);
 }
 
 // ---------------------------------------------------------------- K3 Jacobi
