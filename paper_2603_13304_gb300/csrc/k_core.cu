@@ -628,11 +628,14 @@ __global__ void __launch_bounds__(1024) k_tsqr_smem(const C* __restrict__ Ag, in
 
 
 // complex64 variant of k_tsqr_smem: the panel is kept row-major with an odd
-// row stride (n + 1, so that a warp reading one column down 32 rows touches
-// distinct banks), global loads and stores run along rows, and the columns a
-// warp works on are cached in registers: lane l holds rows l + 32 i,
-// i < MAXR (m <= 32 MAXR), so every column pass issues its loads back to
-// back; 16 warps.  Same steps, barriers and results as k_tsqr_smem.
+// row stride (so that a warp reading one column down 32 rows touches distinct
+// banks), global loads and stores run along rows, and the columns a warp works
+// on are cached in registers: lane l holds rows l + 32 i, i < MAXR (m <= 32
+// MAXR, in steps of 64 rows: rows past m only add zeros), so every column pass
+// issues its loads back to back; at most 16 warps.  Same steps and barriers as
+// k_tsqr_smem.  Bound by the instructions of the columns and, of narrow panels,
+// by the reflector's chain: 432 x 27 166 us with an even stride and 512 rows'
+// worth of registers, 119 us; 288 x 32 148 and 109; 512 x 48 285.
 template <int MAXR>
 __device__ __forceinline__ void tsqr_params_reg(const float2* A, int ldr, int c, int j, int m, float2* s_tau,
                                                 float2* s_sc, float2* s_beta) {
@@ -855,9 +858,17 @@ cudaError_t tsqr_launch(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, cuda
     const size_t sr = tsqr_reg_bytes(rb, n);
     if (sr <= (size_t)kSmemMax) {
       const int threads = 32 * std::min(16, std::max(4, n));
-      if (rb <= 128) return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-      if (rb <= 256) return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-      if (rb <= 512) return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+      switch ((rb + 63) / 64) {              // rows a lane, in twos
+        case 1: return tsqr_run<k_tsqr_reg<2>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 2: return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 3: return tsqr_run<k_tsqr_reg<6>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 4: return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 5: return tsqr_run<k_tsqr_reg<10>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 6: return tsqr_run<k_tsqr_reg<12>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 7: return tsqr_run<k_tsqr_reg<14>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        case 8: return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
+        default: break;
+      }
     }
   }
   const int threads = 32 * std::min(32, std::max({4, n, rb / 64}));   // (a warp a column)
@@ -2243,8 +2254,13 @@ cudaError_t init_kernel_attributes() {
   cudaError_t e;
   if ((e = smem_optin<k_tsqr_smem<double2>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_tsqr_smem<float2>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<2>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_tsqr_reg<4>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<6>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_tsqr_reg<8>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<10>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<12>>()) != cudaSuccess) return e;
+  if ((e = smem_optin<k_tsqr_reg<14>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_tsqr_reg<16>>()) != cudaSuccess) return e;
   if ((e = smem_optin<k_jacobi_cut64>()) != cudaSuccess) return e;
   for (const void* f : {(const void*)k_msg_normalise<double2>, (const void*)k_msg_normalise<float2>,

@@ -36,12 +36,12 @@
 // a pair are taken side by side in lanes of one instruction and the sums share
 // their addition tree (6 additions for 20), two pairs a CTA: 128 instructions
 // a pair, half of them scalars.  complex64: the chain of one reduction and
-// five roots and quotients a round, eight pairs a CTA.  Measured, us, one CTA
-// with all rows (a warp or half a warp a pair, every lane its own scalars) and
-// here: complex128 8 x 8 261 and 178, 31 x 40 6170 and 1430, 64 x 64 28400 and
-// 3470 (graded rows 62600 and 8090); complex64 31 x 40 315 and 280, 64 x 64
-// 1030 and 757, 96 x 90 1737 and 1190; from device memory and here: complex128
-// 128 x 128 45600 and 11250.
+// five roots and quotients a round.  Measured, us, one CTA with all rows (a warp
+// or half a warp a pair, every lane its own scalars) and here: complex128 8 x 8
+// 261 and 178, 31 x 40 6170 and 1430, 64 x 64 28400 and 3470 (graded rows 62600
+// and 8090); complex64 31 x 40 315 and 278, 64 x 64 1030 and 717, 96 x 90 1737 and
+// 1167 (long rows of few pairs are no faster: 20 x 900 323 and 354); from device
+// memory and here: complex128 128 x 128 45600 and 11250.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -58,6 +58,7 @@ namespace bbp {
 namespace {
 
 constexpr int kJacMaxCluster = 16;
+constexpr int kJacWarps = 20;
 constexpr size_t kJacSmemMax = 227 * 1024;
 constexpr size_t kJacStaged = 211 * 1024;   // rows that one CTA's shared memory held: the staged orders
 
@@ -162,11 +163,11 @@ template <typename C> constexpr int kJacUnscaled = sizeof(C) == sizeof(float2) ?
 
 __host__ __device__ inline size_t jac_header(int M) {
   const size_t Mp = M + (M & 1);
-  return 64 + 160 + 512 + ((2 * sizeof(double) + sizeof(int)) * Mp + 15) / 16 * 16;
+  return 64 + 176 + 512 + ((2 * sizeof(double) + sizeof(int)) * Mp + 15) / 16 * 16;
 }
 
 template <typename C, int ORD, bool CL>
-__global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__ Z, C* __restrict__ Gout,
+__global__ void __launch_bounds__(32 * kJacWarps, 1) k_jac(JacArgs p, const C* __restrict__ Z, C* __restrict__ Gout,
                                                 C* __restrict__ WHout, double* __restrict__ sigma,
                                                 int* __restrict__ idx, double* __restrict__ zn2_out, int* counters,
                                                 C* __restrict__ U, C* __restrict__ Rem, int* status, double* flops) {
@@ -184,8 +185,8 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
   volatile int* failed = (volatile int*)(smem_raw + 48);
   int* s_rot = (int*)(smem_raw + 52);
   double* s_sum = (double*)(smem_raw + 64);         // [0] this CTA's sum, [1 ..] warps' sums
-  int* s_cnt = (int*)(smem_raw + 64 + 160);         // [2][16][4] rotations of a sweep, by CTA
-  double* s_sig = (double*)(smem_raw + 64 + 160 + 512);   // [Mp] singular values
+  int* s_cnt = (int*)(smem_raw + 64 + 176);         // [2][16][4] rotations of a sweep, by CTA
+  double* s_sig = (double*)(smem_raw + 64 + 176 + 512);   // [Mp] singular values
   double* s_inv = s_sig + Mp;            // [Mp] their inverses, zero below the floor
   int* s_rank = (int*)(s_inv + Mp);      // [Mp], and a pad to sixteen bytes
   C* rows = (C*)(smem_raw + jac_header(M));
@@ -216,7 +217,9 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
   double part = 0.0;
 #pragma unroll 4
   for (int e = tid; e < 2 * pl * ld; e += nt) {
-    const int rr = e / ld, c = e - rr * ld, j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
+    // neighbouring threads along the contiguous index of Z
+    const int rr = p.conj_t ? e % (2 * pl) : e / ld, c = p.conj_t ? e / (2 * pl) : e - rr * ld;
+    const int j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
     if (!CL && a >= M) continue;         // (no slot for the row that rounds M up)
     C v = zero;
     if (a < M) {
@@ -390,7 +393,8 @@ __global__ void __launch_bounds__(512, 1) k_jac(JacArgs p, const C* __restrict__
   __syncthreads();
 #pragma unroll 2
   for (int e = tid; e < 2 * pl * len; e += nt) {
-    const int rr = e / len, c = e - rr * len, j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
+    const int rr = p.conj_t ? e % (2 * pl) : e / len, c = p.conj_t ? e / (2 * pl) : e - rr * len;
+    const int j = rr >> 1, a = rr & 1 ? id_b(j) : id_a(j);
     if (a >= M) continue;
     const C x = (rr & 1 ? second(j, CL ? R0 : 0) : first(j, CL ? R0 : 0))[c];
     const int rank = s_rank[a];
@@ -429,18 +433,19 @@ struct JacPlan {
 };
 
 // Places a CTA.  complex128: two (four pairs an SM wait for its FP64 unit:
-// 64 clocks a warp-wide instruction).  complex64: one CTA up to
-// sixteen places (pushing rows costs more than two CTAs save: 31 x 40 280 us,
-// on two CTAs 335), else eight a CTA.  More when sixteen CTAs need it, and one CTA
-// alone where a cluster's rings (pp + 2 slots each) do not fit.
+// 64 clocks a warp-wide instruction; 64 rows 7.26 ms, on four places 7.62).
+// complex64: one CTA up to twenty places, nine of long rows (pushing rows costs
+// more than several CTAs save: 40 x 40 692 us, on a cluster of five 749; 40 x 200
+// 1003 and 907), else four a CTA (96 x 96 2450 us, eight 2585, sixteen 3104).  More when sixteen CTAs need it, and one
+// CTA alone where a cluster's rings (pp + 2 slots each) do not fit.
 template <typename C>
 bool jac_plan(int M, int N, JacPlan& p) {
   const bool c64 = sizeof(C) == sizeof(float2);
-  const int P = (M + 1) / 2, pref = c64 ? 8 : 2;
+  const int P = (M + 1) / 2, pref = c64 ? 4 : 2;
   const size_t row = sizeof(C) * (size_t)((N + M + 1) & ~1);
   const bool staged = sizeof(C) * ((size_t)M * N + (size_t)M * M) <= kJacStaged;
   p.order = !staged ? kJacPlain32 : (M > 64 ? kJacStaged16 : kJacStaged32);
-  if (P > (c64 ? 16 : pref)) {
+  if (P > (c64 ? (N + M <= 160 ? 20 : 9) : pref)) {
     p.pp = std::max(pref, (P + kJacMaxCluster - 1) / kJacMaxCluster);
     p.cs = (P + p.pp - 1) / p.pp;
     p.bytes = jac_header(M) + row * (2 * (p.pp + 2) + 1);
@@ -470,7 +475,9 @@ cudaError_t jac_run(const JacPlan& p, const JacArgs& a, const C* Z, C* G, C* WH,
   if (p.cs == 0) return cudaSuccess;     // (the attributes only)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.cs, 1, 1);
-  cfg.blockDim = dim3(32 * std::min(std::max(p.pp, 8), 16), 1, 1);   // (eight warps load and store)
+  // (eight warps load and store short rows, all long ones)
+  const int least = (a.M * (a.N + a.M)) / p.cs >= 8192 ? kJacWarps : 8;
+  cfg.blockDim = dim3(32 * std::min(std::max(p.pp, least), kJacWarps), 1, 1);
   cfg.dynamicSmemBytes = p.bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
