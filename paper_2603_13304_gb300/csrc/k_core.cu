@@ -637,16 +637,16 @@ __global__ void __launch_bounds__(1024) k_tsqr_smem(const C* __restrict__ Ag, in
 // by the reflector's chain: 432 x 27 166 us with an even stride and 512 rows'
 // worth of registers, 119 us; 288 x 32 148 and 109; 512 x 48 285.
 template <int MAXR>
-__device__ __forceinline__ void tsqr_params_reg(const float2* A, int ldr, int c, int j, int m, float2* s_tau,
+__device__ __forceinline__ void tsqr_params_reg(const float2* A, int ld, int c, int j, int m, float2* s_tau,
                                                 float2* s_sc, float2* s_beta) {
   const int lane = threadIdx.x & 31;
   float2 x[MAXR];
 #pragma unroll
   for (int i = 0; i < MAXR; ++i) {
     const int r = lane + 32 * i;
-    x[i] = (r > j && r < m) ? A[(size_t)r * ldr + c] : make_float2(0.f, 0.f);
+    x[i] = (r > j && r < m) ? A[c * ld + r] : make_float2(0.f, 0.f);
   }
-  const float2 alpha = A[(size_t)j * ldr + c];
+  const float2 alpha = A[c * ld + j];
   float amax = fmaxf(fabsf(alpha.x), fabsf(alpha.y));
 #pragma unroll
   for (int i = 0; i < MAXR; ++i) amax = fmaxf(amax, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
@@ -678,14 +678,20 @@ __device__ __forceinline__ void tsqr_params_reg(const float2* A, int ldr, int c,
   }
 }
 
-inline size_t tsqr_reg_bytes(int m, int n) {
+// which panels take this kernel (its results differ from k_tsqr_smem's in the
+// order of the sums), and its shared memory at a column stride
+inline bool tsqr_reg_takes(int m, int n) {
   const int k = m < n ? m : n;
-  return sizeof(float2) * ((size_t)m * (n + 1) + 2 * (size_t)m + 3 * (size_t)k + 8);
+  return m <= 512 && sizeof(float2) * ((size_t)m * (n + 1) + 2 * (size_t)m + 3 * (size_t)k + 8) <= (size_t)kSmemMax;
+}
+inline size_t tsqr_reg_bytes(int m, int n, int ld) {
+  const int k = m < n ? m : n;
+  return sizeof(float2) * ((size_t)ld * n + 2 * (size_t)m + 3 * (size_t)k + 8);
 }
 
 template <int MAXR>
 __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ Ag, int m_all, int n, float2* Q,
-                                                     float2* Rm, int rb) {
+                                                     float2* Rm, int rb, int ld) {
   using C = float2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int row0 = blockIdx.x * rb;
@@ -693,9 +699,8 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
   Ag += (size_t)row0 * n;
   if (gridDim.x > 1) Rm += (size_t)blockIdx.x * n * n;
   const int k = m < n ? m : n;
-  const int ldr = n | 1;                     // odd: the rows of a column lie in different banks
-  C* A = (C*)smem_raw;                       // (r, c) at A[r * ldr + c]
-  C* vbuf = A + (size_t)m * ldr;
+  C* A = (C*)smem_raw;                       // (r, c) at A[c * ld + r]
+  C* vbuf = A + ld * n;
   C* s_tau = vbuf + 2 * (size_t)m;
   C* s_sc = s_tau + k;
   C* s_beta = s_sc + k;
@@ -715,19 +720,19 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int r = r0 + q, c = c0 + lane + 32 * h;
-          if (r < m && c < n) A[(size_t)r * ldr + c] = v[q][h];
+          if (r < m && c < n) A[c * ld + r] = v[q][h];
         }
     }
   __syncthreads();
-  if (warp == 0 && k > 0) tsqr_params_reg<MAXR>(A, ldr, 0, 0, m, s_tau, s_sc, s_beta);
+  if (warp == 0 && k > 0) tsqr_params_reg<MAXR>(A, ld, 0, 0, m, s_tau, s_sc, s_beta);
   __syncthreads();
   for (int j = 0; j < k; ++j) {
     const C tj = s_tau[j], sc = s_sc[j];
     const C ctau = cconj(tj);
     if (j > 0 && warp == (j - 1) % nw) {     // finalise column j - 1
       const C scp = s_sc[j - 1];
-      for (int r = j + lane; r < m; r += 32) A[(size_t)r * ldr + j - 1] = cmul(A[(size_t)r * ldr + j - 1], scp);
-      if (lane == 0) A[(size_t)(j - 1) * ldr + j - 1] = s_beta[j - 1];
+      for (int r = j + lane; r < m; r += 32) A[(j - 1) * ld + r] = cmul(A[(j - 1) * ld + r], scp);
+      if (lane == 0) A[(j - 1) * ld + (j - 1)] = s_beta[j - 1];
     }
     const int c0 = j + 1 + ((warp - (j + 1)) % nw + nw) % nw;
     if (!(tj.x == 0.f && tj.y == 0.f) && c0 < n) {
@@ -735,14 +740,14 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
 #pragma unroll
       for (int i = 0; i < MAXR; ++i) {
         const int r = lane + 32 * i;
-        xj[i] = (r > j && r < m) ? A[(size_t)r * ldr + j] : make_float2(0.f, 0.f);
+        xj[i] = (r > j && r < m) ? A[j * ld + r] : make_float2(0.f, 0.f);
       }
       for (int c = c0; c < n; c += nw) {
         C y[MAXR];
 #pragma unroll
         for (int i = 0; i < MAXR; ++i) {
           const int r = lane + 32 * i;
-          y[i] = (r > j && r < m) ? A[(size_t)r * ldr + c] : make_float2(0.f, 0.f);
+          y[i] = r < m ? A[c * ld + r] : make_float2(0.f, 0.f);
         }
         C a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -753,39 +758,39 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
         C acc = cadd(a0, a1);
         acc.x = warp_sum(acc.x);
         acc.y = warp_sum(acc.y);
-        const C ajc = A[(size_t)j * ldr + c];
+        const C ajc = A[c * ld + j];
         const C dot = cadd(ajc, cmulc(sc, acc));
         const C f = cmul(ctau, dot);
         const C fs = cmul(f, sc);
 #pragma unroll
         for (int i = 0; i < MAXR; ++i) {
           const int r = lane + 32 * i;
-          if (r > j && r < m) A[(size_t)r * ldr + c] = csub(y[i], cmul(xj[i], fs));
+          if (r < m) A[c * ld + r] = csub(y[i], cmul(xj[i], fs));   // (xj is zero above: those rows stay)
         }
         __syncwarp();
-        if (lane == 0) A[(size_t)j * ldr + c] = csub(ajc, f);
+        if (lane == 0) A[c * ld + j] = csub(ajc, f);
       }
     }
     __syncwarp();
-    if (j + 1 < k && warp == (j + 1) % nw) tsqr_params_reg<MAXR>(A, ldr, j + 1, j + 1, m, s_tau, s_sc, s_beta);
+    if (j + 1 < k && warp == (j + 1) % nw) tsqr_params_reg<MAXR>(A, ld, j + 1, j + 1, m, s_tau, s_sc, s_beta);
     __syncthreads();
   }
   if (k > 0 && warp == (k - 1) % nw) {
     const C scp = s_sc[k - 1];
-    for (int r = k + lane; r < m; r += 32) A[(size_t)r * ldr + k - 1] = cmul(A[(size_t)r * ldr + k - 1], scp);
-    if (lane == 0) A[(size_t)(k - 1) * ldr + k - 1] = s_beta[k - 1];
+    for (int r = k + lane; r < m; r += 32) A[(k - 1) * ld + r] = cmul(A[(k - 1) * ld + r], scp);
+    if (lane == 0) A[(k - 1) * ld + (k - 1)] = s_beta[k - 1];
   }
   __syncthreads();
   if (Rm) {
     const int krows = gridDim.x > 1 ? n : k;
     for (int i = warp; i < krows; i += nw)
       for (int c = lane; c < n; c += 32)
-        Rm[(size_t)i * n + c] = (i < k && c >= i) ? A[(size_t)i * ldr + c] : make_float2(0.f, 0.f);
+        Rm[(size_t)i * n + c] = (i < k && c >= i) ? A[c * ld + i] : make_float2(0.f, 0.f);
   }
   if (!Q) return;
   if (k > 0 && warp == (k - 1) % nw)
     for (int r = k - 1 + lane; r < m; r += 32)
-      vbuf[((k - 1) & 1) * m + r] = (r == k - 1) ? make_float2(1.f, 0.f) : A[(size_t)r * ldr + k - 1];
+      vbuf[((k - 1) & 1) * m + r] = (r == k - 1) ? make_float2(1.f, 0.f) : A[(k - 1) * ld + r];
   __syncthreads();
   for (int i = k - 1; i >= 0; --i) {
     const C* v = vbuf + (i & 1) * m;
@@ -804,7 +809,7 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
 #pragma unroll
         for (int q = 0; q < MAXR; ++q) {
           const int r = lane + 32 * q;
-          y[q] = (r >= i && r < m) ? A[(size_t)r * ldr + c] : make_float2(0.f, 0.f);
+          y[q] = r < m ? A[c * ld + r] : make_float2(0.f, 0.f);
         }
         C a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -819,7 +824,7 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
 #pragma unroll
         for (int q = 0; q < MAXR; ++q) {
           const int r = lane + 32 * q;
-          if (r >= i && r < m) A[(size_t)r * ldr + c] = csub(y[q], cmul(vv[q], f));
+          if (r < m) A[c * ld + r] = csub(y[q], cmul(vv[q], f));
         }
       }
       if (own_i) {                          // column i := e_i - tau_i v_i
@@ -828,46 +833,48 @@ __global__ void __launch_bounds__(512, 1) k_tsqr_reg(const float2* __restrict__ 
         for (int q = 0; q < MAXR; ++q) {
           const int r = lane + 32 * q;
           if (r < m)
-            A[(size_t)r * ldr + i] =
+            A[i * ld + r] =
                 (r == i) ? make_float2(1.f - ti.x, -ti.y) : (r > i ? cmul(mt, vv[q]) : make_float2(0.f, 0.f));
         }
       }
     }
     if (i > 0 && warp == (i - 1) % nw)
       for (int r = i - 1 + lane; r < m; r += 32)
-        vbuf[((i - 1) & 1) * m + r] = (r == i - 1) ? make_float2(1.f, 0.f) : A[(size_t)r * ldr + i - 1];
+        vbuf[((i - 1) & 1) * m + r] = (r == i - 1) ? make_float2(1.f, 0.f) : A[(i - 1) * ld + r];
     __syncthreads();
   }
   for (int r = warp; r < m; r += nw)
-    for (int c = lane; c < k; c += 32) Q[(size_t)r * k + c] = A[(size_t)r * ldr + c];
+    for (int c = lane; c < k; c += 32) Q[(size_t)r * k + c] = A[c * ld + r];
 }
 
 // One staged QR launch (grid = row blocks): the register-cached kernel for
 // complex64 panels of at most 512 rows per block, the generic one otherwise.
-template <auto kKernel, typename C>
-cudaError_t tsqr_run(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, int threads, size_t bytes, cudaStream_t s) {
+template <auto kKernel, typename C, typename... More>
+cudaError_t tsqr_run(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, int threads, size_t bytes, cudaStream_t s,
+                     More... more) {
   cudaError_t e = smem_optin<kKernel>();
   if (e != cudaSuccess) return e;
-  kKernel<<<(m_all + rb - 1) / rb, threads, bytes, s>>>(Ag, m_all, n, Q, Rm, rb);
+  kKernel<<<(m_all + rb - 1) / rb, threads, bytes, s>>>(Ag, m_all, n, Q, Rm, rb, more...);
   return cudaGetLastError();
 }
 
 template <typename C>
 cudaError_t tsqr_launch(const C* Ag, int m_all, int n, C* Q, C* Rm, int rb, cudaStream_t s) {
   if constexpr (sizeof(C) == sizeof(float2)) {
-    const size_t sr = tsqr_reg_bytes(rb, n);
-    if (sr <= (size_t)kSmemMax) {
+    if (tsqr_reg_takes(rb, n)) {
+      // an odd column stride (no bank conflicts between rows and columns) where it fits
+      const int ld = tsqr_reg_bytes(rb, n, rb | 1) <= (size_t)kSmemMax ? rb | 1 : rb;
+      const size_t sr = tsqr_reg_bytes(rb, n, ld);
       const int threads = 32 * std::min(16, std::max(4, n));
       switch ((rb + 63) / 64) {              // rows a lane, in twos
-        case 1: return tsqr_run<k_tsqr_reg<2>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 2: return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 3: return tsqr_run<k_tsqr_reg<6>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 4: return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 5: return tsqr_run<k_tsqr_reg<10>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 6: return tsqr_run<k_tsqr_reg<12>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 7: return tsqr_run<k_tsqr_reg<14>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        case 8: return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s);
-        default: break;
+        case 1: return tsqr_run<k_tsqr_reg<2>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        case 2: return tsqr_run<k_tsqr_reg<4>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        case 3: return tsqr_run<k_tsqr_reg<6>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        case 4: return tsqr_run<k_tsqr_reg<8>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        case 5: return tsqr_run<k_tsqr_reg<10>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        case 6: return tsqr_run<k_tsqr_reg<12>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        case 7: return tsqr_run<k_tsqr_reg<14>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
+        default: return tsqr_run<k_tsqr_reg<16>>(Ag, m_all, n, Q, Rm, rb, threads, sr, s, ld);
       }
     }
   }
