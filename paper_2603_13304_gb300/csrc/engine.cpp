@@ -58,12 +58,13 @@ cudaError_t merge_call(int M, int N, int K, const float2* A, const float2* B, fl
   return launch_zgemm('N', 'N', M, N, K, make_float2(1, 0), A, K, 0, B, N, 0, make_float2(0, 0), C, N, 0, 1, s);
 }
 
-// launches of one truncated SVD (statistics only)
+// launches of one truncated SVD (statistics only): the sketch, 2 (1 + q) panels
+// and as many products, the Jacobi, the FP64 finish, the gathered rows, U and Rem
 long long svd_launches(int m, int n, int chi, bool c64, int q) {
   const int M = std::min(m, n);
   const int b = c64 ? rand_block(m, n, chi) : rand_block64(m, n, chi);
   if (b >= M) return 1;
-  return 8 + 4 * q + (c64 ? 1 : 0);
+  return 9 + 4 * q + (c64 ? 1 : 0);
 }
 cudaError_t svd_call(const float2* Z, int m, int n, int chi, float2* U, float2* Rem, void* work, int* status,
                      cudaStream_t s, int power_iters, bool tensor_cores, int* tc_err) {
@@ -1008,7 +1009,7 @@ int Engine::run_sweep(SweepJob& job, SweepWork& w, bool want_log) {
     if (tc_mode && sizeof(C) == sizeof(float2)) {
       // split TF32 / BF16 on the tensor cores, FP32 accumulation
       CK(launch_tc_absorb(tc_mode == 2, X, (int)P, Q, Sp, l, r, Rb[0], w.tc, w.status + 1, s));
-      launches += 6;
+      launches += 4;
     } else {
       KTimerScope timer(KC_ABSORB, s, 8.0 * l * (double)P * Q * r);
       CK(launch_zgemm('T', 'N', Q, r, (int)P, one, X, Q, 0, Sp, r, P * r, zero, Rb[0], r, (long long)Q * r, l, s));
