@@ -115,8 +115,8 @@ class ClockSampler:
 # with CUDA events on the streams its launches run on (library-side timer).
 KERNELS = {
     "jacobi": (1, "one-sided Jacobi SVD of the reduced matrix (k_jac; k_jacobi beyond a cluster's shared memory)"),
-    "orth": (2, "blocked Householder QR of the range panels (k_bqr on clusters)"),
-    "qr": (3, "blocked Householder QR of the canonical moves and distances (k_bqr)"),
+    "orth": (2, "Householder QR of the range panels (k_panel_qr on clusters, k_tsqr_reg / k_tsqr_smem on one CTA)"),
+    "qr": (3, "Householder QR of the canonical moves and distances (k_tsqr_reg / k_tsqr_smem, k_panel_qr)"),
     "tc": (4, "tcgen05 split-precision GEMM: the absorb contraction and the segment merges (k_tc_gemm)"),
     "absorb": (5, "SIMT complex absorb GEMM (k_gemm)"),
     "gemm": (6, "every SIMT complex GEMM (k_gemm)"),
@@ -127,13 +127,13 @@ KERNELS = {
 # precision); an entry is removed when its kernel changes.
 TRAFFIC = {
     ("orth", "kagome-6x2-L2-D6-chi64", "tf32"): {
-        "bytes": 1.91e6,
-        "note": "one 2304 x 96 complex64 panel with Q (bench.py --kernel-case panel): DRAM read 1.91 MB, write 0 "
+        "bytes": 1.88e6,
+        "note": "one 2304 x 96 complex64 panel with Q (bench.py --kernel-case panel): DRAM read 1.88 MB, write 0 "
                 "(the 1.8 MB of Q stays in L2)"},
     ("tc", "kagome-6x2-L2-D6-chi64", "tf32"): {
-        "bytes": 345.6e6,
-        "note": "one absorb GEMM at P = Q = 1296, l = r = 64 (bench.py --kernel-case absorb): DRAM read 320.1 MB + "
-                "write 25.4 MB against 181 MB of operands and output"},
+        "bytes": 350.0e6,
+        "note": "one absorb GEMM at P = Q = 1296, l = r = 64 (bench.py --kernel-case absorb): DRAM read 324.1 MB + "
+                "write 25.9 MB against 181 MB of operands and output"},
 }
 
 # TF32 / BF16 dense tensor rates of the part, nominal (for the ratio only)

@@ -410,9 +410,10 @@ bbp_status bbp_k_qr(double* A, int m, int n, double* Q, double* R, double* tau, 
  * least bbp_k_panel_cluster(c64, m, n) (the fewest whose shared memory holds
  * the panel with Q; 0 when even 16 do not) and at most 16.  A call with
  * Q = NULL needs a little less shared memory (no reflector scalars), so it
- * may fit where bbp_k_panel_cluster reports 0.  A CTA beyond
- * the rows a given cluster needs holds none.  BBP_ERR_ARG when m < n or the
- * panel does not fit. */
+ * may fit where bbp_k_panel_cluster reports 0.  Each CTA caches 32, 64, ...
+ * rows per warp lane (complex64 up to 256 rows a CTA, complex128 up to 128),
+ * and a CTA beyond the rows a given cluster needs holds none.  BBP_ERR_ARG
+ * when m < n or the panel does not fit. */
 int bbp_k_panel_cluster(int c64, int m, int n);
 bbp_status bbp_k_panel_qr(int c64, const void* A, int m, int n, void* Q, void* R, int batch, int cluster,
                           void* stream);
@@ -452,13 +453,15 @@ bbp_status bbp_k_tc_gemm_tile(int bf16, const void* A, long long lda, const void
                               void* stream);
 
 /* Tile autotuner of the tensor-core GEMM (process-wide; thread-safe).
- * bbp_autotune_record(1) collects the shape (precision, M, N, K) of every
+ * bbp_autotune_record(1) collects the shape (precision, M, N, K, form) of every
  * later tensor-core GEMM launch that has no table entry, for example during
  * an eager first iteration; bbp_autotune_run times every candidate tile of
  * each collected shape on scratch operands it allocates (synchronously, on
  * its own stream; not inside a graph capture), keeps the fastest, sets
  * *n_tuned, and writes the whole table to cache_path when it is not NULL
- * (one line "tc bf16 M N K bn group_m microseconds" per shape).
+ * (one line "tc bf16 M N K bn group_m microseconds form" per shape; form: 0 a
+ * real product, 1 to 4 an absorb into complex64 (odd) or complex128, above 2
+ * with each limb stored once; lines without a form are read as form 0).
  * bbp_autotune_load merges a table written that way (*n_loaded entries).
  * Every table change advances a generation that the contexts' captured
  * iteration graphs check, so later iterations re-capture with the new tiles.

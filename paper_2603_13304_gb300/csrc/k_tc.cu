@@ -24,8 +24,8 @@
 // accumulate in FP32 in one pass to about FP32 accuracy.  The sums run over
 // the segments as one K dimension, one MMA (32 bytes of K) after the other:
 // which entries share an MMA is part of the result.  Where a segment is whole
-// MMAs, each limb is stored once and read as often as it occurs; else a row
-// holds every segment (kOnce).
+// MMAs, each limb is stored once and read as often as it occurs (kOnce); else
+// a row holds every segment.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
